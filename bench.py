@@ -173,7 +173,7 @@ def load_traffic(kernel_key):
 def gather_source_sha():
     import hashlib
     h = hashlib.sha256()
-    for f in ("gather.cu", "gather_tma.cu", "cp_internal.h"):
+    for f in ("gather.cu", "gather_chunk.cu", "cp_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_1005_3609_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -193,13 +193,8 @@ def table_layout(cp, args):
 
 
 def tile_name(tile):
-    rows, ring, edges, cpt = tile & 0xFFF, (tile >> 12) & 0xFF, (tile >> 20) & 15, (tile >> 24) & 15
-    shape = (tile >> 28) & 3
-    if rows <= 8:
-        return "register gather kernel, %d rows/warp" % rows
-    return "TMA gather kernel, %d rows/block, %s KB ring, %s edge(s) per stage, %s chunk(s) per thread, %s" % (
-        rows, ring or "auto", edges or "auto", cpt or "auto",
-        {1: "wide blocks", 2: "narrow blocks"}.get(shape, "block shape auto"))
+    rows = tile & 0xFFF
+    return "register gather kernel, %d rows/warp" % rows if rows <= 8 else "chunk gather kernel"
 
 
 def plain_run(cp, torch, lattice, k, primes, stream):
@@ -692,7 +687,7 @@ def paper_arm(args):
     lattice, k = args.lattice, 41
     primes = cp.select_primes(synthetic_inputs.prime_draws(0, 128), 16)
     stream = torch.cuda.Stream()
-    tile = args.tile or 32  # TMA kernel, rows/block 32, ring, stages and chunks per thread picked by row width
+    tile = args.tile or 32  # the chunk gather kernel
     table_layout(cp, args)
     peak = (load_peaks() or {}).get("hbm_gbs") or 6800.0
     groups, res_all = [], []
@@ -866,7 +861,7 @@ def probe_arm(args):
                                   "reset to e_0, %d rows, read-out" % (lattice, L, n_states[0], n_states[1], P, D,
                                                                        rows),
                       "l2": "no flush: vectors %.1f GB each, > 100x L2" % (n_states[1] * (D + 1) * P * 4 / 1e9),
-                      "tables": "built before timing (%.1f s)" % setup_s, "tile": "strip default (TMA gather)",
+                      "tables": "built before timing (%.1f s)" % setup_s, "tile": "strip default (chunk gather)",
                       "factor_tables": layout,
                       "updates_per_step": upd_step},
            "e2e": {"value": upd_step * args.steps / (e2e_ms / 1e3), "unit": "updates/s", "h2d_bytes_per_step": 0,
@@ -877,7 +872,7 @@ def probe_arm(args):
                         "traffic": traffic["dram_bytes_per_launch"] if traffic else None,
                         "algorithmic_bytes_per_launch": row_bytes / len_row, "avg_launch_ms": row_ms / len_row,
                         "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks else "fallback 6800 GB/s",
-                        "kernel": "TMA gather (row advance = %d launches)" % len_row,
+                        "kernel": "chunk gather (row advance = %d launches)" % len_row,
                         "tables_own_bytes": {"bytes_per_launch": row_own / len_row, "achieved": round(own, 1),
                                              "frac": round(own / peak, 4)}}}
     if clk:

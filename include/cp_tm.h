@@ -56,7 +56,8 @@ typedef struct cp_strip cp_strip;
  * cp_create_strip -- a strip of width L, height 1, state vector = e_0.
  * Builds (or reuses from the per-device cache) the rank tables and the CSR
  * tables of every per-site factor T_i and T_i^last on the GPU, and allocates
- * the two state vectors [S][D+1][n_primes] (S = M_{L-1} + M_{L-2} on the
+ * the two state vectors [S][D+1][n_primes, rounded up to a multiple of four where
+ * that fits] (S = M_{L-1} + M_{L-2} on the
  * square lattice, M_{L-1} on the triangular one; Sec. 3.2-3.3).
  *   lattice    CP_SQUARE or CP_TRIANGULAR
  *   L          1..CP_MAX_L sites per row (strip width m of the paper)
@@ -130,10 +131,8 @@ int cp_strip_info(const cp_strip *s, uint64_t n_states[2], int *degree, int *hei
 int cp_strip_work(const cp_strip *s, uint64_t work[6]);
 
 /* Gather tile of the strip's launches, encoded as cp_sweep_create's tile
- * (0 = the default: TMA kernel, 32 rows per block -- 16 where 32-row blocks
- * would give a launch fewer than eight waves of resident blocks -- stages,
- * chunks per thread and ring picked from the row width).  A tuning knob: results are identical
- * for every tile.  Synchronises the strip's stream.  CP_EINVAL on a bad tile. */
+ * (0 = the default, the chunk kernel).  A tuning knob: results are identical for
+ * every tile.  Synchronises the strip's stream.  CP_EINVAL on a bad tile. */
 int cp_strip_set_tile(cp_strip *s, int tile);
 
 /* Restart the strip at height 1 with the state vector e_0 (keeps its tables
@@ -270,17 +269,12 @@ int cp_select_primes(const uint64_t *draws_host, int n_draws, int n_primes, uint
  */
 typedef struct cp_sweep cp_sweep;
 
-/* tile: 0 = autotune; 1, 2, 4, 8 = register gather kernel, rows per warp;
- *       16, 32, 64, 128 = TMA gather kernel, rows per block, optionally plus
- *       (ring KB << 12) with ring KB in 16..192 (shared-memory ring per block,
- *       0 = what fills the SM at the kernel's occupancy; raised to hold two
- *       stages), (edges per stage << 20) with 1, 2, 4 or 8 (0 = about 20 KB
- *       of source rows per stage, at most 32 / row groups; 4 in narrow blocks), (16-byte chunks
- *       per consumer thread << 24) with 1, 2 or 4 (0 = 2 for rows wider than
- *       3 KB, else 1) and (block shape << 28) with 1 = wide (8 / chunks-per-
- *       thread consumer warps) or 2 = narrow (5 consumer warps; one chunk per
- *       thread, rows of at most 160 chunks) (0 = narrow where every row of a
- *       launch has 129..160 chunks at one chunk per thread, else wide);
+/* tile: 0 = the default; 1, 2, 4, 8 = register gather kernel, rows per warp;
+ *       16, 32, 64, 128 = chunk gather kernel (rows of 16-byte chunks, dealt to the
+ *       warps by edges).  With the latter the bits above, (16..192 << 12),
+ *       (1, 2, 4, 8 << 20), (1, 2, 4 << 24) and (1, 2 << 28), are accepted and
+ *       choose nothing.  Launches that the chunk kernel cannot take (large
+ *       coefficients, small primes) run on the register kernel;
  * prime_groups: number of strips per width, dividing n_primes, or 0 = autotune.
  * cuda_stream must be a non-default stream (the program is graph-captured on it).
  * Errors: CP_EINVAL (k < 4, k/2 > CP_MAX_L, series longer than 128 terms, bad
@@ -412,8 +406,7 @@ const char *cp_last_error(void);
 int cp_debug_check_space(int kind, int m, int e, uint64_t *n_bad, uint64_t *size);
 
 /* Launch a wait that can never complete (an mbarrier nothing arrives on),
- * bounded by `cycles` SM clock cycles, exactly like the bounded waits of the
- * TMA gather kernel; returns CP_ETIMEOUT once it has expired (the device error
+ * bounded by `cycles` SM clock cycles; returns CP_ETIMEOUT once it has expired (the device error
  * word is read and cleared), leaving the context usable.  For testing the
  * timeout path without faulting or hanging the GPU. */
 int cp_debug_wait_timeout(long long cycles);
@@ -427,12 +420,11 @@ int cp_debug_wait_timeout(long long cycles);
  * otherwise.  Synchronous. */
 int cp_debug_reduce(const int64_t *v_host, const uint32_t *p_host, int n, uint32_t *out_host);
 
-/* The 32-bit reduction of the bulk-copy gather (Sec. 3.5), which it uses when
- * every prime of a launch is at least 2^17: a word's sum is kept as two
- * 32-bit halves, u = hi_host[k] 2^16 + lo_host[k], and reduced from them with
- * 32-bit operations.  out_host[k] = u mod p_host[k] in [0, p) when full != 0,
- * else (u mod p) or (u mod p) - p, a signed representative in [-p, p) as the
- * kernel stores for outputs that only feed further gathers.  Requires
+/* A 32-bit reduction (Sec. 3.5) of a word's sum kept as two 32-bit halves, u =
+ * hi_host[k] 2^16 + lo_host[k], for primes of at least 2^17:
+ * out_host[k] = u mod p_host[k] in [0, p) when full != 0,
+ * else (u mod p) or (u mod p) - p, a signed representative in [-p, p), as the
+ * gathers store.  Requires
  * 2^17 <= p_host[k] < 2^31 and 0 < u < p_host[k] 2^16; CP_EINVAL otherwise.
  * A diagnostic (it allocates device buffers).  Synchronous. */
 int cp_debug_reduce_halves(const int32_t *lo_host, const int32_t *hi_host, const uint32_t *p_host, int n, int full,

@@ -318,7 +318,7 @@ def debug_reduce(values, primes):
 
 
 def debug_reduce_halves(lo, hi, primes, full=True):
-    """The bulk-copy gather's 32-bit reduction of u = hi 2^16 + lo on the GPU
+    """A 32-bit reduction of u = hi 2^16 + lo on the GPU
     (cp_debug_reduce_halves): u mod p, or a representative in [-p, p) (as
     signed ints) when full is False."""
     lo_a = np.ascontiguousarray(np.asarray(lo, dtype=np.int32))

@@ -95,14 +95,29 @@ inline int potts_src_bits(uint64_t n_states) {
     return b;
 }
 
+// Degree windows.  P~ counts w^(vertices - components) (a horizontal or vertical
+// edge that joins two components costs one factor w), so the polynomial of a
+// state s of a strip with V vertices so far has terms only in the degrees
+//   lo_s <= d <= V - blocks_s:
+// V - d components, of which the state's own blocks are a part, and at least
+// lo_s joins to have built its blocks at all (lo_s: shortest path from e_0 in the
+// factors' tables, with each transition's shift as its length, over any number
+// of rows).  A window word packs lo (low byte; 254: at least 254; 255: never
+// reached) and the number of blocks (high byte).  On truncated vectors, d <= D,
+// most states of a wide strip have a short window or none.
+//
 // CSR-by-destination table of one per-site factor, on the device.
 struct SiteTable {
     OpDesc op;
     uint64_t n_src = 0, n_dst = 0, nnz = 0;
     uint64_t n_site_out = 0;  // output states of the per-site factors it stands for (n_dst, or mid + n_dst)
     uint32_t *row_ptr = nullptr;  // [n_dst + 1]
-    uint32_t *edges = nullptr;    // [nnz]
-    uint32_t *block_order = nullptr;  // row blocks by smallest source (GatherTask::block_order), or null
+    uint32_t *edges = nullptr;    // [nnz] while the table is built
+    uint2 *wedges = nullptr;      // [nnz] the edges as the gathers read them (GatherTask::edges)
+    uint4 *units = nullptr;           // [n_units] units of work of the chunk kernel (GatherTask::units)
+    uint32_t n_units = 0;
+    const uint16_t *win_in = nullptr, *win_out = nullptr;  // window words of the source and destination states
+    int sites = 1;                    // per-site factors it stands for (vertices added)
     uint32_t max_coef_sum = 0;        // largest sum of |coefficient| into one destination (an upper bound)
     uint32_t max_abs_coef = 0;        // largest |coefficient|
 };
@@ -117,15 +132,13 @@ struct TableSet {
     std::vector<SiteTable> row;
     std::vector<SiteTable> last;
     std::vector<uint32_t *> x_prefix;  // square lattice: prefix table of X_e, e = 0..L-2
+    std::vector<uint16_t *> wins;      // window words of every space of the two chains
     size_t bytes = 0;
     ~TableSet();
 };
 
 // Rank tables on the current device (built once per device by a kernel).
 int device_rank_tables(const RankTables **out_dev, RankTables *host_copy);
-
-// Prefix table of the interleaved space X_e on m sites (device, [M_{m-1} + 1]).
-int build_x_prefix(int m, int e, cudaStream_t st, uint32_t **out);
 
 // Build or fetch from the cache the tables of (lattice, L) on the current device
 // (chromatic polynomial: the projected factorisation of Sec. 3.2-3.3), paired
@@ -142,97 +155,141 @@ int set_factor_pairing(int mode);
 int get_potts_tables(int lattice, int L, int v, cudaStream_t stream, std::shared_ptr<TableSet> *out);
 
 // ------------------------------------------------------------------ gather
-// One per-site factor application: out[dst] = sum_e coef_e * w^{shift_e} in[src_e]  (mod p)
+// One per-site factor application: out[dst] = sum_e coef_e * w^{shift_e} in[src_e]  (mod p),
+// on the degree windows of the source and destination states: words outside a
+// state's window are never read nor written.  Words are signed representatives
+// in [-p, p) as 32-bit two's complement.
 struct GatherTask {
     const uint32_t *in;
     uint32_t *out;
     const uint32_t *row_ptr;
-    const uint32_t *edges;
-    const uint32_t *primes;   // n_primes words, device
+    const uint2 *edges;       // x: packed edge; y: window word of its source, row within its unit << 16, first edge of
+                              // the row << 21
+    const uint32_t *primes;   // prime block (fill_prime_block) on the device
+    const uint16_t *win_out;  // window words (lo | blocks << 8) of the destination states
+    const uint4 *units;       // chunk kernel: the table's units of work
+    uint32_t n_units;
     uint32_t rows;            // destination rows of this task
     uint32_t C;               // chunks per row (16-byte chunks if vec4, else words)
     uint32_t cpd;             // chunks per degree (= n_primes / VEC)
     uint32_t vec4;            // 1: 16-byte chunks, 0: 4-byte chunks
-    uint32_t block_begin;     // first block of this task in the launch
+    uint32_t block_begin;     // first block (chunk kernel: unit) of this task in the launch
     uint32_t magic_cpd;       // x / cpd = umulhi(x, magic_cpd) for x * cpd < 2^32 (0: cpd == 1)
     uint32_t n_primes;
-    uint32_t c0;              // first chunk of the rows handled by this task
-    uint32_t cw;              // chunks handled (a column range [c0, c0 + cw) of every row)
     uint32_t src_bits;        // edge format of the table
-    uint32_t partial;         // 1: the output feeds further gathers only (words may be left in [-p, p))
-    uint32_t small_coefs;     // 1: |coefficient| <= 127 and their sum into any destination < 2^15 (TMA kernel)
-    // TMA kernel: the order in which its blocks visit the row blocks, for 16,
-    // 32, 64 and 128 rows per block one after another (block_order_offset),
-    // or null for row-block order
-    const uint32_t *block_order;
+    uint32_t seg;             // chunk kernel: degrees of one pass over a row
+    uint32_t r32;             // 32 modulo cpd
+    uint32_t fast;            // 1: the coefficients and primes suit the chunk kernel's sums (fast_ok, modred.cuh)
+    uint32_t fast_k0;         // their offset
+    int32_t v_in, v_out;      // vertices of the input and of the output vector (window bound V - blocks)
+    int32_t cap;              // highest degree kept, D
+    uint32_t first;           // 1: the input vector is e_0 at height 1 (degree 0: nothing else is read)
 };
 
-// Start of the order for `rpb` rows per block in a table of `rows` rows.
-__host__ __device__ inline uint32_t block_order_offset(uint32_t rows, uint32_t rpb) {
-    uint32_t off = 0;
-    for (uint32_t l = 16; l < rpb; l *= 2) off += (rows + l - 1) / l;
-    return off;
+// Units of work of the chunk kernel, in row order: consecutive destination rows with
+// at most unit_edges(nnz) edges together and at most 32 rows, or a part of one row
+// with more than split_edges of them.  {first row; rows | heavy << 6 | part << 8;
+// first edge; one past the last edge}.  Rows differ a hundredfold in edges (the
+// states of many single sites collect most) and the heavy ones lie together, so
+// work is dealt out by edges and not by rows, and a heavy row's degrees are split
+// over kSplitParts warps.  A warp walks its edges one after another: tables too
+// small to give every resident warp 32 of them have smaller units.
+constexpr uint32_t kSplitParts = 4;
+inline uint32_t unit_edges(uint64_t nnz) {
+    uint32_t u = 32;
+    while (u > 4 && nnz < 4096ull * u) u /= 2;
+    return u;
 }
+inline uint32_t split_edges(uint32_t unit) { return unit < 16 ? 16 : unit; }
+constexpr uint32_t kPackRows = 32;   // rows packed into units together
+
+// What a vector's primes are to the gathers: the prime lanes, then each lane's
+// multiplier of the chunk kernel's reduction (256 bytes).
+constexpr int kPrimeWords = 2 * CP_MAX_PRIMES;
+void fill_prime_block(const uint32_t *primes, int n_primes, int lanes, uint32_t *block);
 
 constexpr int kGatherThreads = 256;  // 8 warps; one warp per destination row at a time
 constexpr int kGatherItems = 4;      // default rows per warp (the tile: 8 * rows per block)
 
-// Append the task(s) of one per-site factor: rows of 16-byte chunks wider than
-// 256 chunks are split into column tasks of at most 256 chunks each.
-// partial: the output vector is read by further gathers only, so the TMA kernel
-// may store signed representatives in [-p, p) (every gather reads its input
-// words as signed 32-bit values).
-void append_gather_tasks(std::vector<GatherTask> *tasks, const SiteTable &tab, const uint32_t *in,
-                         uint32_t *out, const uint32_t *primes_dev, int D1, int P, bool partial = false);
+// Append the task of one per-site factor applied to a vector of v_in vertices.
+// final: the output is the read-out's result, whose row is written whole.
+constexpr int kFinalVertices = 1 << 29;
+void append_gather_task(std::vector<GatherTask> *tasks, const SiteTable &tab, const uint32_t *in, uint32_t *out,
+                        const uint32_t *primes_dev, int D1, int P, int v_in, uint32_t min_prime, bool final = false);
+// Prime lanes of a vector's rows: padded to a multiple of four (repeats of the
+// last prime), so that rows are 16-byte chunked and take the chunk kernel.
+inline int padded_primes(int P) { return (P + 3) & ~3; }
 // Gather tile (low 12 bits): 1, 2, 4, 8 = register kernel with that many rows
-// per warp (8 warps per block); 16, 32, 64, 128 = TMA kernel with that many rows
-// per block.  For TMA tiles, bits 12..19 = ring size in KB (0: default) and
-// bits 20..23 = edges per stage, 1, 2, 4 or 8 (0: picked from the row size),
-// bits 24..27 = 16-byte chunks per consumer thread, 1, 2 or 4 (0: 2 for rows
-// wider than 3 KB, else 1), bits 28..29 = consumer block shape, 1 = wide
-// (8 / chunks-per-thread consumer warps), 2 = narrow (5 consumer warps, one
-// chunk per thread, rows of at most 160 chunks), 0 = narrow for batches whose
-// rows all have 129..160 chunks at one chunk per thread, else wide.  A batch
-// whose rows are not all 16-byte chunked uses the register kernel.
-constexpr int kTmaRingKbDefault = 48;
-constexpr int kTileWide = 1 << 28;
-constexpr int kTileNarrow = 2 << 28;
-constexpr int kTmaNarrowWarps = 5;  // consumer warps of a narrow block
-inline int make_tile(int rows, int ring_kb, int edges = 0, int cpt = 0) {
-    return rows | (ring_kb << 12) | (edges << 20) | (cpt << 24);
-}
-inline int tile_edges(int tile) { return (tile >> 20) & 15; }
-inline int tile_cpt(int tile) { int c = (tile >> 24) & 15; return c ? c : 1; }
-inline int tile_ring_kb(int tile) { int r = (tile >> 12) & 0xFF; return r ? r : kTmaRingKbDefault; }
-inline int tile_shape(int tile) { return (tile >> 28) & 3; }
-// Blocks per SM the TMA kernel's launch bounds aim at (its registers), and the
-// shared-memory ring that fills the SM at that occupancy; W = consumer warps
-// (0: the wide block, 8 / CPT).
-__host__ __device__ constexpr int tma_min_blocks(int E, int CPT, int W = 0) {
-    return W == kTmaNarrowWarps ? 4
-                                : (CPT == 1 ? (E >= 2 ? 3 : 4) : (CPT == 2 ? 4 : (E >= 4 ? 4 : 5)));
-}
-__host__ __device__ constexpr int tma_ring_kb_for(int E, int CPT, int W = 0) {
-    return W == kTmaNarrowWarps ? 52
-                                : (tma_min_blocks(E, CPT) <= 3 ? 64 : (tma_min_blocks(E, CPT) == 4 ? 48 : 40));
-}
-bool tile_is_tma(int items);
-bool tma_usable(const GatherTask &t);
-// Blocks of one task and of a whole launch (fills block_begin; returns the grid size).
+// per warp (8 warps per block); 16, 32, 64, 128 = chunk kernel.  The other bits are
+// accepted as cp_tm.h lists them and choose nothing.  A batch with rows that are
+// not 16-byte chunked, large coefficients or small primes uses the register kernel.
+constexpr int kTileChunk = 32;
+constexpr int kChunkWarps = 4;         // warps of a block of the chunk kernel
+constexpr int kChunkBlocksPerSM = 7;   // its launch bound
+constexpr int kChunkSteps = 4;         // 32-chunk steps of a row held in registers
+// The encodings cp_strip_set_tile and cp_sweep_create accept (besides 0).
+bool tile_valid(int tile);
+bool tile_is_chunk(int items);
+bool chunk_usable(const GatherTask &t);
+// Blocks (chunk kernel: units) of one task and of a whole launch (fills block_begin; returns the total).
 uint32_t task_blocks(const GatherTask &t, int items);
 uint32_t assign_blocks(std::vector<GatherTask> &tasks, int items);
-// Effective tile for a batch (falls back from TMA to the register kernel when needed).
+// Effective tile for a batch (falls back to the register kernel when needed).
 int effective_tile(const std::vector<GatherTask> &tasks, int items);
-// The TMA kernel accumulates coef * x as two 16 x 8-bit dot products into 32-bit
-// halves (gather_tma.cu), exact while |coef| <= kTmaMaxCoef and the sum of
-// |coef| into any destination stays below kTmaMaxCoefSum; other tables use the
-// register kernel.
-constexpr uint32_t kTmaMaxCoef = 127;
-constexpr uint32_t kTmaMaxCoefSum = 1u << 15;
-// Rows per block of the default TMA tile for a launch of these tasks (16 or 32).
-int default_rows(const std::vector<GatherTask> &tasks);
-// Launch a batch of tasks (tasks_dev = device copy, block_begin assigned for `items`).
-int launch_gather(const GatherTask *tasks_dev, int n_tasks, uint32_t total_blocks, int items, cudaStream_t st);
+// The chunk kernel takes coefficients as signed bytes; fast_ok (modred.cuh) bounds their sums.
+constexpr uint32_t kChunkMaxCoef = 127;
+bool table_fast(const SiteTable &tab, uint32_t min_prime);
+// Launch a batch of tasks (block_begin assigned for `items`), by value in the
+// kernel's parameters.  dv is added to the tasks' vertex counts (a strip's row h
+// uses the tasks of row 1 with dv = L (h - 1)); first: as if GatherTask::first were
+// set in each task.
+int launch_gather(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, int items, cudaStream_t st, int dv = 0,
+                  bool first = false);
+constexpr int kMaxLaunchTasks = 128;  // tasks of one launch; larger batches take several
+template <int N>
+struct TaskPack {
+    GatherTask t[N];
+};
+// The pack's task whose blocks (units) hold id.
+template <int N>
+__device__ __forceinline__ int find_task(const TaskPack<N> &pack, int n_tasks, uint32_t id) {
+    int lo = 0, hi = n_tasks - 1;
+    while (N > 1 && lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (pack.t[mid].block_begin <= id) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+// Calls f with the tasks copied into the smallest pack that holds them, in runs of
+// at most kMaxLaunchTasks with block_begin counted from the run's first task;
+// f(pack, n_tasks, blocks).
+template <class F>
+inline int for_packs(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, F f) {
+    for (int i = 0; i < n_tasks; i += kMaxLaunchTasks) {
+        const int n = n_tasks - i < kMaxLaunchTasks ? n_tasks - i : kMaxLaunchTasks;
+        const uint32_t begin = tasks[i].block_begin, end = i + n < n_tasks ? tasks[i + n].block_begin : total_blocks;
+        auto fill = [&](auto &pack) {
+            for (int k = 0; k < n; ++k) {
+                pack.t[k] = tasks[i + k];
+                pack.t[k].block_begin -= begin;
+            }
+            return f(pack, n, end - begin);
+        };
+        int rc;
+        if (n == 1) {
+            TaskPack<1> p;
+            rc = fill(p);
+        } else if (n <= 32) {
+            TaskPack<32> p;
+            rc = fill(p);
+        } else {
+            TaskPack<kMaxLaunchTasks> p;
+            rc = fill(p);
+        }
+        if (rc) return rc;
+    }
+    return CP_OK;
+}
 // Set the kernels' shared-memory attributes (call outside stream capture).
 int prepare_gather_kernels();
 // Device error word set by bounded waits in kernels; check_device_error syncs
@@ -240,8 +297,10 @@ int prepare_gather_kernels();
 int *device_error_flag();
 int check_device_error(cudaStream_t st);
 
-// Extract the e0 row laid out [D1][P] into [P][D1].
-int launch_transpose_row(const uint32_t *row, uint32_t *out, int D1, int P, cudaStream_t st);
+// Extract the e0 row laid out [D1][Pp] (signed representatives) into [P][D1]
+// residues in [0, p).
+int launch_transpose_row(const uint32_t *row, uint32_t *out, const uint32_t *primes_dev, int D1, int P, int Pp,
+                         cudaStream_t st);
 
 // ------------------------------------------------------------------ CRT (crt.cu)
 // Device CRT of residues [P][n_coeffs] into limbs [n_coeffs][limbs]; with

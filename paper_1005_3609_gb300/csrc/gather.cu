@@ -12,7 +12,8 @@
 // representatives in [-p, p) that intermediate launches store) is added to a
 // signed 64-bit accumulator and
 // the sum is reduced modulo p once per word (Sec. 3.5), in integer arithmetic
-// only (modred.cuh).
+// only (modred.cuh).  Only the degrees in the states' windows (cp_internal.h)
+// are read, computed and written.
 //
 // One launch processes a batch of independent tasks (factors of different
 // strips); each block belongs to one task and covers 8 * RPW consecutive
@@ -39,20 +40,31 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t x, uint32_t magic) { retur
 constexpr int kWarps = kGatherThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
+// The degrees [lo, hi) that an edge contributes to its destination.
+struct EdgeWin {
+    int lo, hi;
+};
+__device__ __forceinline__ EdgeWin edge_window(const GatherTask &t, const uint2 &q, int dcap_in, int dv) {
+    const int sh = (int)edge_shift(q.x, t.src_bits), lo = (int)(q.y & 0xffu);
+    const int hi = min(dcap_in, t.v_in + dv - (int)((q.y >> 8) & 0xffu)) + 1;
+    return lo == 0xff ? EdgeWin{0, 0} : EdgeWin{lo + sh, hi + sh};
+}
+
 // acc += coef * in[src][chunk c - shift*cpd], for the edges held one per lane
-// in `my` (edge j in lane j), up to four loads in flight per lane.
+// in `my` and `win` (edge j in lane j), up to four loads in flight per lane.
 template <bool V4>
-__device__ __forceinline__ void gather_edges(const GatherTask &t, uint32_t my, int n, uint32_t c, uint32_t deg,
-                                             bool active, long long *acc) {
+__device__ __forceinline__ void gather_edges(const GatherTask &t, uint32_t my, const EdgeWin &win, int n, uint32_t c,
+                                             int deg, bool active, long long *acc) {
     for (int e = 0; e < n; e += 4) {
         uint32_t q[4];
         uint4 x[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             q[j] = __shfl_sync(kFull, my, min(e + j, 31));
+            const int lo = __shfl_sync(kFull, win.lo, min(e + j, 31)), hi = __shfl_sync(kFull, win.hi, min(e + j, 31));
             const uint32_t sh = edge_shift(q[j], t.src_bits);
             x[j] = make_uint4(0, 0, 0, 0);
-            if (e + j < n && active && deg >= sh) {
+            if (e + j < n && active && deg >= lo && deg < hi) {
                 const size_t off = (size_t)edge_src(q[j], t.src_bits) * t.C + (c - sh * t.cpd);
                 if (V4) x[j] = __ldg(reinterpret_cast<const uint4 *>(t.in) + off);
                 else x[j].x = __ldg(t.in + off);
@@ -72,33 +84,41 @@ __device__ __forceinline__ void gather_edges(const GatherTask &t, uint32_t my, i
 }
 
 // One warp per destination row: the row's CSR entries are read once (two
-// row_ptr words, then the edge list one edge per lane) and broadcast with
-// shuffles; the lanes sweep the row's chunks 32 at a time.  The next row's
-// CSR is fetched while the current row is computed.
+// row_ptr words, then the edge list one edge per lane, each with its source's
+// window) and broadcast with shuffles; the lanes sweep the chunks of the row's
+// window 32 at a time.  The next row's CSR is fetched while the current row is
+// computed.
 template <int RPW, bool V4>
-__device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, const ModRed *s_mr) {
+__device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, const ModRed *s_mr, int dv, int first) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int dcap_in = first || t.first ? 0 : t.cap;
     uint32_t row = row0 + warp;
     uint32_t rp = (row < t.rows && lane < 2) ? __ldg(t.row_ptr + row + lane) : 0;
     uint32_t e0 = __shfl_sync(kFull, rp, 0), ne = __shfl_sync(kFull, rp, 1) - e0;
-    uint32_t my = (row < t.rows && lane < ne) ? __ldg(t.edges + e0 + lane) : 0;
+    uint2 my = (row < t.rows && lane < ne) ? __ldg(t.edges + e0 + lane) : make_uint2(0, 0);
 #pragma unroll 1
     for (int k = 0; k < RPW; ++k) {
         if (row >= t.rows) return;
         const uint32_t nrow = row + kWarps;
         uint32_t nrp = (k + 1 < RPW && nrow < t.rows && lane < 2) ? __ldg(t.row_ptr + nrow + lane) : 0;
+        const uint32_t w = __ldg(t.win_out + row);
+        const int lo = (int)(w & 0xffu);
+        const int end = lo == 0xff ? 0 : min(t.cap, t.v_out + dv - (int)(w >> 8)) + 1;
+        const EdgeWin win = (lo < end && lane < ne) ? edge_window(t, my, dcap_in, dv) : EdgeWin{0, 0};
+        const uint32_t c_end = (uint32_t)max(end, 0) * t.cpd;
 #pragma unroll 1
-        for (uint32_t j = t.c0; j < t.c0 + t.cw; j += 32) {
+        for (uint32_t j = (uint32_t)lo * t.cpd; j < c_end; j += 32) {
             const uint32_t c = j + lane;
-            const bool active = c < t.c0 + t.cw;
+            const bool active = c < c_end;
             const uint32_t deg = fast_div(c, t.magic_cpd);
             const uint32_t pc = (c - deg * t.cpd) * (V4 ? 4 : 1);  // prime of the first word
             long long acc[4] = {modred_bias(s_mr[pc].p), V4 ? modred_bias(s_mr[pc + 1].p) : 0,
                                 V4 ? modred_bias(s_mr[pc + 2].p) : 0, V4 ? modred_bias(s_mr[pc + 3].p) : 0};
-            gather_edges<V4>(t, my, (int)min(ne, 32u), c, deg, active, acc);
+            gather_edges<V4>(t, my.x, win, (int)min(ne, 32u), c, (int)deg, active, acc);
             for (uint32_t eb = 32; eb < ne; eb += 32) {  // rows with more than 32 edges
-                const uint32_t mb = (eb + lane < ne) ? __ldg(t.edges + e0 + eb + lane) : 0;
-                gather_edges<V4>(t, mb, (int)min(ne - eb, 32u), c, deg, active, acc);
+                const uint2 mb = (eb + lane < ne) ? __ldg(t.edges + e0 + eb + lane) : make_uint2(0, 0);
+                const EdgeWin wb = (eb + lane < ne) ? edge_window(t, mb, dcap_in, dv) : EdgeWin{0, 0};
+                gather_edges<V4>(t, mb.x, wb, (int)min(ne - eb, 32u), c, (int)deg, active, acc);
             }
             if (active) {
                 const size_t o = (size_t)row * t.C + c;
@@ -114,96 +134,47 @@ __device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, 
         row = nrow;
         e0 = __shfl_sync(kFull, nrp, 0);
         ne = __shfl_sync(kFull, nrp, 1) - e0;
-        my = (row < t.rows && lane < ne) ? __ldg(t.edges + e0 + lane) : 0;
+        my = (row < t.rows && lane < ne) ? __ldg(t.edges + e0 + lane) : make_uint2(0, 0);
     }
 }
 
-template <int RPW>
-__global__ void __launch_bounds__(kGatherThreads) gather_kernel(const GatherTask *__restrict__ tasks, int n_tasks) {
+template <int RPW, int N>
+__global__ void __launch_bounds__(kGatherThreads)
+    gather_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, int dv, int first) {
     __shared__ ModRed s_mr[CP_MAX_PRIMES];
-    // task of this block: the last one whose block_begin <= blockIdx.x (block-uniform)
-    int lo = 0, hi = n_tasks - 1;
-    const uint32_t b = blockIdx.x;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (tasks[mid].block_begin <= b) lo = mid; else hi = mid - 1;
-    }
-    const GatherTask t = tasks[lo];
+    const GatherTask &t = pack.t[find_task(pack, n_tasks, blockIdx.x)];
     if (threadIdx.x < t.n_primes) {
         s_mr[threadIdx.x] = modred_make(__ldg(t.primes + threadIdx.x));
     }
     __syncthreads();
     // rows of the block: row0 + warp + 8 k, k < RPW
-    const uint32_t row0 = (b - t.block_begin) * (uint32_t)(kWarps * RPW);
-    if (t.vec4) gather_rows<RPW, true>(t, row0, s_mr);
-    else gather_rows<RPW, false>(t, row0, s_mr);
+    const uint32_t row0 = (blockIdx.x - t.block_begin) * (uint32_t)(kWarps * RPW);
+    if (t.vec4) gather_rows<RPW, true>(t, row0, s_mr, dv, first);
+    else gather_rows<RPW, false>(t, row0, s_mr, dv, first);
 }
 
-bool tile_is_tma(int items) { return (items & 0xFFF) >= 16; }
+bool tile_is_chunk(int items) { return (items & 0xFFF) >= 16; }
 
 uint32_t task_blocks(const GatherTask &t, int items) {
-    const uint32_t per = tile_is_tma(items) ? (uint32_t)(items & 0xFFE) : (uint32_t)(kWarps * items);
+    if (tile_is_chunk(items)) return t.n_units;
+    const uint32_t per = (uint32_t)(kWarps * items);
     return (t.rows + per - 1) / per;
 }
 
-// For TMA tiles: chunks per thread (bits 24..27) default to 2 for rows wider
-// than 3 KB (192 chunks), else 1; the block shape (bits 28..29) to narrow for
-// rows of 129..160 chunks at one chunk per thread; edges per stage (bits
-// 20..23) to about 20 KB of rows per stage (4 in narrow blocks); the ring
-// (bits 12..19) to what fills the SM at the
-// kernel's occupancy, raised to hold at least two stages of the widest row
-// group.  A batch the TMA kernel cannot take uses the register kernel.
+// A batch the chunk kernel cannot take uses the register kernel.
 int effective_tile(const std::vector<GatherTask> &tasks, int items) {
-    if (!tile_is_tma(items)) return items & 0xFFF;
-    uint32_t max_rb = 0, max_cw = 0, min_cw = 0xffffffffu;
-    for (auto &t : tasks) {
-        if (!tma_usable(t)) return kGatherItems;
-        max_rb = std::max(max_rb, t.cw * 16u);
-        max_cw = std::max(max_cw, t.cw);
-        min_cw = std::min(min_cw, t.cw);
-    }
-    int cpt = (items >> 24) & 15;
-    if (cpt != 1 && cpt != 2 && cpt != 4) cpt = max_cw > 192 ? 2 : 1;
-    // narrow blocks: 5 consumer warps cover rows of 129..160 chunks with at most
-    // 31 idle lanes where the wide block leaves 3 of its 8 warps without a chunk
-    const uint32_t cover = 32u * kTmaNarrowWarps;
-    int shape = tile_shape(items);
-    if (shape != 1 && shape != 2) shape = (cpt == 1 && min_cw > 128 && max_cw <= cover) ? 2 : 1;
-    if (shape == 2 && (cpt != 1 || max_cw > cover)) shape = 1;
-    uint32_t max_g = 1;
-    if (shape == 1)
-        for (auto &t : tasks) {
-            uint32_t G = 1;  // row groups of the kernel's blocks (G * cw <= 256, at most one per consumer warp)
-            while (G < 8u / (uint32_t)cpt && 2 * G * t.cw <= 256) G *= 2;
-            max_g = std::max(max_g, G);
-        }
-    // (a narrow block has one row group)
-    int edges = tile_edges(items);
-    if (edges != 1 && edges != 2 && edges != 4 && edges != 8) {
-        const uint32_t per = max_rb ? 20480u / max_rb : 8u;
-        edges = per >= 8 ? 8 : (per >= 4 ? 4 : (per >= 2 ? 2 : 1));
-        if (shape == 2) edges = 4;  // narrow blocks: six stages of 4 in the 52 KB ring beat three of 8
-    }
-    while ((uint32_t)edges * max_g > 32) edges /= 2;  // the producer warp has one lane per group and slot
-    int ring = (items >> 12) & 0xFF;
-    if (!ring) ring = tma_ring_kb_for(edges, cpt, shape == 2 ? kTmaNarrowWarps : 0);
-    // a row group spans at most 4 KB of slot (G rows of cw chunks, G cw <= 256): two stages need 8 KB per edge
-    ring = std::min(192, std::max(ring, std::max(16, 8 * edges)));
-    return make_tile(items & 0xFFF, ring, edges, cpt) | (shape << 28);
+    if (!tile_is_chunk(items)) return items & 0xFFF;
+    for (auto &t : tasks)
+        if (!chunk_usable(t)) return kGatherItems;
+    return items;
 }
 
-// Rows per block of the default TMA tile: 32, or 16 where 32-row blocks would
-// give a launch fewer than eight waves of resident blocks (about four per SM):
-// on small strips the idle SMs of the last wave then cost more than the
-// smaller blocks' set-up.
-int default_rows(const std::vector<GatherTask> &tasks) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-        sms = 152;
-    uint64_t blocks = 0;
-    for (auto &t : tasks) blocks += (t.rows + 31) / 32;
-    return blocks >= 8ull * 4 * (uint64_t)sms ? 32 : 16;
+bool tile_valid(int tile) {
+    const int rows = tile & 0xFFF, ring = (tile >> 12) & 0xFF, edges = (tile >> 20) & 15, cpt = (tile >> 24) & 15;
+    if (rows == 1 || rows == 2 || rows == 4 || rows == 8) return (tile >> 12) == 0;
+    return (rows == 16 || rows == 32 || rows == 64 || rows == 128) && (tile >> 30) == 0 && ((tile >> 28) & 3) != 3 &&
+           (ring == 0 || (ring >= 16 && ring <= 192)) && (edges <= 2 || edges == 4 || edges == 8) &&
+           (cpt <= 2 || cpt == 4);
 }
 
 uint32_t assign_blocks(std::vector<GatherTask> &tasks, int items) {
@@ -218,57 +189,74 @@ uint32_t assign_blocks(std::vector<GatherTask> &tasks, int items) {
 // ceil(2^32 / d) for d >= 2 (0 encodes d == 1).
 static uint32_t magic_for(uint32_t d) { return d <= 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d); }
 
-void append_gather_tasks(std::vector<GatherTask> *tasks, const SiteTable &tab, const uint32_t *in, uint32_t *out,
-                         const uint32_t *primes_dev, int D1, int P, bool partial) {
+void fill_prime_block(const uint32_t *primes, int n_primes, int lanes, uint32_t *block) {
+    for (int k = 0; k < lanes; ++k) {
+        block[k] = primes[std::min(k, n_primes - 1)];
+        block[CP_MAX_PRIMES + k] = fast_magic(block[k]);
+    }
+}
+
+bool table_fast(const SiteTable &tab, uint32_t min_prime) {
+    return tab.max_abs_coef <= kChunkMaxCoef && fast_ok(tab.max_coef_sum, min_prime);
+}
+
+void append_gather_task(std::vector<GatherTask> *tasks, const SiteTable &tab, const uint32_t *in, uint32_t *out,
+                        const uint32_t *primes_dev, int D1, int P, int v_in, uint32_t min_prime, bool final) {
     const bool v4 = (P % 4) == 0;
     const uint32_t vec = v4 ? 4 : 1;
     GatherTask t{};
     t.in = in;
     t.out = out;
     t.row_ptr = tab.row_ptr;
-    t.edges = tab.edges;
+    t.edges = tab.wedges;
     t.primes = primes_dev;
+    t.win_out = tab.win_out;
+    t.units = tab.units;
+    t.n_units = tab.n_units;
     t.rows = (uint32_t)tab.n_dst;
     t.C = (uint32_t)((uint64_t)D1 * P / vec);
     t.cpd = (uint32_t)P / vec;
     t.vec4 = v4 ? 1 : 0;
     t.magic_cpd = magic_for(t.cpd);
+    t.seg = 32u * kChunkSteps / std::min(t.cpd, 32u * kChunkSteps);
+    t.r32 = 32u % t.cpd;
     t.n_primes = (uint32_t)P;
     t.src_bits = (uint32_t)tab.op.src_bits;
-    t.block_order = tab.block_order;
-    t.partial = partial ? 1u : 0u;
-    t.small_coefs = (tab.max_abs_coef <= kTmaMaxCoef && tab.max_coef_sum < kTmaMaxCoefSum) ? 1u : 0u;
-    const uint32_t ncol = v4 ? (t.C + 255) / 256 : 1;
-    for (uint32_t k = 0; k < ncol; ++k) {  // balanced column ranges
-        t.c0 = (uint32_t)((uint64_t)t.C * k / ncol);
-        t.cw = (uint32_t)((uint64_t)t.C * (k + 1) / ncol) - t.c0;
-        tasks->push_back(t);
-    }
+    t.fast = table_fast(tab, min_prime) ? 1u : 0u;
+    t.fast_k0 = fast_offset(tab.max_coef_sum);
+    t.v_in = v_in;
+    t.v_out = final ? kFinalVertices : v_in + tab.sites;
+    t.cap = D1 - 1;
+    tasks->push_back(t);
 }
 
-int launch_gather_tma(const GatherTask *tasks_dev, int n_tasks, uint32_t total_blocks, int rpb, int *err,
-                      cudaStream_t st, int edges, int ring_kb, int cpt, bool narrow);
-int prepare_gather_tma();
+int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, cudaStream_t st, int dv, bool first);
 
-int launch_gather(const GatherTask *tasks_dev, int n_tasks, uint32_t total_blocks, int items, cudaStream_t st) {
+template <int RPW>
+static int launch_gather_rows(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, cudaStream_t st, int dv,
+                              bool first) {
+    return for_packs(tasks, n_tasks, total_blocks, [&](const auto &pack, int n, uint32_t blocks) -> int {
+        constexpr int N = sizeof(pack.t) / sizeof(GatherTask);
+        if (blocks) gather_kernel<RPW, N><<<blocks, kGatherThreads, 0, st>>>(pack, n, dv, first ? 1 : 0);
+        CP_CUDA_TRY(cudaGetLastError());
+        return CP_OK;
+    });
+}
+
+int launch_gather(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, int items, cudaStream_t st, int dv,
+                  bool first) {
     if (n_tasks <= 0 || total_blocks == 0) return CP_OK;
-    if (tile_is_tma(items))
-        return launch_gather_tma(tasks_dev, n_tasks, total_blocks, items & 0xFFE, device_error_flag(), st,
-                                 tile_edges(items), tile_ring_kb(items), tile_cpt(items), tile_shape(items) == 2);
+    if (tile_is_chunk(items)) return launch_gather_chunk(tasks, n_tasks, total_blocks, st, dv, first);
     switch (items & 0xFFF) {
-        case 1: gather_kernel<1><<<total_blocks, kGatherThreads, 0, st>>>(tasks_dev, n_tasks); break;
-        case 2: gather_kernel<2><<<total_blocks, kGatherThreads, 0, st>>>(tasks_dev, n_tasks); break;
-        case 4: gather_kernel<4><<<total_blocks, kGatherThreads, 0, st>>>(tasks_dev, n_tasks); break;
-        case 8: gather_kernel<8><<<total_blocks, kGatherThreads, 0, st>>>(tasks_dev, n_tasks); break;
-        default: return fail(CP_EINVAL, "gather tile must be 1, 2, 4, 8, 16, 32, 64 or 128");
+        case 1: return launch_gather_rows<1>(tasks, n_tasks, total_blocks, st, dv, first);
+        case 2: return launch_gather_rows<2>(tasks, n_tasks, total_blocks, st, dv, first);
+        case 4: return launch_gather_rows<4>(tasks, n_tasks, total_blocks, st, dv, first);
+        case 8: return launch_gather_rows<8>(tasks, n_tasks, total_blocks, st, dv, first);
     }
-    CP_CUDA_TRY(cudaGetLastError());
-    return CP_OK;
+    return fail(CP_EINVAL, "gather tile must be 1, 2, 4, 8, 16, 32, 64 or 128");
 }
 
 int prepare_gather_kernels() {
-    int rc = prepare_gather_tma();
-    if (rc) return rc;
     return device_error_flag() ? CP_OK : CP_ECUDA;
 }
 
@@ -294,23 +282,25 @@ int check_device_error(cudaStream_t st) {
     CP_CUDA_TRY(cudaMemcpy(&h, f, sizeof(int), cudaMemcpyDeviceToHost));
     if (h) {
         CP_CUDA_TRY(cudaMemset(f, 0, sizeof(int)));
-        return fail(CP_ETIMEOUT, "a bounded wait in the TMA gather kernel ran out, or a block refused its "
+        return fail(CP_ETIMEOUT, "a bounded wait in the chunk gather kernel ran out, or a block refused its "
                                  "configuration (flags " + std::to_string(h) + ")");
     }
     return CP_OK;
 }
 
-// [D1][P] -> [P][D1]
-__global__ void transpose_row_kernel(const uint32_t *row, uint32_t *out, int D1, int P) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
+// [D1][Pp] signed representatives -> [P][D1] residues
+__global__ void transpose_row_kernel(const uint32_t *row, uint32_t *out, const uint32_t *primes, int D1, int P, int Pp) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= D1 * P) return;
-    int d = k / P, p = k - d * P;
-    out[p * D1 + d] = row[k];
+    const int p = k / D1, d = k - p * D1;
+    const uint32_t x = row[(size_t)d * Pp + p];
+    out[k] = (int)x < 0 ? x + primes[p] : x;
 }
 
-int launch_transpose_row(const uint32_t *row, uint32_t *out, int D1, int P, cudaStream_t st) {
-    int n = D1 * P;
-    transpose_row_kernel<<<(n + 255) / 256, 256, 0, st>>>(row, out, D1, P);
+int launch_transpose_row(const uint32_t *row, uint32_t *out, const uint32_t *primes_dev, int D1, int P, int Pp,
+                         cudaStream_t st) {
+    const int n = D1 * P;
+    transpose_row_kernel<<<(n + 255) / 256, 256, 0, st>>>(row, out, primes_dev, D1, P, Pp);
     CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }

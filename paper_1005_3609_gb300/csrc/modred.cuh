@@ -72,4 +72,14 @@ __device__ __forceinline__ uint32_t modred_reduce(long long acc, uint32_t p, uin
     return min(r, r - p);
 }
 
+// The chunk gather's sums (gather_chunk.cu): offset k0 of the upper halves for a
+// coefficient sum s, whether a prime suits it, and the prime's multiplier (below
+// 2^31, as such primes are above 2^17).
+constexpr uint32_t kFastMaxSum = 8192;
+__host__ __device__ __forceinline__ uint32_t fast_offset(uint32_t s) { return (3 * s + 1) / 2; }
+__host__ __device__ __forceinline__ bool fast_ok(uint32_t s, uint32_t p) {
+    return s <= kFastMaxSum && (uint64_t)s * 163840u + 65536u + (((uint64_t)p * (s + 2)) >> 17) + 2u < p;
+}
+__host__ __device__ __forceinline__ uint32_t fast_magic(uint32_t p) { return (uint32_t)((1ull << 48) / p); }
+
 }  // namespace cp

@@ -126,7 +126,7 @@ __device__ uint32_t mu_mod(int idx, const Mod &M) {
 // logarithm, then one thread per coefficient for the weighted sums, then one
 // warp per series for the exponential (the sum of each step spread over the
 // lanes).
-__global__ void flm_series_kernel(const uint32_t *__restrict__ ptilde, const int2 *__restrict__ rects,
+__global__ void flm_series_kernel(uint32_t *__restrict__ ptilde, const int2 *__restrict__ rects,
                                   const uint32_t *__restrict__ primes, SeriesParams sp, uint32_t *__restrict__ out,
                                   int *err) {
     extern __shared__ uint32_t logs[];
@@ -134,7 +134,7 @@ __global__ void flm_series_kernel(const uint32_t *__restrict__ ptilde, const int
     __shared__ uint32_t acc[3][kMaxSeries];
     __shared__ uint32_t E[3][kMaxSeries];
     const int pi = blockIdx.x;
-    const uint32_t p = primes[pi];
+    const uint32_t p = primes[pi / sp.Pg * kPrimeWords + pi % sp.Pg];
     const Mod M = make_mod(p);
     const int n = sp.n, D1 = sp.D1, P = sp.P;
     for (int i = threadIdx.x; i < n; i += blockDim.x) inv[i] = i ? pw((uint32_t)i, p - 2, M) : 0u;
@@ -142,7 +142,7 @@ __global__ void flm_series_kernel(const uint32_t *__restrict__ ptilde, const int
     for (int j = threadIdx.x; j < sp.n_rects; j += blockDim.x) {
         uint32_t f[kMaxSeries], h[kMaxSeries];
         const int grp = pi / sp.Pg, pk = pi - grp * sp.Pg;
-        const uint32_t *src = ptilde + ((size_t)grp * sp.n_rects + j) * D1 * sp.Pg;
+        uint32_t *src = ptilde + ((size_t)grp * sp.n_rects + j) * D1 * sp.Pp;
         for (int i = 0; i < n; ++i) f[i] = 0;
         // Horner: f = P~(w(t)) mod t^n, multiplying by w(t) with its recurrence
         for (int d = min(D1 - 1, n - 1); d >= 0; --d) {
@@ -164,7 +164,10 @@ __global__ void flm_series_kernel(const uint32_t *__restrict__ ptilde, const int
                 }
             }
             for (int i = 0; i < n; ++i) f[i] = h[i];
-            f[0] = ad(f[0], src[(size_t)d * sp.Pg + pk], p);
+            uint32_t c = src[(size_t)d * sp.Pp + pk];  // a signed representative: its residue stays in its place
+            c = (int)c < 0 ? c + p : c;
+            src[(size_t)d * sp.Pp + pk] = c;
+            f[0] = ad(f[0], c, p);
         }
         if (f[0] != 1) atomicOr(err, 1);
         // log f: h = f'/f, g_i = h_{i-1}/i
@@ -226,7 +229,7 @@ __global__ void flm_series_kernel(const uint32_t *__restrict__ ptilde, const int
     }
 }
 
-int launch_flm_series(const uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
+int launch_flm_series(uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
                       uint32_t *out, int *err, cudaStream_t st) {
     size_t shm = (size_t)sp.n_rects * sp.n * 4;
     if (shm > 200 * 1024) return fail(CP_EINVAL, "too many rectangles for the series kernel");

@@ -14,14 +14,16 @@ struct SeriesParams {
     int n;        // terms per series
     int D1;       // coefficients per P~ row (D+1 >= n)
     int P;        // primes
-    int Pg;       // primes per group: ptilde is laid out [P/Pg][n_rects][D1][Pg]
+    int Pg;       // primes per group
+    int Pp;       // prime lanes per group (>= Pg): ptilde is laid out [P/Pg][n_rects][D1][Pp]
     int n_rects;
     int mmax;     // widest strip, (k-1)/2 when the extra square-lattice term applies
     int add_mu;   // 1: add the mu_{2m} z^{4m-1} terms (square lattice, odd k)
 };
 
-// ptilde [P/Pg][n_rects][D1][Pg], rects (r, s), primes [P] -> out [3][P][n].  err |= 1 if a P~ lacks constant term 1.
-int launch_flm_series(const uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
+// ptilde [P/Pg][n_rects][D1][Pp] (signed representatives; each is replaced by its residue in [0, p)), rects (r, s),
+// primes: a prime block per group -> out [3][P][n].  err |= 1 if a P~ lacks constant term 1.
+int launch_flm_series(uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
                       uint32_t *out, int *err, cudaStream_t st);
 
 }  // namespace cp

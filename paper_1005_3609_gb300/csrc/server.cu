@@ -9,7 +9,7 @@
 // traffic.  A job's vectors live in a device arena owned by the server (one
 // allocation made at creation, so admission never calls cudaMalloc); its
 // tables come from the per-device cache.  A step issues ONE batched gather
-// launch (two if some rows cannot take the TMA kernel) holding the next
+// launch (two if some rows cannot take the chunk kernel) holding the next
 // per-site factor of every active job: row factors T_i while the strip grows,
 // then its read-out chain T_i^last, then the extraction of the e_0 row.
 // Requests that arrive while others run are admitted at the next step if
@@ -18,6 +18,7 @@
 // their memory at once.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <deque>
 #include <map>
@@ -106,6 +107,7 @@ struct Job {
     uint32_t *vec[2] = {nullptr, nullptr}, *scratch[2] = {nullptr, nullptr}, *row = nullptr, *tr = nullptr;
     uint32_t *primes_dev = nullptr;
     int op = 0, n_ops = 0;  // next factor, number of factors (rows + read-out)
+    int vertices = 0;       // of the vector the next factor reads (cp_internal.h: degree windows)
     std::vector<uint32_t> result;  // [P][D1]
 };
 
@@ -124,13 +126,10 @@ struct cp_server {
     std::deque<Request *> queue;
     std::vector<std::unique_ptr<Job>> active;
     std::map<uint64_t, std::unique_ptr<Request>> reqs;
-    GatherTask *tasks_dev = nullptr;
-    size_t tasks_cap = 0;
     std::vector<uint64_t> finished;  // ids finished since the last poll
     uint64_t steps = 0, launches = 0, updates = 0;
     ~cp_server() {
         if (stream) cudaStreamSynchronize(stream);
-        dev_free(tasks_dev);
     }
 };
 
@@ -138,7 +137,7 @@ static size_t request_bytes(const TableSet &ts, int L, size_t RB) {
     (void)L;
     const uint64_t sA = ts.last[0].n_dst, sB = ts.last.size() >= 2 ? ts.last[1].n_dst : 1;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    return 2 * al(ts.S_max * RB) + al(sA * RB) + al(sB * RB) + 2 * al(RB) + al(4 * CP_MAX_PRIMES);
+    return 2 * al(ts.S_max * RB) + al(sA * RB) + al(sB * RB) + 2 * al(RB) + al(4 * kPrimeWords);
 }
 
 // Motzkin numbers M_0..M_{CP_MAX_L+1} by eq. (M_recurs), for footprints.
@@ -162,11 +161,11 @@ static size_t request_bytes_estimate(int lattice, int L, int D1, int P) {
     const uint64_t Smax = (lattice == CP_SQUARE && L >= 2) ? cnt(L) + cnt(L - 1) : cnt(L);
     const uint64_t sA = L >= 2 ? cnt(L - 1) : 1, sB = L >= 3 ? cnt(L - 2) : 1;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    return 2 * al(Smax * RB) + al(sA * RB) + al(sB * RB) + 2 * al(RB) + al(4 * CP_MAX_PRIMES);
+    return 2 * al(Smax * RB) + al(sA * RB) + al(sB * RB) + 2 * al(RB) + al(4 * kPrimeWords);
 }
 
 // Largest padded prime count of a job on D1 coefficients: the row must stay a
-// TMA row (at most 1536 16-byte chunks) and within CP_MAX_PRIMES.
+// row of at most 1536 16-byte chunks and within CP_MAX_PRIMES.
 static int job_prime_limit(int D1) {
     int lim = (6144 / D1) & ~3;
     if (lim > CP_MAX_PRIMES) lim = CP_MAX_PRIMES;
@@ -197,13 +196,15 @@ static int admit(cp_server *sv, Job *j, bool *fits) {
     j->scratch[1] = take(sB * RB);
     j->row = take(RB);
     j->tr = take(RB);
-    j->primes_dev = take(4 * CP_MAX_PRIMES);
-    CP_CUDA_TRY(cudaMemcpyAsync(j->primes_dev, j->primes.data(), 4 * j->P, cudaMemcpyHostToDevice, sv->stream));
-    CP_CUDA_TRY(cudaMemsetAsync(j->vec[0], 0, ts.S_b * RB, sv->stream));
+    j->primes_dev = take(4 * kPrimeWords);
+    uint32_t block[kPrimeWords] = {};
+    fill_prime_block(j->primes.data(), j->P, j->P, block);
+    CP_CUDA_TRY(cudaMemcpyAsync(j->primes_dev, block, sizeof(block), cudaMemcpyHostToDevice, sv->stream));
     static const uint32_t ones[CP_MAX_PRIMES] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1,
                                                  1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1};
     CP_CUDA_TRY(cudaMemcpyAsync(j->vec[0], ones, 4 * j->P, cudaMemcpyHostToDevice, sv->stream));
     j->op = 0;
+    j->vertices = j->L;
     j->n_ops = (j->N - 1) * (int)ts.row.size() + (int)ts.last.size();
     return CP_OK;
 }
@@ -216,7 +217,7 @@ static bool next_tasks(Job *j, std::vector<GatherTask> *tasks, uint64_t *upd) {
     const SiteTable *tab;
     const uint32_t *in;
     uint32_t *out;
-    bool partial = true;  // every output but the result feeds further gathers only
+    bool final = false;
     if (j->op < main_ops) {
         const int i = j->op % nrow;
         tab = &ts.row[i];
@@ -226,10 +227,13 @@ static bool next_tasks(Job *j, std::vector<GatherTask> *tasks, uint64_t *upd) {
         const int k = j->op - main_ops;
         tab = &ts.last[k];
         in = k == 0 ? j->vec[main_ops & 1] : j->scratch[(k - 1) & 1];
-        partial = k + 1 < (int)ts.last.size();
-        out = partial ? j->scratch[k & 1] : j->row;
+        final = k + 1 == (int)ts.last.size();
+        out = final ? j->row : j->scratch[k & 1];
     }
-    append_gather_tasks(tasks, *tab, in, out, j->primes_dev, j->D1, j->P, partial);
+    append_gather_task(tasks, *tab, in, out, j->primes_dev, j->D1, j->P, j->vertices,
+                       *std::min_element(j->primes.begin(), j->primes.end()), final);
+    if (j->op == 0) tasks->back().first = 1;
+    j->vertices += tab->sites;
     // updates count the requested primes only (padding lanes are not work asked for)
     int real = 0;
     for (auto &m : j->members) real += m.first->P;
@@ -239,33 +243,18 @@ static bool next_tasks(Job *j, std::vector<GatherTask> *tasks, uint64_t *upd) {
 
 static int launch_batch(cp_server *sv, std::vector<GatherTask> &tasks) {
     if (tasks.empty()) return CP_OK;
-    // TMA-able tasks in one launch, the others in a register-kernel launch
+    // Tasks the chunk kernel takes in one launch, the others in a register-kernel launch
     std::vector<GatherTask> a, b;
-    for (auto &t : tasks) (tma_usable(t) ? a : b).push_back(t);
-    std::vector<GatherTask> all;
-    int tile_a = 0, tile_b = kGatherItems;
-    uint32_t blk_a = 0, blk_b = 0;
-    if (!a.empty()) {
-        tile_a = effective_tile(a, make_tile(default_rows(a), 0, 0, 0));
-        blk_a = assign_blocks(a, tile_a);
-    }
-    if (!b.empty()) blk_b = assign_blocks(b, tile_b);
-    all.insert(all.end(), a.begin(), a.end());
-    all.insert(all.end(), b.begin(), b.end());
-    if (all.size() > sv->tasks_cap) {
-        dev_free(sv->tasks_dev);
-        sv->tasks_dev = nullptr;
-        size_t cap = std::max<size_t>(64, all.size() * 2);
-        int rc = dev_alloc((void **)&sv->tasks_dev, cap * sizeof(GatherTask));
-        if (rc) return rc;
-        sv->tasks_cap = cap;
-    }
-    CP_CUDA_TRY(cudaMemcpyAsync(sv->tasks_dev, all.data(), all.size() * sizeof(GatherTask), cudaMemcpyHostToDevice,
-                                sv->stream));
+    for (auto &t : tasks) (chunk_usable(t) ? a : b).push_back(t);
     int rc;
-    if (!a.empty() && (rc = launch_gather(sv->tasks_dev, (int)a.size(), blk_a, tile_a, sv->stream))) return rc;
-    if (!b.empty() && (rc = launch_gather(sv->tasks_dev + a.size(), (int)b.size(), blk_b, tile_b, sv->stream)))
-        return rc;
+    if (!a.empty()) {
+        const uint32_t units = assign_blocks(a, kTileChunk);
+        if ((rc = launch_gather(a.data(), (int)a.size(), units, kTileChunk, sv->stream))) return rc;
+    }
+    if (!b.empty()) {
+        const uint32_t blocks = assign_blocks(b, kGatherItems);
+        if ((rc = launch_gather(b.data(), (int)b.size(), blocks, kGatherItems, sv->stream))) return rc;
+    }
     sv->launches += (a.empty() ? 0 : 1) + (b.empty() ? 0 : 1);
     return CP_OK;
 }
@@ -314,8 +303,8 @@ extern "C" int cp_server_step(cp_server *sv, int *n_active, int *n_queued, int *
     if (!sv) return fail(CP_EINVAL, "server is NULL");
     int rc;
     // admission: rectangles in the queue order of their first request; queued
-    // requests of the same rectangle form one job (merged while the row stays a
-    // TMA row and the job fits the largest free block)
+    // requests of the same rectangle form one job (merged while the row stays
+    // within job_prime_limit and the job fits the largest free block)
     std::vector<Request *> q(sv->queue.begin(), sv->queue.end());
     std::vector<char> taken(q.size(), 0);
     std::map<uint64_t, std::vector<size_t>> by_shape;
@@ -378,7 +367,7 @@ extern "C" int cp_server_step(cp_server *sv, int *n_active, int *n_queued, int *
         if (next_tasks(j.get(), &tasks, &upd)) finishing.push_back(j.get());
     if ((rc = launch_batch(sv, tasks))) return rc;
     for (Job *j : finishing) {
-        if ((rc = launch_transpose_row(j->row, j->tr, j->D1, j->P, sv->stream))) return rc;
+        if ((rc = launch_transpose_row(j->row, j->tr, j->primes_dev, j->D1, j->P, j->P, sv->stream))) return rc;
         j->result.resize((size_t)j->P * j->D1);
         CP_CUDA_TRY(cudaMemcpyAsync(j->result.data(), j->tr, 4ull * j->P * j->D1, cudaMemcpyDeviceToHost, sv->stream));
     }

@@ -2,6 +2,7 @@
 // C-ABI entry points declared in cp_tm.h.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -78,23 +79,24 @@ int check_primes(const uint32_t *primes, int n) {
 using namespace cp;
 
 struct cp_strip {
-    int lattice = 0, L = 0, P = 0, D1 = 0, max_rows = 0, height = 1;
+    int lattice = 0, L = 0, P = 0, Pp = 0, D1 = 0, max_rows = 0, height = 1;  // Pp: prime lanes of a row
     cudaStream_t stream = nullptr;
     std::shared_ptr<TableSet> tabs;
-    uint32_t *primes_dev = nullptr;
+    uint32_t *primes_dev = nullptr;  // prime block of Pp lanes
     uint32_t *vec[2] = {nullptr, nullptr};
     int cur = 0;
     uint32_t *scratch[2] = {nullptr, nullptr};
     uint32_t *row_out = nullptr;  // [P][D1]
-    uint32_t *ones_dev = nullptr;  // P ones (the e_0 row)
+    uint32_t *ones_dev = nullptr;  // Pp ones (the e_0 row)
     uint32_t *crt_dev = nullptr;   // cp_read_integers: limbs, then flags, then bounds (grown on demand)
     size_t crt_words = 0;
-    GatherTask *tasks_dev = nullptr;
-    int tile = kGatherItems;  // gather tile of this strip's launches
-    // precomputed launches: row factors from vec[0] / vec[1], read-out chain
-    std::vector<std::vector<GatherTask>> row_tasks[2];
-    std::vector<std::vector<GatherTask>> last_tasks[2];
-    std::vector<GatherTask *> row_dev[2], last_dev[2];
+    // precomputed launches: row factors from vec[0] / vec[1] (at height 1), read-out chain
+    struct Launch {
+        GatherTask task;
+        int tile;          // the tile its table can take
+        uint32_t blocks;
+    };
+    std::vector<Launch> row_l[2], last_l[2];
     const uint32_t *last_result[2] = {nullptr, nullptr};
 
     ~cp_strip() {
@@ -105,25 +107,18 @@ struct cp_strip {
         dev_free(scratch[1]);
         dev_free(row_out);
         dev_free(ones_dev);
-        dev_free(tasks_dev);
         dev_free(crt_dev);
     }
 };
 
-static int upload_tasks(cp_strip *s, std::vector<std::vector<GatherTask>> &lists, std::vector<GatherTask *> &ptrs,
-                        std::vector<GatherTask> &all) {
-    for (auto &l : lists) {
-        assign_blocks(l, s->tile);
-        ptrs.push_back(reinterpret_cast<GatherTask *>(all.size()));  // offset, fixed up later
-        all.insert(all.end(), l.begin(), l.end());
-    }
-    return CP_OK;
-}
-
-static uint32_t list_blocks(const std::vector<GatherTask> &l, int tile) {
-    uint32_t n = 0;
-    for (auto &t : l) n += task_blocks(t, tile);
-    return n;
+// Tiles and block counts of the strip's launches.
+static void set_tiles(cp_strip *s, int tile) {
+    for (auto *lists : {s->row_l, s->last_l})
+        for (int b = 0; b < 2; ++b)
+            for (auto &l : lists[b]) {
+                l.tile = effective_tile({l.task}, tile);
+                l.blocks = task_blocks(l.task, l.tile);
+            }
 }
 
 static int check_strip_args(int lattice, int L, const uint32_t *primes, int n_primes, int max_degree, int max_rows,
@@ -141,8 +136,9 @@ static int check_strip_args(int lattice, int L, const uint32_t *primes, int n_pr
     return CP_OK;
 }
 
-// The strip around a table set: state vectors, read-out scratch, precomputed launches.
-static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const uint32_t *primes, int n_primes,
+// The strip around a table set, with Pp prime lanes per row (n_primes, or padded with repeats
+// of the last prime): state vectors, read-out scratch, precomputed launches.
+static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const uint32_t *primes, int n_primes, int Pp,
                       int max_degree, int max_rows, void *cuda_stream, cp_strip **out) {
     int rc = CP_OK;
     long long D = max_degree >= 0 ? max_degree : (long long)L * max_rows - 1;
@@ -150,14 +146,18 @@ static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const 
     s->lattice = lattice;
     s->L = L;
     s->P = n_primes;
+    s->Pp = Pp;
     s->D1 = (int)D + 1;
     s->max_rows = max_rows;
     s->stream = (cudaStream_t)cuda_stream;
     s->tabs = std::move(tabs);
     const TableSet &ts = *s->tabs;
-    const size_t row_words = (size_t)s->D1 * s->P;
-    if ((rc = dev_alloc((void **)&s->primes_dev, 4 * CP_MAX_PRIMES))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(s->primes_dev, primes, 4 * n_primes, cudaMemcpyHostToDevice));
+    const size_t row_words = (size_t)s->D1 * Pp;
+    uint32_t block[kPrimeWords] = {};
+    fill_prime_block(primes, n_primes, Pp, block);
+    const uint32_t min_prime = *std::min_element(primes, primes + n_primes);
+    if ((rc = dev_alloc((void **)&s->primes_dev, sizeof(block)))) return rc;
+    CP_CUDA_TRY(cudaMemcpy(s->primes_dev, block, sizeof(block), cudaMemcpyHostToDevice));
     for (int k = 0; k < 2; ++k)
         if ((rc = dev_alloc((void **)&s->vec[k], ts.S_max * row_words * 4))) return rc;
     // read-out scratch: T_1^last writes cnt[L-1] rows, T_2^last cnt[L-2], ...
@@ -165,53 +165,52 @@ static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const 
     if ((rc = dev_alloc((void **)&s->scratch[0], sA * row_words * 4))) return rc;
     if ((rc = dev_alloc((void **)&s->scratch[1], sB * row_words * 4))) return rc;
     if ((rc = dev_alloc((void **)&s->row_out, row_words * 4))) return rc;
-    // TMA gather when the rows are 16-byte chunked and fit the ring, else the register kernel
-    {
-        std::vector<GatherTask> probe;
-        append_gather_tasks(&probe, ts.row[0], s->vec[0], s->vec[1], s->primes_dev, s->D1, s->P);
-        s->tile = effective_tile(probe, make_tile(default_rows(probe), 0, 0, 0));
-    }
-    // launches of one row (starting from vec[b]) and of the read-out chain from vec[b]
-    std::vector<GatherTask> all;
+    // launches of one row (from vec[b], at height 1) and of the read-out chain from vec[b]
     for (int b = 0; b < 2; ++b) {
-        int cur = b;
-        for (size_t i = 0; i < ts.row.size(); ++i) {
-            std::vector<GatherTask> l;
-            append_gather_tasks(&l, ts.row[i], s->vec[cur], s->vec[cur ^ 1], s->primes_dev, s->D1, s->P, true);
-            s->row_tasks[b].push_back(l);
+        int cur = b, v = L;
+        std::vector<GatherTask> l;
+        for (auto &tab : ts.row) {
+            append_gather_task(&l, tab, s->vec[cur], s->vec[cur ^ 1], s->primes_dev, s->D1, Pp, v, min_prime);
+            v += tab.sites;
             cur ^= 1;
         }
+        for (auto &t : l) s->row_l[b].push_back({t, 0, 0});
+        l.clear();
         const uint32_t *src = s->vec[b];
         int sc = 0;
+        v = L;
         for (size_t i = 0; i < ts.last.size(); ++i) {
-            std::vector<GatherTask> l;
-            append_gather_tasks(&l, ts.last[i], src, s->scratch[sc], s->primes_dev, s->D1, s->P,
-                                i + 1 < ts.last.size());
-            s->last_tasks[b].push_back(l);
+            append_gather_task(&l, ts.last[i], src, s->scratch[sc], s->primes_dev, s->D1, Pp, v, min_prime,
+                               i + 1 == ts.last.size());
+            v += ts.last[i].sites;
             src = s->scratch[sc];
             sc ^= 1;
         }
+        for (auto &t : l) s->last_l[b].push_back({t, 0, 0});
         s->last_result[b] = src;
-        upload_tasks(s.get(), s->row_tasks[b], s->row_dev[b], all);
-        upload_tasks(s.get(), s->last_tasks[b], s->last_dev[b], all);
     }
-    if ((rc = dev_alloc((void **)&s->tasks_dev, all.size() * sizeof(GatherTask)))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(s->tasks_dev, all.data(), all.size() * sizeof(GatherTask), cudaMemcpyHostToDevice));
-    for (int b = 0; b < 2; ++b) {
-        for (auto &p : s->row_dev[b]) p = s->tasks_dev + reinterpret_cast<size_t>(p);
-        for (auto &p : s->last_dev[b]) p = s->tasks_dev + reinterpret_cast<size_t>(p);
-    }
-    // e_0: rank 0 of the NCNNN space, polynomial 1
-    std::vector<uint32_t> one(s->P, 1u);
-    if ((rc = dev_alloc((void **)&s->ones_dev, 4 * s->P))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(s->ones_dev, one.data(), 4 * s->P, cudaMemcpyHostToDevice));
-    CP_CUDA_TRY(cudaMemsetAsync(s->vec[0], 0, ts.S_max * row_words * 4, s->stream));
-    CP_CUDA_TRY(cudaMemcpyAsync(s->vec[0], s->ones_dev, 4 * s->P, cudaMemcpyDeviceToDevice, s->stream));
+    set_tiles(s.get(), kTileChunk);
+    // e_0: rank 0 of the NCNNN space, polynomial 1.  At height 1 no other word is read (degree windows).
+    std::vector<uint32_t> one(Pp, 1u);
+    if ((rc = dev_alloc((void **)&s->ones_dev, 4 * Pp))) return rc;
+    CP_CUDA_TRY(cudaMemcpy(s->ones_dev, one.data(), 4 * Pp, cudaMemcpyHostToDevice));
+    CP_CUDA_TRY(cudaMemcpyAsync(s->vec[0], s->ones_dev, 4 * Pp, cudaMemcpyDeviceToDevice, s->stream));
     CP_CUDA_TRY(cudaStreamSynchronize(s->stream));
     s->cur = 0;
     s->height = 1;
     *out = s.release();
     return CP_OK;
+}
+
+// Rows padded to 16-byte chunks (the chunk kernel); where the vectors do not fit
+// that way, rows of the given primes alone (the register kernel).
+static int make_strip_padded(std::shared_ptr<TableSet> tabs, int lattice, int L, const uint32_t *primes, int n_primes,
+                             int max_degree, int max_rows, void *cuda_stream, cp_strip **out) {
+    const int Pp = padded_primes(n_primes);
+    int rc = make_strip(tabs, lattice, L, primes, n_primes, Pp, max_degree, max_rows, cuda_stream, out);
+    if (rc == CP_ENOMEM && Pp != n_primes)
+        rc = make_strip(std::move(tabs), lattice, L, primes, n_primes, n_primes, max_degree, max_rows, cuda_stream, out);
+    return rc;
 }
 
 extern "C" int cp_create_strip(int lattice, int L, const uint32_t *primes, int n_primes, int max_degree,
@@ -222,7 +221,7 @@ extern "C" int cp_create_strip(int lattice, int L, const uint32_t *primes, int n
     std::shared_ptr<TableSet> tabs;
     const long long D1 = max_degree >= 0 ? max_degree + 1 : (long long)L * max_rows;
     if ((rc = get_tables(lattice, L, (size_t)D1 * n_primes * 4, (cudaStream_t)cuda_stream, &tabs))) return rc;
-    return make_strip(std::move(tabs), lattice, L, primes, n_primes, max_degree, max_rows, cuda_stream, out);
+    return make_strip_padded(std::move(tabs), lattice, L, primes, n_primes, max_degree, max_rows, cuda_stream, out);
 }
 
 extern "C" int cp_create_strip_potts(int lattice, int L, int v, const uint32_t *primes, int n_primes, int max_degree,
@@ -234,34 +233,37 @@ extern "C" int cp_create_strip_potts(int lattice, int L, int v, const uint32_t *
     if ((rc = prepare_gather_kernels()) || (rc = crt_static_touch())) return rc;
     std::shared_ptr<TableSet> tabs;
     if ((rc = get_potts_tables(lattice, L, v, (cudaStream_t)cuda_stream, &tabs))) return rc;
-    return make_strip(std::move(tabs), lattice, L, primes, n_primes, max_degree, max_rows, cuda_stream, out);
+    return make_strip_padded(std::move(tabs), lattice, L, primes, n_primes, max_degree, max_rows, cuda_stream, out);
+}
+
+// One precomputed launch; the tasks' vertex counts are those of height 1.
+static int run_launch(cp_strip *s, const cp_strip::Launch &l, bool first) {
+    const long long dv = (long long)s->L * (s->height - 1);
+    return launch_gather(&l.task, 1, l.blocks, l.tile, s->stream, (int)std::min(dv, 1ll << 24), first);
 }
 
 extern "C" int cp_advance_rows(cp_strip *s, int n_rows) {
     if (!s) return fail(CP_EINVAL, "strip is NULL");
     if (n_rows < 0 || (long long)s->height + n_rows > s->max_rows) return fail(CP_EINVAL, "height would exceed max_rows");
     for (int r = 0; r < n_rows; ++r) {
-        const int b = s->cur;
-        const int nrow = (int)s->row_tasks[b].size();
-        for (int i = 0; i < nrow; ++i) {
-            int rc = launch_gather(s->row_dev[b][i], (int)s->row_tasks[b][i].size(),
-                                   list_blocks(s->row_tasks[b][i], s->tile), s->tile, s->stream);
+        const auto &row = s->row_l[s->cur];
+        for (size_t i = 0; i < row.size(); ++i) {
+            int rc = run_launch(s, row[i], i == 0 && s->height == 1);
             if (rc) return rc;
         }
-        s->cur = (b + nrow) & 1;
+        s->cur = (s->cur + (int)row.size()) & 1;
         s->height += 1;
     }
     return CP_OK;
 }
 
 static int readout(cp_strip *s) {
-    const int b = s->cur;
-    for (size_t i = 0; i < s->last_tasks[b].size(); ++i) {
-        int rc = launch_gather(s->last_dev[b][i], (int)s->last_tasks[b][i].size(),
-                               list_blocks(s->last_tasks[b][i], s->tile), s->tile, s->stream);
+    const auto &last = s->last_l[s->cur];
+    for (size_t i = 0; i < last.size(); ++i) {
+        int rc = run_launch(s, last[i], i == 0 && s->height == 1);
         if (rc) return rc;
     }
-    return launch_transpose_row(s->last_result[b], s->row_out, s->D1, s->P, s->stream);
+    return launch_transpose_row(s->last_result[s->cur], s->row_out, s->primes_dev, s->D1, s->P, s->Pp, s->stream);
 }
 
 extern "C" int cp_read_coeffs_device(cp_strip *s, uint32_t *out_dev, size_t out_len) {
@@ -354,31 +356,15 @@ extern "C" int cp_strip_work(const cp_strip *s, uint64_t work[6]) {
 
 extern "C" int cp_strip_set_tile(cp_strip *s, int tile) {
     if (!s) return fail(CP_EINVAL, "strip is NULL");
-    const int rows = tile & 0xFFF, ring = (tile >> 12) & 0xFF, edges = (tile >> 20) & 15, cpt = (tile >> 24) & 15;
-    const bool reg = (rows == 1 || rows == 2 || rows == 4 || rows == 8) && (tile >> 12) == 0;
-    const bool tma = (rows == 16 || rows == 32 || rows == 64 || rows == 128) && (tile >> 30) == 0 && tile_shape(tile) != 3 &&
-                     (ring == 0 || (ring >= 16 && ring <= 192)) && (edges <= 2 || edges == 4 || edges == 8) &&
-                     (cpt <= 2 || cpt == 4);
-    if (tile != 0 && !reg && !tma) return fail(CP_EINVAL, "bad tile (encoding as for cp_sweep_create)");
-    const int t = effective_tile(s->row_tasks[0][0],
-                                 tile ? tile : make_tile(default_rows(s->row_tasks[0][0]), 0, 0, 0));
+    if (tile != 0 && !tile_valid(tile)) return fail(CP_EINVAL, "bad tile (encoding as for cp_sweep_create)");
     CP_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    s->tile = t;
-    std::vector<GatherTask> all;
-    std::vector<GatherTask *> unused;
-    for (int b = 0; b < 2; ++b) {
-        upload_tasks(s, s->row_tasks[b], unused, all);
-        upload_tasks(s, s->last_tasks[b], unused, all);
-    }
-    CP_CUDA_TRY(cudaMemcpy(s->tasks_dev, all.data(), all.size() * sizeof(GatherTask), cudaMemcpyHostToDevice));
+    set_tiles(s, tile ? tile : kTileChunk);
     return CP_OK;
 }
 
 extern "C" int cp_strip_reset(cp_strip *s) {
     if (!s) return fail(CP_EINVAL, "strip is NULL");
-    const size_t row_words = (size_t)s->D1 * s->P;
-    CP_CUDA_TRY(cudaMemsetAsync(s->vec[0], 0, s->tabs->S_b * row_words * 4, s->stream));
-    CP_CUDA_TRY(cudaMemcpyAsync(s->vec[0], s->ones_dev, 4 * s->P, cudaMemcpyDeviceToDevice, s->stream));
+    CP_CUDA_TRY(cudaMemcpyAsync(s->vec[0], s->ones_dev, 4 * s->Pp, cudaMemcpyDeviceToDevice, s->stream));
     s->cur = 0;
     s->height = 1;
     return CP_OK;

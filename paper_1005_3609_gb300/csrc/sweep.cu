@@ -12,8 +12,8 @@
 // straight into the P~ array.  The primes are split into groups of Pg primes
 // (one strip per width and group).  The whole program -- vector resets, every
 // batched launch and the series kernel -- is captured once into a CUDA graph,
-// so a sweep is a single graph launch.  The gather tile and the prime grouping
-// are picked by timing the candidates (autotune) unless given.
+// so a sweep is a single graph launch.  The prime grouping is picked by timing the
+// candidates (autotune) unless given.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,20 +47,20 @@ int n_terms_for(int lattice, int k) {
 }  // namespace
 
 struct cp_sweep {
-    int lattice = 0, k = 0, P = 0, D1 = 0, n = 0, tile = 0, groups = 0, Pg = 0;
+    int lattice = 0, k = 0, P = 0, D1 = 0, n = 0, tile = 0, groups = 0, Pg = 0, Pp = 0;  // Pp: prime lanes of a group's rows
     cudaStream_t stream = nullptr;
-    uint32_t *primes_dev = nullptr, *ones_dev = nullptr;
+    uint32_t *primes_dev = nullptr, *ones_dev = nullptr;  // primes: a prime block per group
     std::vector<SweepStrip> strips;
     std::vector<int2> rects;
     int2 *rects_dev = nullptr;
-    uint32_t *ptilde_dev = nullptr;  // [groups][n_rects][D1][Pg]
+    uint32_t *ptilde_dev = nullptr;  // [groups][n_rects][D1][Pp]
     uint32_t *series_dev = nullptr;  // [3][P][n]
     uint32_t *crt_dev = nullptr;     // cp_sweep_series_integers: limbs [3][n][limbs], then flags [3][n]
     size_t crt_words = 0;
     std::vector<uint32_t> primes_host;
     int *err_dev = nullptr;
-    GatherTask *tasks_dev = nullptr;
-    std::vector<uint32_t> step_off, step_ntasks, step_blocks;
+    std::vector<std::vector<GatherTask>> steps;  // tasks of each batched launch
+    std::vector<uint32_t> step_blocks;
     std::vector<int> step_tile;
     uint64_t updates = 0, bytes = 0, site_bytes = 0;
     cudaGraph_t graph = nullptr;
@@ -82,7 +82,6 @@ struct cp_sweep {
         dev_free(series_dev);
         dev_free(crt_dev);
         dev_free(err_dev);
-        dev_free(tasks_dev);
     }
 };
 
@@ -104,7 +103,7 @@ static void count_work(cp_sweep *sw, const SiteTable &t, int Pg) {
 // Strips and buffers: one strip per width (and prime group), band rectangles.
 static int build_strips(cp_sweep *sw) {
     const int ngroups = sw->groups, Pg = sw->Pg;
-    const size_t row_words = (size_t)sw->D1 * Pg;
+    const size_t row_words = (size_t)sw->D1 * sw->Pp;
     int rc;
     // band rectangles (r <= s, k-3 <= r+s <= k), ordered by r then s
     for (int r = 1; 2 * r <= sw->k; ++r)
@@ -119,7 +118,7 @@ static int build_strips(cp_sweep *sw) {
             for (auto &rs : sw->rects)
                 if (rs.x == r) st.heights.push_back(rs.y);
             if (st.heights.empty()) continue;
-            if ((rc = get_tables(sw->lattice, r, row_words * 4, sw->stream, &st.tabs))) return rc;
+            if ((rc = get_tables(sw->lattice, r, (size_t)sw->D1 * Pg * 4, sw->stream, &st.tabs))) return rc;
             const TableSet &ts = *st.tabs;
             sw->strips.push_back(st);
             SweepStrip &sp = sw->strips.back();
@@ -140,21 +139,19 @@ static int enqueue_program(cp_sweep *sw);
 static int build_program(cp_sweep *sw, int tile) {
     const int Pg = sw->Pg;
     const int n_rects = (int)sw->rects.size();
-    const size_t row_words = (size_t)sw->D1 * Pg;
+    const size_t row_words = (size_t)sw->D1 * sw->Pp;
     int rc;
     sw->tile = tile;
     sw->updates = sw->bytes = sw->site_bytes = 0;
-    sw->step_off.clear();
-    sw->step_ntasks.clear();
     sw->step_blocks.clear();
     sw->step_tile.clear();
     if (sw->exec) cudaGraphExecDestroy(sw->exec);
     if (sw->graph) cudaGraphDestroy(sw->graph);
     sw->exec = nullptr;
     sw->graph = nullptr;
-    dev_free(sw->tasks_dev);
-    sw->tasks_dev = nullptr;
-    std::vector<std::vector<GatherTask>> steps;
+    const uint32_t pmin = *std::min_element(sw->primes_host.begin(), sw->primes_host.end());
+    auto &steps = sw->steps;
+    steps.clear();
     auto at = [&](size_t t) -> std::vector<GatherTask> & {
         if (steps.size() <= t) steps.resize(t + 1);
         return steps[t];
@@ -162,14 +159,17 @@ static int build_program(cp_sweep *sw, int tile) {
     for (auto &st : sw->strips) {
         const TableSet &ts = *st.tabs;
         const int r = st.r;
-        const uint32_t *pr = sw->primes_dev + st.group * Pg;
+        const uint32_t *pr = sw->primes_dev + st.group * kPrimeWords;
         const int smax = st.heights.back();
         const int nf = (int)ts.row.size();  // launches per row (factors, or pairs of factors)
         // main lane: rows 1..smax-1, launch i of row h is step (h-1)*nf + i
+        int v = r;
         for (int row = 0; row < smax - 1; ++row)
             for (int i = 0; i < nf; ++i) {
                 const size_t t = (size_t)row * nf + i;
-                append_gather_tasks(&at(t), ts.row[i], st.vec[t & 1], st.vec[(t & 1) ^ 1], pr, sw->D1, Pg, true);
+                append_gather_task(&at(t), ts.row[i], st.vec[t & 1], st.vec[(t & 1) ^ 1], pr, sw->D1, sw->Pp, v, pmin);
+                if (t == 0) at(t).back().first = 1;
+                v += ts.row[i].sites;
                 count_work(sw, ts.row[i], Pg);
             }
         // read-out lanes
@@ -178,27 +178,24 @@ static int build_program(cp_sweep *sw, int tile) {
             const uint32_t *src = st.vec[t0 & 1];
             uint32_t *slot = sw->ptilde_dev + ((size_t)st.group * n_rects + rect_index(sw, r, h)) * row_words;
             int sc = 0;
+            v = r * h;
             for (size_t i = 0; i < ts.last.size(); ++i) {
                 const bool final = i + 1 == ts.last.size();
                 uint32_t *dst = final ? slot : st.scratch[sc];
-                append_gather_tasks(&at(t0 + i), ts.last[i], src, dst, pr, sw->D1, Pg, !final);
+                append_gather_task(&at(t0 + i), ts.last[i], src, dst, pr, sw->D1, sw->Pp, v, pmin, final);
+                if (t0 + i == 0) at(0).back().first = 1;  // read out at height 1
+                v += ts.last[i].sites;
                 count_work(sw, ts.last[i], Pg);
                 src = dst;
                 sc ^= 1;
             }
         }
     }
-    std::vector<GatherTask> all;
     for (auto &l : steps) {
         const int et = effective_tile(l, tile);
-        sw->step_off.push_back((uint32_t)all.size());
-        sw->step_ntasks.push_back((uint32_t)l.size());
         sw->step_tile.push_back(et);
         sw->step_blocks.push_back(assign_blocks(l, et));
-        all.insert(all.end(), l.begin(), l.end());
     }
-    if ((rc = dev_alloc((void **)&sw->tasks_dev, std::max<size_t>(1, all.size()) * sizeof(GatherTask)))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(sw->tasks_dev, all.data(), all.size() * sizeof(GatherTask), cudaMemcpyHostToDevice));
     // capture the program into one graph
     CP_CUDA_TRY(cudaStreamBeginCapture(sw->stream, cudaStreamCaptureModeThreadLocal));
     rc = enqueue_program(sw);
@@ -214,16 +211,19 @@ static int build_program(cp_sweep *sw, int tile) {
     return CP_OK;
 }
 
+// Every vector := e_0; at height 1 no other word is read (degree windows).
+static int enqueue_reset(cp_sweep *sw) {
+    for (auto &st : sw->strips)
+        CP_CUDA_TRY(cudaMemcpyAsync(st.vec[0], sw->ones_dev, 4 * sw->Pp, cudaMemcpyDeviceToDevice, sw->stream));
+    return CP_OK;
+}
+
 // Enqueue the whole sweep on sw->stream (used once, under graph capture).
 static int enqueue_program(cp_sweep *sw) {
-    const size_t row_words = (size_t)sw->D1 * sw->Pg;
-    for (auto &st : sw->strips) {  // vector := e_0 over the NCNNN input space of T_1
-        CP_CUDA_TRY(cudaMemsetAsync(st.vec[0], 0, st.tabs->S_b * row_words * 4, sw->stream));
-        CP_CUDA_TRY(cudaMemcpyAsync(st.vec[0], sw->ones_dev, 4 * sw->Pg, cudaMemcpyDeviceToDevice, sw->stream));
-    }
-    for (size_t t = 0; t < sw->step_off.size(); ++t) {
-        int rc = launch_gather(sw->tasks_dev + sw->step_off[t], (int)sw->step_ntasks[t], sw->step_blocks[t],
-                               sw->step_tile[t], sw->stream);
+    int rc = enqueue_reset(sw);
+    if (rc) return rc;
+    for (size_t t = 0; t < sw->steps.size(); ++t) {
+        rc = launch_gather(sw->steps[t].data(), (int)sw->steps[t].size(), sw->step_blocks[t], sw->step_tile[t], sw->stream);
         if (rc) return rc;
     }
     SeriesParams sp{};
@@ -233,6 +233,7 @@ static int enqueue_program(cp_sweep *sw) {
     sp.D1 = sw->D1;
     sp.P = sw->P;
     sp.Pg = sw->Pg;
+    sp.Pp = sw->Pp;
     sp.n_rects = (int)sw->rects.size();
     sp.mmax = sw->k / 2;
     sp.add_mu = (sw->lattice == CP_SQUARE && sw->k % 2 == 1) ? 1 : 0;
@@ -240,8 +241,30 @@ static int enqueue_program(cp_sweep *sw) {
                              sw->stream);
 }
 
+// The primes as the strips hold them: a prime block per group.
+static std::vector<uint32_t> prime_blocks(const cp_sweep *sw) {
+    std::vector<uint32_t> l((size_t)sw->groups * kPrimeWords, 0u);
+    for (int g = 0; g < sw->groups; ++g)
+        fill_prime_block(sw->primes_host.data() + g * sw->Pg, sw->Pg, sw->Pp, l.data() + (size_t)g * kPrimeWords);
+    return l;
+}
+
+// Pp: prime lanes per group, P / groups or that padded to 16-byte chunks.
+static int sweep_build_lanes(int lattice, int k, const uint32_t *primes, int P, int tile, int groups, int Pp,
+                             cudaStream_t stream, cp_sweep **out);
+
+// Rows padded to 16-byte chunks (the chunk kernel); where the vectors do not fit that way, rows of
+// the given primes alone (the register kernel).
 static int sweep_build(int lattice, int k, const uint32_t *primes, int P, int tile, int groups, cudaStream_t stream,
                        cp_sweep **out) {
+    const int Pg = P / groups, Pp = padded_primes(Pg);
+    int rc = sweep_build_lanes(lattice, k, primes, P, tile, groups, Pp, stream, out);
+    if (rc == CP_ENOMEM && Pp != Pg) rc = sweep_build_lanes(lattice, k, primes, P, tile, groups, Pg, stream, out);
+    return rc;
+}
+
+static int sweep_build_lanes(int lattice, int k, const uint32_t *primes, int P, int tile, int groups, int Pp,
+                             cudaStream_t stream, cp_sweep **out) {
     auto sw = std::make_unique<cp_sweep>();
     sw->lattice = lattice;
     sw->k = k;
@@ -250,12 +273,14 @@ static int sweep_build(int lattice, int k, const uint32_t *primes, int P, int ti
     sw->D1 = sw->n;
     sw->groups = groups;
     sw->Pg = P / groups;
+    sw->Pp = Pp;
     sw->stream = stream;
     int rc;
     if ((rc = prepare_gather_kernels()) || (rc = crt_static_touch())) return rc;
     sw->primes_host.assign(primes, primes + P);
-    if ((rc = dev_alloc((void **)&sw->primes_dev, 4 * CP_MAX_PRIMES))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(sw->primes_dev, primes, 4 * P, cudaMemcpyHostToDevice));
+    const std::vector<uint32_t> lanes = prime_blocks(sw.get());
+    if ((rc = dev_alloc((void **)&sw->primes_dev, 4 * lanes.size()))) return rc;
+    CP_CUDA_TRY(cudaMemcpy(sw->primes_dev, lanes.data(), 4 * lanes.size(), cudaMemcpyHostToDevice));
     std::vector<uint32_t> ones(CP_MAX_PRIMES, 1u);
     if ((rc = dev_alloc((void **)&sw->ones_dev, 4 * CP_MAX_PRIMES))) return rc;
     CP_CUDA_TRY(cudaMemcpy(sw->ones_dev, ones.data(), 4 * CP_MAX_PRIMES, cudaMemcpyHostToDevice));
@@ -263,7 +288,7 @@ static int sweep_build(int lattice, int k, const uint32_t *primes, int P, int ti
     for (int r = 1; 2 * r <= k; ++r)
         for (int s = r; r + s <= k; ++s)
             if (r + s >= k - 3) ++n_rects;
-    if ((rc = dev_alloc((void **)&sw->ptilde_dev, 4ull * n_rects * sw->D1 * P))) return rc;
+    if ((rc = dev_alloc((void **)&sw->ptilde_dev, 4ull * n_rects * sw->D1 * Pp * groups))) return rc;
     if ((rc = dev_alloc((void **)&sw->series_dev, 4ull * 3 * P * sw->n))) return rc;
     if ((rc = dev_alloc((void **)&sw->err_dev, sizeof(int)))) return rc;
     CP_CUDA_TRY(cudaMemset(sw->err_dev, 0, sizeof(int)));
@@ -292,7 +317,7 @@ static int sweep_time_once(cp_sweep *sw, float *ms) {
 }
 
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_tuned;  // (dev, lattice, k, P) -> (tile, groups)
+static std::map<std::tuple<int, int, int, int>, int> g_tuned;  // (dev, lattice, k, P) -> groups
 
 extern "C" int cp_sweep_create(int lattice, int k, const uint32_t *primes, int n_primes, int tile, int prime_groups,
                                void *cuda_stream, cp_sweep **out) {
@@ -304,19 +329,10 @@ extern "C" int cp_sweep_create(int lattice, int k, const uint32_t *primes, int n
     int rc = check_primes(primes, n_primes);
     if (rc) return rc;
     if (!cuda_stream) return fail(CP_EINVAL, "the sweep needs a non-default stream (graph capture)");
-    {
-        const int rows = tile & 0xFFF, ring = (tile >> 12) & 0xFF, edges = (tile >> 20) & 15,
-                  cpt = (tile >> 24) & 15;
-        const bool reg = (rows == 1 || rows == 2 || rows == 4 || rows == 8) && (tile >> 12) == 0;
-        const bool tma = (rows == 16 || rows == 32 || rows == 64 || rows == 128) && (tile >> 30) == 0 && tile_shape(tile) != 3 &&
-                         (cpt <= 2 || cpt == 4) &&
-                         (ring == 0 || (ring >= 16 && ring <= 192)) &&
-                         (edges <= 2 || edges == 4 || edges == 8);
-        if (tile != 0 && !reg && !tma)
-            return fail(CP_EINVAL, "tile must be 0 (autotune), 1, 2, 4, 8 (register kernel) or 16, 32, 64, 128 "
-                                   "(TMA) + (ring KB 16..192 << 12) + (edges per stage 1, 2, 4, 8 << 20) + "
-                                   "(chunks per thread 1, 2, 4 << 24) + (block shape 1 wide, 2 narrow << 28)");
-    }
+    if (tile != 0 && !tile_valid(tile))
+        return fail(CP_EINVAL, "tile must be 0 (default), 1, 2, 4, 8 (register kernel) or 16, 32, 64, 128 (chunk "
+                               "kernel), the latter with (16..192 << 12), (1, 2, 4, 8 << 20), (1, 2, 4 << 24) or "
+                               "(1, 2 << 28) or'ed in");
     if (prime_groups < 0 || (prime_groups > 0 && n_primes % prime_groups != 0))
         return fail(CP_EINVAL, "prime_groups must divide n_primes");
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -328,18 +344,12 @@ extern "C" int cp_sweep_create(int lattice, int k, const uint32_t *primes, int n
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(key);
         if (it != g_tuned.end())
-            return sweep_build(lattice, k, primes, n_primes, tile ? tile : it->second.first,
-                               prime_groups ? prime_groups : it->second.second, st, out);
+            return sweep_build(lattice, k, primes, n_primes, tile ? tile : kTileChunk,
+                               prime_groups ? prime_groups : it->second, st, out);
     }
-    // autotune: for each prime grouping build the strips once, re-tile the
-    // launch program for each candidate tile, time one graph run (after a
-    // warm-up run) and keep the fastest (tile, grouping)
-    std::vector<int> tiles = tile ? std::vector<int>{tile}
-                                  : std::vector<int>{make_tile(32, 0, 0, 0), make_tile(64, 0, 0, 0),
-                                                     make_tile(32, 48, 4, 2), make_tile(64, 48, 4, 2),
-                                                     make_tile(32, 64, 8, 1) | kTileWide,
-                                                     make_tile(64, 64, 8, 1) | kTileWide,
-                                                     make_tile(16, 0, 0, 0), 4};
+    // autotune: for each prime grouping build the strips, time one graph run (after a
+    // warm-up run) and keep the fastest grouping
+    const int use = tile ? tile : kTileChunk;
     std::vector<int> grps;
     if (prime_groups) grps = {prime_groups};
     else
@@ -347,29 +357,25 @@ extern "C" int cp_sweep_create(int lattice, int k, const uint32_t *primes, int n
             if (n_primes % g == 0 && (n_primes / g) % 4 == 0) grps.push_back(g);
     if (grps.empty()) grps = {1};
     float best = 1e30f;
-    int bt = tiles[0], bg = grps[0];
+    int bg = grps[0];
     for (int g : grps) {
         cp_sweep *cand = nullptr;
-        if ((rc = sweep_build(lattice, k, primes, n_primes, tiles[0], g, st, &cand))) return rc;
-        for (size_t ti = 0; ti < tiles.size(); ++ti) {
-            if (ti > 0 && (rc = build_program(cand, tiles[ti]))) break;
-            float ms = 0;
-            if ((rc = sweep_time_once(cand, &ms))) break;
-            if ((rc = check_device_error(st))) break;
-            if (ms < best) {
-                best = ms;
-                bt = tiles[ti];
-                bg = g;
-            }
-        }
+        if ((rc = sweep_build(lattice, k, primes, n_primes, use, g, st, &cand))) return rc;
+        float ms = 0;
+        rc = sweep_time_once(cand, &ms);
+        if (!rc) rc = check_device_error(st);
         delete cand;
         if (rc) return rc;
+        if (ms < best) {
+            best = ms;
+            bg = g;
+        }
     }
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tuned[key] = {bt, bg};
+        g_tuned[key] = bg;
     }
-    return sweep_build(lattice, k, primes, n_primes, bt, bg, st, out);
+    return sweep_build(lattice, k, primes, n_primes, use, bg, st, out);
 }
 
 extern "C" int cp_sweep_run(cp_sweep *sw) {
@@ -406,7 +412,7 @@ extern "C" int cp_sweep_info(const cp_sweep *sw, int *n_rects, int *n_terms, int
     if (prime_groups) *prime_groups = sw->groups;
     if (updates_per_run) *updates_per_run = sw->updates;
     if (bytes_per_run) *bytes_per_run = sw->bytes;
-    if (launches_per_run) *launches_per_run = (int)sw->step_off.size() + 1;
+    if (launches_per_run) *launches_per_run = (int)sw->steps.size() + 1;
     return CP_OK;
 }
 
@@ -422,16 +428,16 @@ extern "C" int cp_sweep_rects(const cp_sweep *sw, int *rs_host, int max_rects) {
 
 extern "C" int cp_sweep_read_ptilde(cp_sweep *sw, uint32_t *out_host, size_t out_len) {
     if (!sw || !out_host) return fail(CP_EINVAL, "NULL argument");
-    const int nr = (int)sw->rects.size(), D1 = sw->D1, Pg = sw->Pg;
+    const int nr = (int)sw->rects.size(), D1 = sw->D1, Pg = sw->Pg, Pp = sw->Pp;
     if (out_len < (size_t)nr * sw->P * D1) return fail(CP_EINVAL, "out_len < n_rects*n_primes*n_terms");
-    std::vector<uint32_t> raw((size_t)sw->groups * nr * D1 * Pg);
+    std::vector<uint32_t> raw((size_t)sw->groups * nr * D1 * Pp);
     CP_CUDA_TRY(cudaStreamSynchronize(sw->stream));
     CP_CUDA_TRY(cudaMemcpy(raw.data(), sw->ptilde_dev, raw.size() * 4, cudaMemcpyDeviceToHost));
     for (int g = 0; g < sw->groups; ++g)
         for (int j = 0; j < nr; ++j)
             for (int d = 0; d < D1; ++d)
                 for (int q = 0; q < Pg; ++q)
-                    out_host[((size_t)j * sw->P + g * Pg + q) * D1 + d] = raw[(((size_t)g * nr + j) * D1 + d) * Pg + q];
+                    out_host[((size_t)j * sw->P + g * Pg + q) * D1 + d] = raw[(((size_t)g * nr + j) * D1 + d) * Pp + q];
     return CP_OK;
 }
 
@@ -456,8 +462,20 @@ extern "C" int cp_sweep_set_primes(cp_sweep *sw, const uint32_t *primes, int n_p
     if (n_primes != sw->P) return fail(CP_EINVAL, "n_primes differs from the sweep's");
     int rc = check_primes(primes, n_primes);
     if (rc) return rc;
-    CP_CUDA_TRY(cudaMemcpyAsync(sw->primes_dev, primes, 4ull * n_primes, cudaMemcpyHostToDevice, sw->stream));
+    const uint32_t was = *std::min_element(sw->primes_host.begin(), sw->primes_host.end());
+    const uint32_t now = *std::min_element(primes, primes + n_primes);
     sw->primes_host.assign(primes, primes + n_primes);
+    // primes that another kernel takes (fast_ok) need other launches
+    bool other = false;
+    for (auto &st : sw->strips)
+        for (auto *chain : {&st.tabs->row, &st.tabs->last})
+            for (auto &t : *chain) other = other || table_fast(t, was) != table_fast(t, now);
+    if (other) {
+        CP_CUDA_TRY(cudaStreamSynchronize(sw->stream));
+        if ((rc = build_program(sw, sw->tile))) return rc;
+    }
+    const std::vector<uint32_t> lanes = prime_blocks(sw);
+    CP_CUDA_TRY(cudaMemcpyAsync(sw->primes_dev, lanes.data(), 4 * lanes.size(), cudaMemcpyHostToDevice, sw->stream));
     return CP_OK;
 }
 
@@ -496,20 +514,14 @@ extern "C" int cp_sweep_series_integers(cp_sweep *sw, uint32_t *limbs_out, size_
 // gather launch: sum of gather kernel times and number of gather launches.
 extern "C" int cp_sweep_profile(cp_sweep *sw, float *gather_ms, int *n_gather, float *total_ms) {
     if (!sw) return fail(CP_EINVAL, "sweep is NULL");
-    const size_t nst = sw->step_off.size();
+    const size_t nst = sw->steps.size();
     std::vector<cudaEvent_t> ev(2 * nst + 2);
     for (auto &e : ev) CP_CUDA_TRY(cudaEventCreate(&e));
-    const size_t row_words = (size_t)sw->D1 * sw->Pg;
-    int rc = CP_OK;
     CP_CUDA_TRY(cudaEventRecord(ev[2 * nst], sw->stream));
-    for (auto &st : sw->strips) {
-        CP_CUDA_TRY(cudaMemsetAsync(st.vec[0], 0, st.tabs->S_b * row_words * 4, sw->stream));
-        CP_CUDA_TRY(cudaMemcpyAsync(st.vec[0], sw->ones_dev, 4 * sw->Pg, cudaMemcpyDeviceToDevice, sw->stream));
-    }
+    int rc = enqueue_reset(sw);
     for (size_t t = 0; t < nst && rc == CP_OK; ++t) {
         cudaEventRecord(ev[2 * t], sw->stream);
-        rc = launch_gather(sw->tasks_dev + sw->step_off[t], (int)sw->step_ntasks[t], sw->step_blocks[t],
-                           sw->step_tile[t], sw->stream);
+        rc = launch_gather(sw->steps[t].data(), (int)sw->steps[t].size(), sw->step_blocks[t], sw->step_tile[t], sw->stream);
         cudaEventRecord(ev[2 * t + 1], sw->stream);
     }
     CP_CUDA_TRY(cudaEventRecord(ev[2 * nst + 1], sw->stream));

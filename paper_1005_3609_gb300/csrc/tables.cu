@@ -399,113 +399,216 @@ __global__ void x_partner_kernel(int m, int e, const RankTables *Tg, uint32_t *f
     flag[b] = (alone && (e == 0 || s.v[e - 1] != s.v[e + 1])) ? 1u : 0u;
 }
 
+// ------------------------------------------------------------------ degree windows
+
+// Window words of a space before the shortest paths are known: lo = 255 (not
+// reached), the number of blocks in the high byte; e0 != 0: rank 0 is e_0, lo = 0.
+__global__ void init_win_kernel(Space sp, const RankTables *Tg, uint16_t *win, int e0) {
+    __shared__ RankTables T;
+    stage_tables(T, Tg);
+    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= sp.size) return;
+    Labels s;
+    space_unrank(r, sp, s, T);
+    int blocks = 0;
+    for (int i = 0; i < sp.m; ++i) blocks = max(blocks, (int)s.v[i] + 1);
+    win[r] = (uint16_t)((blocks << 8) | (e0 && r == 0 ? 0 : 255));
+}
+
+// The same for a read-out space: its states are the first ranks of the row space.
+__global__ void copy_blocks_kernel(const uint16_t *win_row, uint16_t *win, uint64_t n) {
+    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < n) win[r] = win_row[r] | 255;
+}
+
+// One relaxation of the shortest paths over a table: lo_dst = min(lo_dst, lo_src + shift).
+// Skipped when *prev is given and zero (the pass before changed nothing); *changed
+// is set where a value fell.
+__global__ void relax_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits,
+                                 const uint16_t *win_in, uint16_t *win_out, const int *prev, int *changed) {
+    if (prev && *prev == 0) return;
+    const uint64_t d = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (d >= n_dst) return;
+    const uint32_t mask = (1u << src_bits) - 1u;
+    uint32_t m = 255;
+    for (uint32_t e = row_ptr[d], e1 = row_ptr[d + 1]; e < e1; ++e) {
+        const uint32_t q = edges[e], lo = win_in[q & mask] & 0xffu;
+        if (lo != 255) m = min(m, min(lo + ((q >> src_bits) & 3u), 254u));
+    }
+    const uint32_t w = win_out[d];
+    if (m < (w & 0xffu)) {
+        win_out[d] = (uint16_t)((w & 0xff00u) | m);
+        *changed = 1;
+    }
+}
+
+// Every transition keeps its source's window inside its destination's: lo_dst <=
+// lo_src + shift, and V_src - blocks_src + shift <= V_dst - blocks_dst.
+__global__ void check_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits, int sites,
+                                 const uint16_t *win_in, const uint16_t *win_out, int *bad) {
+    const uint64_t d = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (d >= n_dst) return;
+    const uint32_t mask = (1u << src_bits) - 1u, w = win_out[d];
+    bool ok = true;
+    for (uint32_t e = row_ptr[d], e1 = row_ptr[d + 1]; e < e1; ++e) {
+        const uint32_t q = edges[e], sh = (q >> src_bits) & 3u, x = win_in[q & mask];
+        if ((x & 0xffu) == 255) continue;
+        ok = ok && (w & 0xffu) <= min((x & 0xffu) + sh, 254u) && (w >> 8) + sh <= (x >> 8) + (uint32_t)sites;
+    }
+    if (!ok) *bad = 1;
+}
+
+// States of degree 0 other than e_0 (rank 0): none in a row space.
+__global__ void check_e0_kernel(const uint16_t *win, uint64_t n, int *bad) {
+    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < n && ((win[r] & 0xffu) == 0) != (r == 0)) *bad = 1;
+}
+
 // ------------------------------------------------------------------ host side
 
-static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *row_ptr, cudaStream_t st) {
+// Working memory of one table set's build: one device allocation, handed out from
+// the start for each table (the build's kernels run on one stream, in order) and
+// freed with the object, instead of a dozen allocations and frees, each a
+// synchronisation, per table.
+struct Scratch {
+    char *base = nullptr;
+    size_t cap = 0, used = 0;
+    cudaStream_t st;
+    explicit Scratch(cudaStream_t s) : st(s) {}
+    Scratch(const Scratch &) = delete;
+    ~Scratch() {
+        if (base) cudaStreamSynchronize(st);
+        dev_free(base);
+    }
+    // Start over with at least `bytes` bytes.
+    int reset(size_t bytes) {
+        used = 0;
+        if (bytes <= cap) return CP_OK;
+        if (base) cudaStreamSynchronize(st);
+        dev_free(base);
+        base = nullptr;
+        cap = 0;
+        const int rc = dev_alloc((void **)&base, bytes);
+        if (!rc) cap = bytes;
+        return rc;
+    }
+    static size_t span(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+    template <class T>
+    T *take(size_t n) {  // (reset() made room)
+        T *p = reinterpret_cast<T *>(base + used);
+        used += span(n * sizeof(T));
+        return p;
+    }
+};
+
+static size_t scan_bytes(uint64_t n) { return Scratch::span(((n + kScanThreads - 1) / kScanThreads + 1) * 4); }
+
+// out[0..n]: exclusive scan of cnt, with the total at the end (asynchronous on sc->st).
+static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *out, Scratch *sc) {
     uint64_t nb = (n + kScanThreads - 1) / kScanThreads;
     if (nb > (1u << 31)) return fail(CP_EINVAL, "scan too large");
-    uint32_t *sums = nullptr;
-    int rc = dev_alloc((void **)&sums, (nb + 1) * sizeof(uint32_t));
-    if (rc) return rc;
-    scan_block_sums<<<(unsigned)nb, kScanThreads, 0, st>>>(cnt, n, sums);
-    scan_sums_serial<<<1, kScanThreads, 0, st>>>(sums, (uint32_t)nb);
-    scan_finish<<<(unsigned)nb, kScanThreads, 0, st>>>(cnt, n, sums, row_ptr);
-    cudaError_t e = cudaGetLastError();
-    cudaStreamSynchronize(st);
-    dev_free(sums);
-    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("scan: ") + cudaGetErrorString(e));
+    uint32_t *sums = sc->take<uint32_t>(nb + 1);
+    scan_block_sums<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums);
+    scan_sums_serial<<<1, kScanThreads, 0, sc->st>>>(sums, (uint32_t)nb);
+    scan_finish<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums, out);
+    CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
 
-int build_x_prefix(int m, int e, cudaStream_t st, uint32_t **out) {
+static int build_x_prefix(int m, int e, Scratch *sc, uint32_t **out) {
     const RankTables *T_dev = nullptr;
     RankTables T;
     int rc = device_rank_tables(&T_dev, &T);
     if (rc) return rc;
     const uint64_t Sb = T.cnt[m];
-    uint32_t *flag = nullptr, *pre = nullptr;
-    if ((rc = dev_alloc((void **)&flag, Sb * 4))) return rc;
-    if ((rc = dev_alloc((void **)&pre, (Sb + 1) * 4))) {
-        dev_free(flag);
-        return rc;
-    }
-    x_partner_kernel<<<(unsigned)((Sb + 127) / 128), 128, 0, st>>>(m, e, T_dev, flag);
-    cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) {
-        dev_free(flag);
-        dev_free(pre);
-        return fail(CP_ECUDA, std::string("x_partner: ") + cudaGetErrorString(ce));
-    }
-    rc = scan_exclusive(flag, Sb, pre, st);
-    dev_free(flag);
+    if ((rc = sc->reset(Scratch::span(Sb * 4) + scan_bytes(Sb)))) return rc;
+    uint32_t *flag = sc->take<uint32_t>(Sb), *pre = nullptr;
+    if ((rc = dev_alloc((void **)&pre, (Sb + 1) * 4))) return rc;
+    x_partner_kernel<<<(unsigned)((Sb + 127) / 128), 128, 0, sc->st>>>(m, e, T_dev, flag);
+    rc = scan_exclusive(flag, Sb, pre, sc);
+    uint32_t total = 0;
+    cudaError_t ce = cudaMemcpyAsync(&total, pre + Sb, 4, cudaMemcpyDeviceToHost, sc->st);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(sc->st);
+    if (!rc && ce != cudaSuccess) rc = fail(CP_ECUDA, std::string("x_partner: ") + cudaGetErrorString(ce));
+    if (!rc && total != T.cnt[m - 1]) rc = fail(CP_ESTATE, "excepted space has the wrong size");
     if (rc) {
         dev_free(pre);
         return rc;
-    }
-    uint32_t total = 0;
-    CP_CUDA_TRY(cudaMemcpy(&total, pre + Sb, 4, cudaMemcpyDeviceToHost));
-    if (total != T.cnt[m - 1]) {
-        dev_free(pre);
-        return fail(CP_ESTATE, "excepted space has the wrong size");
     }
     *out = pre;
     return CP_OK;
 }
 
-// Smallest source state of each row block of `rpb` destination rows (one warp
-// per block; a block without edges gets 0xffffffff).
-__global__ void block_min_src_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint32_t n_dst, uint32_t mask,
-                                     uint32_t rpb, uint32_t nb, uint32_t *key) {
-    const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= nb) return;
-    const uint32_t r0 = w * rpb, r1 = min(n_dst, r0 + rpb);
-    const uint32_t e1 = row_ptr[r1];
-    uint32_t m = 0xffffffffu;
-    for (uint32_t e = row_ptr[r0] + lane; e < e1; e += 32) m = min(m, edges[e] & mask);
-    m = __reduce_min_sync(0xffffffffu, m);
-    if (lane == 0) key[w] = m;
+// Packs the rows of one run of kPackRows into units (cp_internal.h), in order: one
+// thread per run.  Without `units` it only counts them.
+__global__ void pack_units_kernel(const uint32_t *row_ptr, uint64_t n, uint32_t most, uint32_t split, uint32_t *cnt,
+                                  const uint32_t *pos, uint4 *units) {
+    const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, r0 = c * kPackRows;
+    if (r0 >= n) return;
+    const uint64_t r1 = min(n, r0 + kPackRows);
+    uint32_t k = units ? pos[c] : 0;
+    uint64_t u0 = r0;  // first row of the open unit
+    uint32_t ub = row_ptr[r0], b = ub;
+    for (uint64_t r = r0; r <= r1; ++r) {
+        const uint32_t e = r < r1 ? row_ptr[r + 1] : b;  // the row's edges are [b, e)
+        const bool heavy = e - b > split;
+        if (r > u0 && (r == r1 || heavy || e - ub > most || r - u0 == 32)) {  // close the open unit
+            if (units) units[k] = make_uint4((uint32_t)u0, (uint32_t)(r - u0), ub, b);
+            ++k;
+            u0 = r;
+            ub = b;
+        }
+        if (heavy) {
+            for (uint32_t i = 0; i < kSplitParts; ++i) {
+                if (units) units[k] = make_uint4((uint32_t)r, 1u | (1u << 6) | (i << 8), b, e);
+                ++k;
+            }
+            u0 = r + 1;
+            ub = e;
+        }
+        b = e;
+    }
+    if (!units) cnt[c] = k;
 }
 
-constexpr uint64_t kBlockOrderMinRows = 4096;  // smaller tables keep row-block order
+static uint64_t unit_runs(uint64_t n_dst) { return (n_dst + kPackRows - 1) / kPackRows; }
 
-// The order in which the TMA gather's blocks visit a table's row blocks: by
-// the smallest source state a row block reads (ties in row order), for each
-// rows-per-block choice.  Destinations whose sources lie close together then
-// run at the same time, so a source row fetched into L2 serves the blocks that
-// need it before it is evicted -- the factors of the first sites of a row draw
-// their sources from the whole state vector in rank order.  Any order gives
-// the same results; this one only changes DRAM traffic.
-static int build_block_order(SiteTable *tab, cudaStream_t st) {
-    if (tab->n_dst < kBlockOrderMinRows || tab->nnz == 0) return CP_OK;
-    const uint32_t n = (uint32_t)tab->n_dst;
-    const uint32_t total = block_order_offset(n, 256);  // 16, 32, 64 and 128 rows per block
-    uint32_t *key = nullptr;
-    int rc = dev_alloc((void **)&key, (size_t)total * 4);
+// (in the room that build_table reserved)
+static int build_units(SiteTable *tab, Scratch *sc) {
+    const uint64_t n = tab->n_dst, runs = unit_runs(n);
+    uint32_t *cnt = sc->take<uint32_t>(runs), *pos = sc->take<uint32_t>(runs + 1);
+    const unsigned grid = (unsigned)((runs + 63) / 64);
+    const uint32_t most = unit_edges(tab->nnz), split = split_edges(most);
+    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, cnt, nullptr, nullptr);
+    int rc = scan_exclusive(cnt, runs, pos, sc);
     if (rc) return rc;
-    const uint32_t mask = (1u << tab->op.src_bits) - 1u;
-    for (uint32_t l = 16; l <= 128; l *= 2) {
-        const uint32_t nb = (n + l - 1) / l;
-        block_min_src_kernel<<<(nb + 7) / 8, 256, 0, st>>>(tab->row_ptr, tab->edges, n, mask, l, nb,
-                                                           key + block_order_offset(n, l));
-    }
-    std::vector<uint32_t> hk(total), order(total);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hk.data(), key, (size_t)total * 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    dev_free(key);
-    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("block order: ") + cudaGetErrorString(e));
-    for (uint32_t l = 16; l <= 128; l *= 2) {
-        const uint32_t off = block_order_offset(n, l), nb = (n + l - 1) / l;
-        uint32_t *o = order.data() + off;
-        for (uint32_t i = 0; i < nb; ++i) o[i] = i;
-        std::stable_sort(o, o + nb, [&](uint32_t a, uint32_t b) { return hk[off + a] < hk[off + b]; });
-    }
-    if ((rc = dev_alloc((void **)&tab->block_order, (size_t)total * 4))) return rc;
-    CP_CUDA_TRY(cudaMemcpy(tab->block_order, order.data(), (size_t)total * 4, cudaMemcpyHostToDevice));
+    CP_CUDA_TRY(cudaMemcpyAsync(&tab->n_units, pos + runs, 4, cudaMemcpyDeviceToHost, sc->st));
+    CP_CUDA_TRY(cudaStreamSynchronize(sc->st));
+    if ((rc = dev_alloc((void **)&tab->units, std::max<size_t>(1, tab->n_units) * sizeof(uint4)))) return rc;
+    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, nullptr, pos, tab->units);
+    CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
 
-static int build_table(const OpDesc &op, const RankTables *T_dev, cudaStream_t st, SiteTable *tab) {
+// The edges as the gathers read them, one warp per unit: each with its source's
+// window word, its row within the unit and whether it is the row's first.  (A heavy
+// row's parts write the same words.)
+__global__ void fill_wedges_kernel(const uint4 *units, uint32_t n_units, const uint32_t *row_ptr, const uint32_t *edges,
+                                   int src_bits, const uint16_t *win_in, uint2 *out) {
+    const uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (k >= n_units) return;
+    const uint4 u = units[k];
+    const uint32_t nrows = u.y & 63u;
+    for (uint32_t r = 0; r < nrows; ++r) {
+        const uint32_t b = row_ptr[u.x + r], e1 = row_ptr[u.x + r + 1];
+        for (uint32_t e = b + lane; e < e1; e += 32) {
+            const uint32_t q = edges[e];
+            out[e] = make_uint2(q, (uint32_t)win_in[q & ((1u << src_bits) - 1u)] | (r << 16) | (e == b ? 1u << 21 : 0u));
+        }
+    }
+}
+
+static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, SiteTable *tab) {
     tab->op = op;
     tab->n_src = op.in.size;
     tab->n_dst = op.out.size;
@@ -513,33 +616,16 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, cudaStream_t s
     if (op.in.size > ((1ull << op.src_bits) - 1) || op.out.size >= 0xFFFFFFFFull)
         return fail(CP_EINVAL, "state space too large for the edge format");
     const int K = op.max_terms;
-    uint64_t n_slots = op.in.size * (uint64_t)K;
-    uint32_t *slot_dst = nullptr, *slot_edge = nullptr, *cnt = nullptr, *cursor = nullptr, *csum = nullptr;
-    int *err = nullptr;
-    int rc = CP_OK;
-    auto cleanup = [&]() {
-        dev_free(slot_dst);
-        dev_free(slot_edge);
-        dev_free(cnt);
-        dev_free(cursor);
-        dev_free(csum);
-        dev_free(err);
-    };
-    if ((rc = dev_alloc((void **)&slot_dst, n_slots * 4)) || (rc = dev_alloc((void **)&slot_edge, n_slots * 4)) ||
-        (rc = dev_alloc((void **)&cnt, op.out.size * 4)) || (rc = dev_alloc((void **)&cursor, op.out.size * 4)) ||
-        (rc = dev_alloc((void **)&csum, op.out.size * 4)) ||
-        (rc = dev_alloc((void **)&err, 3 * sizeof(int)))) {
-        cleanup();
-        return rc;
-    }
-    if ((rc = dev_alloc((void **)&tab->row_ptr, (op.out.size + 1) * 4))) {
-        cleanup();
-        return rc;
-    }
-    cudaMemsetAsync(cnt, 0, op.out.size * 4, st);
-    cudaMemsetAsync(cursor, 0, op.out.size * 4, st);
-    cudaMemsetAsync(csum, 0, op.out.size * 4, st);
-    cudaMemsetAsync(err, 0, 3 * sizeof(int), st);
+    const uint64_t n_slots = op.in.size * (uint64_t)K, n_dst = op.out.size, runs = unit_runs(n_dst);
+    const cudaStream_t st = sc->st;
+    int rc = sc->reset(2 * Scratch::span(n_slots * 4) + Scratch::span((3 * n_dst + 3) * 4) + scan_bytes(n_dst) +
+                       2 * Scratch::span((runs + 1) * 4) + scan_bytes(runs));
+    if (rc) return rc;
+    uint32_t *slot_dst = sc->take<uint32_t>(n_slots), *slot_edge = sc->take<uint32_t>(n_slots);
+    uint32_t *cnt = sc->take<uint32_t>(3 * n_dst + 3), *cursor = cnt + n_dst, *csum = cursor + n_dst;
+    int *err = reinterpret_cast<int *>(csum + n_dst);
+    if ((rc = dev_alloc((void **)&tab->row_ptr, (n_dst + 1) * 4))) return rc;
+    CP_CUDA_TRY(cudaMemsetAsync(cnt, 0, (3 * n_dst + 3) * 4, st));
     const int bt = 128;
     if (op.fused)
         build_terms_kernel<kMaxFused><<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
@@ -548,74 +634,142 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, cudaStream_t s
         build_terms_kernel<kMaxTerms><<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
                                                                                             slot_edge, K, err);
     count_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, op.src_bits, cnt, csum, err + 2);
-    max_count_kernel<<<608, 256, 0, st>>>(csum, op.out.size, err + 1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        cleanup();
-        return fail(CP_ECUDA, std::string("build_terms: ") + cudaGetErrorString(e));
-    }
-    if ((rc = scan_exclusive(cnt, op.out.size, tab->row_ptr, st))) {
-        cleanup();
-        return rc;
-    }
+    max_count_kernel<<<608, 256, 0, st>>>(csum, n_dst, err + 1);
+    CP_CUDA_TRY(cudaGetLastError());
+    if ((rc = scan_exclusive(cnt, n_dst, tab->row_ptr, sc))) return rc;
     int herr[3] = {0, 0, 0};
     uint32_t nnz = 0;
-    cudaMemcpyAsync(herr, err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(&nnz, tab->row_ptr + op.out.size, 4, cudaMemcpyDeviceToHost, st);
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        cleanup();
-        return fail(CP_ECUDA, std::string("table build: ") + cudaGetErrorString(e));
-    }
+    CP_CUDA_TRY(cudaMemcpyAsync(herr, err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CP_CUDA_TRY(cudaMemcpyAsync(&nnz, tab->row_ptr + n_dst, 4, cudaMemcpyDeviceToHost, st));
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("table build: ") + cudaGetErrorString(e));
     // The gathers reduce p 2^21 + sum_e coef_e x_e (x_e < p) exactly while
     // sum_e |coef_e| into every state stays below 2^20 (modred.cuh).
-    if (herr[0] == 0 && herr[1] >= (int)kReduceMaxCoefSum) {
-        cleanup();
+    if (herr[0] == 0 && herr[1] >= (int)kReduceMaxCoefSum)
         return fail(CP_EINVAL, "too many transitions into one state for the exact modular reduction");
-    }
-    if (herr[0] == 4) {
-        cleanup();
+    if (herr[0] == 4)
         return fail(CP_EINVAL, "a transition coefficient does not fit the " + std::to_string(30 - op.src_bits) +
                                    "-bit field of this width's edge format (|v| too large)");
-    }
-    if (herr[0]) {
-        cleanup();
+    if (herr[0])
         return fail(CP_ESTATE, "transition table check failed (flags " + std::to_string(herr[0]) + ") for op kind " +
                                    std::to_string(op.kind) + " m=" + std::to_string(op.m) + " i=" +
                                    std::to_string(op.i));
-    }
     tab->nnz = nnz;
     tab->max_coef_sum = (uint32_t)herr[1];
     tab->max_abs_coef = (uint32_t)herr[2];
-    if ((rc = dev_alloc((void **)&tab->edges, (size_t)(nnz ? nnz : 1) * 4))) {
-        cleanup();
-        return rc;
-    }
+    if ((rc = dev_alloc((void **)&tab->edges, (size_t)(nnz ? nnz : 1) * 4))) return rc;
     fill_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, tab->row_ptr, cursor, tab->edges);
-    sort_segments_kernel<<<(unsigned)((op.out.size + 255) / 256), 256, 0, st>>>(tab->row_ptr, op.out.size, tab->edges);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cleanup();
-    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("csr fill: ") + cudaGetErrorString(e));
-    return build_block_order(tab, st);
+    sort_segments_kernel<<<(unsigned)((n_dst + 255) / 256), 256, 0, st>>>(tab->row_ptr, n_dst, tab->edges);
+    CP_CUDA_TRY(cudaGetLastError());
+    return build_units(tab, sc);
 }
 
 TableSet::~TableSet() {
     for (auto p : x_prefix) dev_free(p);
+    for (auto p : wins) dev_free(p);
     for (auto &t : row) {
         dev_free(t.row_ptr);
         dev_free(t.edges);
-        dev_free(t.block_order);
+        dev_free(t.wedges);
+        dev_free(t.units);
     }
     for (auto &t : last) {
         dev_free(t.row_ptr);
         dev_free(t.edges);
-        dev_free(t.block_order);
+        dev_free(t.wedges);
+        dev_free(t.units);
     }
 }
 
+// Window words of every space of the two chains (cp_internal.h): the blocks by
+// unranking, lo by relaxing the row's tables from e_0 until a whole row changes
+// nothing (values only fall, a row per pass; a state needs about as many rows as
+// its blocks are nested, so L / 2 + 3 passes mostly do, each a no-op once
+// nothing changes), then the read-out's tables once.
+static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
+    const cudaStream_t st = sc->st;
+    auto grid = [](uint64_t n) { return (unsigned)((n + 127) / 128); };
+    int rc;
+    auto new_win = [&](uint64_t n, uint16_t **w) -> int {
+        if ((rc = dev_alloc((void **)w, n * 2))) return rc;
+        ts->wins.push_back(*w);
+        ts->bytes += n * 2;
+        return CP_OK;
+    };
+    const size_t nf = ts->row.size();
+    std::vector<uint16_t *> win(nf);
+    for (size_t i = 0; i < nf; ++i) {
+        if ((rc = new_win(ts->row[i].n_src, &win[i]))) return rc;
+        init_win_kernel<<<grid(ts->row[i].n_src), 128, 0, st>>>(ts->row[i].op.in, T_dev, win[i], i == 0 ? 1 : 0);
+    }
+    for (size_t i = 0; i < nf; ++i) {
+        ts->row[i].win_in = win[i];
+        ts->row[i].win_out = win[i + 1 < nf ? i + 1 : 0];
+    }
+    const uint16_t *w = win[0];
+    for (auto &t : ts->last) {
+        uint16_t *o = nullptr;
+        if ((rc = new_win(t.n_dst, &o))) return rc;
+        copy_blocks_kernel<<<grid(t.n_dst), 128, 0, st>>>(win[0], o, t.n_dst);
+        t.win_in = w;
+        t.win_out = o;
+        w = o;
+    }
+    constexpr int kMaxPasses = 64;
+    const int per_round = ts->L / 2 + 3;
+    if ((rc = sc->reset((kMaxPasses + 1) * sizeof(int)))) return rc;
+    int *flags = sc->take<int>(kMaxPasses + 1);  // changed, one per pass; then the checks' flag
+    cudaError_t e = cudaMemsetAsync(flags, 0, (kMaxPasses + 1) * sizeof(int), st);
+    auto relax = [&](const SiteTable &t, const int *prev, int *changed) {
+        relax_win_kernel<<<grid(t.n_dst), 128, 0, st>>>(t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.win_in,
+                                                       const_cast<uint16_t *>(t.win_out), prev, changed);
+    };
+    int host[kMaxPasses + 1] = {}, pass = 0;
+    bool done = false;
+    while (e == cudaSuccess && !done && pass < kMaxPasses) {
+        const int to = std::min(kMaxPasses, pass + per_round);
+        for (; pass < to; ++pass)
+            for (auto &t : ts->row) relax(t, pass ? flags + pass - 1 : nullptr, flags + pass);
+        // (the row's part is complete when the last pass changed nothing; the rest is redone otherwise)
+        for (auto &t : ts->last) relax(t, nullptr, flags + kMaxPasses);
+        e = cudaMemsetAsync(flags + kMaxPasses, 0, sizeof(int), st);
+        for (auto *chain : {&ts->row, &ts->last})
+            for (auto &t : *chain)
+                check_win_kernel<<<grid(t.n_dst), 128, 0, st>>>(t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.sites,
+                                                               t.win_in, t.win_out, flags + kMaxPasses);
+        check_e0_kernel<<<grid(ts->row[0].n_src), 128, 0, st>>>(win[0], ts->row[0].n_src, flags + kMaxPasses);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host, flags, sizeof(host), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        done = host[pass - 1] == 0;
+    }
+    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("degree windows: ") + cudaGetErrorString(e));
+    if (!done || host[kMaxPasses]) return fail(CP_ESTATE, "degree windows of the state spaces are inconsistent");
+    // the edges as the gathers read them replace the plain ones
+    for (auto *chain : {&ts->row, &ts->last})
+        for (auto &t : *chain) {
+            if ((rc = dev_alloc((void **)&t.wedges, std::max<size_t>(1, t.nnz) * sizeof(uint2)))) return rc;
+            if (t.n_units)
+                fill_wedges_kernel<<<(t.n_units + 7) / 8, 256, 0, st>>>(t.units, t.n_units, t.row_ptr, t.edges,
+                                                                       t.op.src_bits, t.win_in, t.wedges);
+            CP_CUDA_TRY(cudaGetLastError());
+            if (t.nnz >= (1u << 24)) {  // a wide strip's tables take gigabytes: no second copy of more than one of them
+                CP_CUDA_TRY(cudaStreamSynchronize(st));
+                dev_free(t.edges);
+                t.edges = nullptr;
+            }
+        }
+    CP_CUDA_TRY(cudaStreamSynchronize(st));
+    for (auto *chain : {&ts->row, &ts->last})
+        for (auto &t : *chain) {
+            dev_free(t.edges);
+            t.edges = nullptr;
+        }
+    return CP_OK;
+}
+
 // Identity factor on a 1-state space (T_1^last = D_1 on the width-1 strip).
-static int identity_table(int m, SiteTable *tab) {
+static int identity_table(int m, Scratch *sc, SiteTable *tab) {
     OpDesc op{};
     op.kind = OP_IDENTITY;
     op.m = m;
@@ -631,7 +785,8 @@ static int identity_table(int m, SiteTable *tab) {
     uint32_t rp[2] = {0, 1}, ed = 0u | (1u << (kSrcBits + 2));
     CP_CUDA_TRY(cudaMemcpy(tab->row_ptr, rp, 8, cudaMemcpyHostToDevice));
     CP_CUDA_TRY(cudaMemcpy(tab->edges, &ed, 4, cudaMemcpyHostToDevice));
-    return CP_OK;
+    if ((rc = sc->reset(4096))) return rc;
+    return build_units(tab, sc);
 }
 
 // Tables of a chain of per-site factors: one per factor, or (paired) one
@@ -641,7 +796,7 @@ static int identity_table(int m, SiteTable *tab) {
 // (square) or 10 (triangular), so the edges keep a 2-bit shift and take 26 or
 // 25 source bits; the build checks both bounds.
 static int build_chain(const std::vector<OpDesc> &ops, int paired, int lattice, const RankTables *T_dev,
-                       cudaStream_t st, TableSet *ts, std::vector<SiteTable> *out) {
+                       Scratch *sc, TableSet *ts, std::vector<SiteTable> *out) {
     int rc;
     for (size_t i = 0; i < ops.size();) {
         SiteTable tab;
@@ -653,14 +808,19 @@ static int build_chain(const std::vector<OpDesc> &ops, int paired, int lattice, 
             f.out = ops[i + 1].out;
             f.max_terms = ops[i].kind == OP_LAST ? 4 : (lattice == CP_SQUARE ? 16 : 24);
             f.src_bits = lattice == CP_SQUARE ? 26 : 25;
-            if ((rc = build_table(f, T_dev, st, &tab))) return rc;
+            rc = build_table(f, T_dev, sc, &tab);
             tab.n_site_out = ops[i].out.size + ops[i + 1].out.size;
+            tab.sites = 2;
             i += 2;
         } else {
-            if ((rc = build_table(ops[i], T_dev, st, &tab))) return rc;
+            rc = build_table(ops[i], T_dev, sc, &tab);
             i += 1;
         }
-        ts->bytes += (tab.n_dst + 1 + tab.nnz) * 4;
+        if (rc) {
+            out->push_back(tab);  // the set frees what there is of it
+            return rc;
+        }
+        ts->bytes += (tab.n_dst + 1 + 2 * tab.nnz) * 4;
         out->push_back(tab);
     }
     return CP_OK;
@@ -672,6 +832,7 @@ static int build_tableset(int lattice, int L, int paired, cudaStream_t st, std::
     int rc = device_rank_tables(&T_dev, &T);
     if (rc) return rc;
     auto ts = std::make_shared<TableSet>();
+    Scratch sc(st);
     cudaGetDevice(&ts->device);
     ts->lattice = lattice;
     ts->L = L;
@@ -683,7 +844,7 @@ static int build_tableset(int lattice, int L, int paired, cudaStream_t st, std::
     if (lattice == CP_SQUARE) {
         for (int e = 0; e + 1 < L; ++e) {
             uint32_t *pre = nullptr;
-            if ((rc = build_x_prefix(L, e, st, &pre))) return rc;
+            if ((rc = build_x_prefix(L, e, &sc, &pre))) return rc;
             ts->x_prefix.push_back(pre);
             ts->bytes += (Sb + 1) * 4;
         }
@@ -718,14 +879,15 @@ static int build_tableset(int lattice, int L, int paired, cudaStream_t st, std::
         op.out = Space{SPACE_B, L, 0, 0, T.cnt[L - i - 1], nullptr};
         last_ops.push_back(op);
     }
-    if ((rc = build_chain(row_ops, paired, lattice, T_dev, st, ts.get(), &ts->row))) return rc;
+    if ((rc = build_chain(row_ops, paired, lattice, T_dev, &sc, ts.get(), &ts->row))) return rc;
     if (L == 1) {
         SiteTable tab;
-        if ((rc = identity_table(1, &tab))) return rc;
+        if ((rc = identity_table(1, &sc, &tab))) return rc;
         ts->last.push_back(tab);
-    } else if ((rc = build_chain(last_ops, paired, lattice, T_dev, st, ts.get(), &ts->last))) {
+    } else if ((rc = build_chain(last_ops, paired, lattice, T_dev, &sc, ts.get(), &ts->last))) {
         return rc;
     }
+    if ((rc = build_windows(ts.get(), T_dev, &sc))) return rc;
     *out = ts;
     return CP_OK;
 }
@@ -737,6 +899,7 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
     int rc = device_rank_tables(&T_dev, &T);
     if (rc) return rc;
     auto ts = std::make_shared<TableSet>();
+    Scratch sc(st);
     cudaGetDevice(&ts->device);
     ts->lattice = lattice;
     ts->L = L;
@@ -756,13 +919,14 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
         op.in = Space{SPACE_C, L, 0, 0, S, nullptr};
         op.out = op.in;
         SiteTable tab;
-        if ((rc = build_table(op, T_dev, st, &tab))) return rc;
-        ts->bytes += (tab.n_dst + 1 + tab.nnz) * 4;
+        rc = build_table(op, T_dev, &sc, &tab);
+        ts->bytes += (tab.n_dst + 1 + 2 * tab.nnz) * 4;
         ts->row.push_back(tab);
+        if (rc) return rc;
     }
     if (L == 1) {
         SiteTable tab;
-        if ((rc = identity_table(1, &tab))) return rc;
+        if ((rc = identity_table(1, &sc, &tab))) return rc;
         ts->last.push_back(tab);
     } else {
         for (int i = 0; i + 1 < L; ++i) {  // D_L is the identity on e_0
@@ -776,11 +940,13 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
             op.in = Space{SPACE_C, L, 0, 0, T.cntc[L - i], nullptr};
             op.out = Space{SPACE_C, L, 0, 0, T.cntc[L - i - 1], nullptr};
             SiteTable tab;
-            if ((rc = build_table(op, T_dev, st, &tab))) return rc;
-            ts->bytes += (tab.n_dst + 1 + tab.nnz) * 4;
+            rc = build_table(op, T_dev, &sc, &tab);
+            ts->bytes += (tab.n_dst + 1 + 2 * tab.nnz) * 4;
             ts->last.push_back(tab);
+            if (rc) return rc;
         }
     }
+    if ((rc = build_windows(ts.get(), T_dev, &sc))) return rc;
     *out = ts;
     return CP_OK;
 }
@@ -869,7 +1035,7 @@ int debug_table(int lattice, int L, int paired, int which, int index, uint32_t *
     }
     if (edges_host) {
         if (max_edges < t.nnz) return fail(CP_EINVAL, "max_edges < nnz");
-        CP_CUDA_TRY(cudaMemcpy(edges_host, t.edges, 4 * t.nnz, cudaMemcpyDeviceToHost));
+        CP_CUDA_TRY(cudaMemcpy2D(edges_host, 4, t.wedges, sizeof(uint2), 4, t.nnz, cudaMemcpyDeviceToHost));
     }
     return CP_OK;
 }
@@ -927,7 +1093,8 @@ int check_space(int kind, int m, int e, uint64_t *n_bad, uint64_t *size) {
     Space sp{kind, m, e, 0, kind == SPACE_X ? T.cnt[m] + T.cnt[m - 1] : (kind == SPACE_C ? T.cntc[m] : T.cnt[m]),
              nullptr};
     uint32_t *pre = nullptr;
-    if (kind == SPACE_X && (rc = build_x_prefix(m, e, 0, &pre))) return rc;
+    Scratch sc(nullptr);
+    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pre))) return rc;
     sp.prefix = pre;
     unsigned long long *bad = nullptr;
     if ((rc = dev_alloc((void **)&bad, 8))) {
@@ -967,7 +1134,8 @@ int enumerate_space(int kind, int m, int e, uint8_t *out_host, uint64_t max_stat
     *size = sp.size;
     if (sp.size > max_states) return fail(CP_EINVAL, "output buffer too small");
     uint32_t *pre = nullptr;
-    if (kind == SPACE_X && (rc = build_x_prefix(m, e, 0, &pre))) return rc;
+    Scratch sc(nullptr);
+    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pre))) return rc;
     sp.prefix = pre;
     uint8_t *d = nullptr;
     if ((rc = dev_alloc((void **)&d, sp.size * m))) {
