@@ -198,7 +198,7 @@ def tile_name(tile):
     shape = (tile >> 28) & 3
     if rows <= 8:
         return "register gather kernel, %d rows/warp" % rows
-    return "chunk gather kernel (encoded: %d rows/block, %s KB ring, %s edge(s) per stage, %s chunk(s) per thread, %s)" % (
+    return "chunk gather kernel, encoded as %d rows/block, %s KB ring, %s edge(s) per stage, %s chunk(s) per thread, %s" % (
         rows, ring or "auto", edges or "auto", cpt or "auto",
         {1: "wide blocks", 2: "narrow blocks"}.get(shape, "block shape auto"))
 
