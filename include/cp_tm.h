@@ -149,10 +149,9 @@ void cp_destroy(cp_strip *s);
  * ... of the row and of the read-out chain (an odd one out stays single): a
  * row of L sites takes ceil(L/2) gather launches and the intermediate vector
  * of each pair is never written -- the same matrix product as the
- * factorisation of Sec. 3.2 with half the vector traffic but as many edge
- * copies, which pays only when a state's row, (D+1) n_primes words, is a few
- * KB long.  mode 1 (the default): two-site tables for square-lattice rows of
- * at least 3 KB; mode 2: for every square-lattice strip; mode 3: for every
+ * factorisation of Sec. 3.2 with half the launches and vector traffic and as
+ * many edge copies.  mode 1 (the default): two-site tables where a state's row,
+ * (D+1) n_primes words, has at least 512 bytes (1024 from width 16 on); mode 2: for every square-lattice strip; mode 3: for every
  * strip of both lattices; mode 0: one table per factor, as in the paper.
  * Results are identical in every mode.  Returns the previous mode.  Not thread-safe
  * against concurrent strip creation.

@@ -146,8 +146,9 @@ int device_rank_tables(const RankTables **out_dev, RankTables *host_copy);
 // row_bytes = bytes of one state's row, (D+1) * n_primes * 4, of the caller's vectors.
 int get_tables(int lattice, int L, size_t row_bytes, cudaStream_t stream, std::shared_ptr<TableSet> *out);
 // Library-wide choice for tables built from now on: 0 = one table per factor, 1 = two-site
-// square-lattice tables for rows of at least kPairRowBytes (default), 2 = every square table.
-constexpr size_t kPairRowBytes = 3072;
+// tables for rows of at least kPairRowBytes (twice that from width kPairWide on; default), 2 = every square table, 3 = every table.
+constexpr size_t kPairRowBytes = 512;
+constexpr int kPairWide = 16;
 int factor_pairing();
 int set_factor_pairing(int mode);
 // Tables of the any-v Potts transfer matrix T_i = V_i H_{i,i+1} (square) or

@@ -953,7 +953,7 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
 
 static std::mutex g_cache_mu;
 static std::map<std::tuple<int, int, int>, std::shared_ptr<TableSet>> g_cache[64];  // per device
-static int g_pairing = 1;  // 0 never, 1 square rows of >= kPairRowBytes, 2 every square table, 3 every table
+static int g_pairing = 1;  // 0 never, 1 rows of >= kPairRowBytes, 2 every square table, 3 every table
 
 int factor_pairing() {
     std::lock_guard<std::mutex> lk(g_cache_mu);
@@ -973,12 +973,16 @@ int get_tables(int lattice, int L, size_t row_bytes, cudaStream_t st, std::share
     CP_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(CP_EINVAL, "device index");
     std::lock_guard<std::mutex> lk(g_cache_mu);
-    // Two-site tables halve the vector traffic but not the number of edge copies,
-    // which set the pace on narrow rows: they pay on square-lattice rows of a few
-    // KB and more; on the triangular lattice a pair has up to 21 terms per source
-    // and the gathers ran slower than one factor at a time.
-    const int paired = g_pairing == 3 ||
-                       (lattice == CP_SQUARE && (g_pairing == 2 || (g_pairing == 1 && row_bytes >= kPairRowBytes)));
+    // Two-site tables halve the launches, the vector traffic and the rows to begin and
+    // reduce, with as many edges in all.  Per row, one table per factor and two-site:
+    // square width 16 D 63 on 16 primes 4.81 and 3.96 ms, width 14 on 4 primes 0.467 and
+    // 0.327 ms, width 8 D 71 on 8 primes 62 and 35 us; triangular width 16 D 32 on 16
+    // primes 1.42 and 1.36 ms, width 13 D 181 on 4 primes 0.274 and 0.247 ms, width 9
+    // D 80 on 8 primes 77 and 45 us.  Not on wide strips of short rows, where launches
+    // are long and there is little to reduce: square width 17 D 40 on 5 primes, four
+    // rows and the read-out, 6.76 and 7.08 ms.
+    const int paired = g_pairing == 3 || (lattice == CP_SQUARE && g_pairing == 2) ||
+                       (g_pairing == 1 && row_bytes >= (L < kPairWide ? kPairRowBytes : 2 * kPairRowBytes));
     auto key = std::make_tuple(lattice, L, paired);
     auto it = g_cache[dev].find(key);
     if (it != g_cache[dev].end()) {
