@@ -284,6 +284,7 @@ struct Warp {
         }
         const uint32_t smask = (1u << t.src_bits) - 1u;
         bool open_row = false;
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // the launch before this one has finished
 #pragma unroll 1
         for (uint32_t cb = u.z;;) {  // passes over the unit, at most t.seg degrees of each row at a time
             const uint32_t b = min(a + t.seg, hi);
@@ -328,6 +329,8 @@ struct Warp {
 };
 
 // dv is added to the tasks' vertex counts; first: as if every task's `first` were set.
+// Launches overlap: a launch's blocks may start while the one before it drains, load
+// their unit's tables (which no launch writes) and only then wait for it.
 template <int N>
 __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, int dv, int first) {
@@ -335,6 +338,7 @@ __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     __shared__ uint4 lists[kWarps][32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t id = blockIdx.x * kWarps + warp;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (id >= n_units) return;
     const GatherTask &t = pack.t[find_task(pack, n_tasks, id)];
     Warp w(t, lists[warp]);
@@ -364,8 +368,18 @@ int debug_wait_timeout(long long cycles, cudaStream_t st) {
 int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, cudaStream_t st, int dv, bool first) {
     return for_packs(tasks, n_tasks, n_units, [&](const auto &pack, int n, uint32_t units) -> int {
         constexpr int N = sizeof(pack.t) / sizeof(GatherTask);
-        if (units) gather_chunk_kernel<N><<<(units + kWarps - 1) / kWarps, 32 * kWarps, kWarps * kDepth * kSlotBytes, st>>>(pack, n, units, dv, first ? 1 : 0);
-        CP_CUDA_TRY(cudaGetLastError());
+        if (!units) return CP_OK;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((units + kWarps - 1) / kWarps);
+        cfg.blockDim = dim3(32 * kWarps);
+        cfg.dynamicSmemBytes = kWarps * kDepth * kSlotBytes;
+        cfg.stream = st;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        CP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N>, pack, n, units, dv, first ? 1 : 0));
         return CP_OK;
     });
 }
