@@ -308,7 +308,7 @@ int launch_transpose_row(const uint32_t *row, uint32_t *out, const uint32_t *pri
 // flags_dev, per-coefficient flags (bit 0: bound_dev[j] + 2 > bit length of the
 // prime product; bit 1: the first P-1 primes give another value).
 int launch_crt(const uint32_t *res_dev, const uint32_t *primes_host, int P, int n_coeffs, uint32_t *limbs_dev,
-               int limbs, const uint32_t *bound_dev, uint32_t *flags_dev, cudaStream_t st);
+               int limbs, const uint32_t *bound_dev, uint32_t *flags_dev, cudaStream_t st, int arrays = 1);
 int primes_product_bits(const uint32_t *primes, int P);
 // Bit lengths of C(n_edges, j), j < n_coeffs (Whitney's bound |c_j| <= C(|E|, j)).
 void binomial_bits(uint64_t n_edges, int n_coeffs, uint32_t *bits_out);

@@ -15,43 +15,10 @@
 #include <cuda_runtime.h>
 
 #include "cp_internal.h"
+#include "modarith.cuh"
 #include "series.h"
 
 namespace cp {
-
-// Arithmetic modulo a prime p < 2^31.  Products use Barrett reduction with
-// m = floor((2^64 - 1) / p): q = floor(x m / 2^64) undershoots floor(x / p) by at
-// most 2 for x < 2^62, so x - q p < 3p needs at most two subtractions.
-struct Mod {
-    uint32_t p;
-    uint64_t m;
-};
-__device__ __forceinline__ Mod make_mod(uint32_t p) { return Mod{p, 0xFFFFFFFFFFFFFFFFull / p}; }
-__device__ __forceinline__ uint32_t mm(uint32_t a, uint32_t b, const Mod &M) {
-    const uint64_t x = (uint64_t)a * b;
-    uint64_t r = x - __umul64hi(x, M.m) * M.p;
-    if (r >= M.p) r -= M.p;
-    if (r >= M.p) r -= M.p;
-    return (uint32_t)r;
-}
-__device__ __forceinline__ uint32_t ad(uint32_t a, uint32_t b, uint32_t p) {
-    uint32_t t = a + b;
-    return t >= p ? t - p : t;
-}
-__device__ __forceinline__ uint32_t sb(uint32_t a, uint32_t b, uint32_t p) { return a >= b ? a - b : a + p - b; }
-__device__ __forceinline__ uint32_t from_int(long long v, uint32_t p) {
-    long long r = v % (long long)p;
-    return (uint32_t)(r < 0 ? r + p : r);
-}
-__device__ uint32_t pw(uint32_t a, uint32_t e, const Mod &M) {
-    uint32_t r = 1;
-    while (e) {
-        if (e & 1) r = mm(r, a, M);
-        a = mm(a, a, M);
-        e >>= 1;
-    }
-    return r;
-}
 
 // Finite-lattice weights (Sec. 4.1); beta with (r+s+2)/2 on delta_{r+s,k-3}
 // (the printed (r+s-2)/2 violates the sum rules), all integers.
@@ -72,170 +39,235 @@ __device__ long long flm_weight(int which, int k, int r, int s) {
     return f * c;
 }
 
+// The value of `v` (one of M registers a lane, entry i in lane i % 32, register i / 32) at index i.
+template <int M>
+__device__ __forceinline__ uint32_t lane_value(const uint32_t (&v)[M], int i) {
+    uint32_t x = 0;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const uint32_t y = __shfl_sync(0xffffffffu, v[m], i & 31);
+        x = (i >> 5) == m ? y : x;
+    }
+    return x;
+}
+
+constexpr int kSeriesWarps = 8;           // rectangles per block
+constexpr int kSeriesRegs = kMaxSeries / 32;
+
 // mu_{2m} mod p from sum_{p>=4} mu_p y^p = y^4 (2-2y-y sqrt(1-4y)) / ((1-4y)(2+y))
 //                                        + y^6 (3-4y-4 sqrt(1-4y)) / (1-4y)^2      (y = x^2)
-__device__ uint32_t mu_mod(int idx, const Mod &M) {
+// by one warp; tmp: six rows of kMaxSeries words.
+__device__ uint32_t mu_mod(int idx, const Mod &M, const uint32_t *inv, uint32_t (*tmp)[kMaxSeries], int lane) {
     const uint32_t p = M.p;
     const int n = idx + 1;
-    uint32_t sq[kMaxSeries], g1[kMaxSeries], q1[kMaxSeries], t1[kMaxSeries], t2[kMaxSeries];
+    uint32_t *sq = tmp[0], *g1 = tmp[1], *q1 = tmp[2], *a = tmp[3], *b = tmp[4], *t = tmp[5];
     // sqrt(1-4y) = 1 - 2 sum_{j>=1} C_{j-1} y^j, Catalan C_j = C_{j-1} 2(2j-1)/(j+1)
-    uint32_t cat = 1;
-    sq[0] = 1;
-    for (int j = 1; j < n; ++j) {
-        sq[j] = sb(0, mm(2, cat, M), p);
-        cat = mm(mm(cat, from_int(2 * (2 * j - 1), p), M), pw(j + 1, p - 2, M), M);
-    }
-    const uint32_t inv2 = pw(2, p - 2, M);
+    const uint32_t inv2 = (p + 1) / 2;
+    uint32_t cat = 1, pow4 = 1, half = inv2;
     for (int j = 0; j < n; ++j) {
-        g1[j] = pw(4, j, M);                                    // 1/(1-4y)
-        q1[j] = mm(j & 1 ? p - 1 : 1, pw(inv2, j + 1, M), M);   // 1/(2+y)
-    }
-    // numerators
-    uint32_t a[kMaxSeries], b[kMaxSeries];
-    for (int j = 0; j < n; ++j) {
-        a[j] = (j == 0 ? 2 : 0);
-        if (j == 1) a[j] = sb(a[j], 2, p);
-        if (j >= 1) a[j] = sb(a[j], sq[j - 1], p);
-        b[j] = (j == 0 ? 3 : 0);
-        if (j == 1) b[j] = sb(b[j], 4, p);
-        b[j] = sb(b[j], mm(4, sq[j], M), p);
-    }
-    for (int j = 0; j < n; ++j) {  // t1 = a * g1 * q1, t2 = b * g1 * g1
-        uint32_t x = 0, y = 0;
-        for (int i = 0; i <= j; ++i) {
-            x = ad(x, mm(a[i], g1[j - i], M), p);
-            y = ad(y, mm(g1[i], g1[j - i], M), p);
+        if (lane == 0) {
+            sq[j] = j ? sb(0, mm(2, cat, M), p) : 1;
+            g1[j] = pow4;                             // 1/(1-4y)
+            q1[j] = j & 1 ? sb(0, half, p) : half;    // 1/(2+y)
         }
-        t1[j] = x;
-        t2[j] = y;
+        if (j) cat = mm(mm(cat, from_int(2 * (2 * j - 1), p), M), inv[j + 1], M);
+        pow4 = mm(pow4, 4, M);
+        half = mm(half, inv2, M);
     }
-    uint32_t u = 0, v = 0;
-    if (idx >= 4) {
-        int j = idx - 4;
-        for (int i = 0; i <= j; ++i) u = ad(u, mm(t1[i], q1[j - i], M), p);
+    __syncwarp();
+    for (int j = lane; j < n; j += 32) {  // numerators
+        uint32_t x = j == 0 ? 2 : 0, y = j == 0 ? 3 : 0;
+        if (j == 1) x = sb(x, 2, p);
+        if (j >= 1) x = sb(x, sq[j - 1], p);
+        if (j == 1) y = sb(y, 4, p);
+        a[j] = x;
+        b[j] = sb(y, mm(4, sq[j], M), p);
     }
-    if (idx >= 6) {
-        int j = idx - 6;
-        for (int i = 0; i <= j; ++i) v = ad(v, mm(b[i], t2[j - i], M), p);
+    __syncwarp();
+    // idx-th coefficients: y^4 (a g1) q1 and y^6 b (g1 g1)
+    for (int j = lane; j < n; j += 32) {
+        uint32_t x = 0;
+        for (int i = 0; i <= j; ++i) x = ad(x, mm(a[i], g1[j - i], M), p);
+        t[j] = x;
     }
-    return ad(u, v, p);
+    __syncwarp();
+    uint32_t u = 0;
+    for (int i = lane; i <= idx - 4; i += 32) u = ad(u, mm(t[i], q1[idx - 4 - i], M), p);
+    __syncwarp();
+    for (int j = lane; j < n; j += 32) {
+        uint32_t y = 0;
+        for (int i = 0; i <= j; ++i) y = ad(y, mm(g1[i], g1[j - i], M), p);
+        t[j] = y;
+    }
+    __syncwarp();
+    for (int i = lane; i <= idx - 6; i += 32) u = ad(u, mm(b[i], t[idx - 6 - i], M), p);
+    for (int o = 16; o > 0; o >>= 1) u = ad(u, __shfl_xor_sync(0xffffffffu, u, o), p);
+    return u;
 }
 
-// One block per prime.  Shared: logs[n_rects][n], the inverses 1/i (i < n) and
-// the three weighted sums; one thread per rectangle for its substitution and
-// logarithm, then one thread per coefficient for the weighted sums, then one
-// warp per series for the exponential (the sum of each step spread over the
-// lanes).
-__global__ void flm_series_kernel(uint32_t *__restrict__ ptilde, const int2 *__restrict__ rects,
-                                  const uint32_t *__restrict__ primes, SeriesParams sp, uint32_t *__restrict__ out,
-                                  int *err) {
-    extern __shared__ uint32_t logs[];
+// One block per prime and kSeriesWarps rectangles, one warp per rectangle for its
+// substitution and logarithm; the block that finishes a prime's last rectangle
+// combines the prime's logarithms and takes the exponentials, one warp per series.
+// What bounds it: chains of dependent modular products.  Every recurrence is run
+// outward -- an entry that is final is sent to all lanes, which add its products to
+// the entries still open -- so a step costs one exchange and one product instead of
+// a sum over the entries before it: k = 17 on 8 primes 178 -> 39 us (one thread per
+// rectangle and one block per prime before), k = 33 on 16 primes 73 us.
+__global__ void __launch_bounds__(32 * kSeriesWarps)
+    flm_series_kernel(uint32_t *__restrict__ ptilde, const int2 *__restrict__ rects, const uint32_t *__restrict__ primes,
+                      SeriesParams sp, uint32_t *__restrict__ logs, uint32_t *__restrict__ finished,
+                      uint32_t *__restrict__ out, int *err) {
+    extern __shared__ uint32_t B[];  // [n][n + 1]: coefficient of t^i in w(t)^d
     __shared__ uint32_t inv[kMaxSeries];
-    __shared__ uint32_t acc[3][kMaxSeries];
-    __shared__ uint32_t E[3][kMaxSeries];
-    const int pi = blockIdx.x;
-    const uint32_t p = primes[pi / sp.Pg * kPrimeWords + pi % sp.Pg];
+    __shared__ uint32_t work[kSeriesWarps][kMaxSeries];
+    __shared__ uint32_t tmp[6][kMaxSeries];
+    __shared__ uint32_t wgt[3][kMaxSeriesRects];
+    __shared__ uint32_t last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int pi = blockIdx.y, grp = pi / sp.Pg, pk = pi - grp * sp.Pg;
+    const uint32_t p = primes[grp * kPrimeWords + pk];
     const Mod M = make_mod(p);
-    const int n = sp.n, D1 = sp.D1, P = sp.P;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) inv[i] = i ? pw((uint32_t)i, p - 2, M) : 0u;
-    __syncthreads();
-    for (int j = threadIdx.x; j < sp.n_rects; j += blockDim.x) {
-        uint32_t f[kMaxSeries], h[kMaxSeries];
-        const int grp = pi / sp.Pg, pk = pi - grp * sp.Pg;
-        uint32_t *src = ptilde + ((size_t)grp * sp.n_rects + j) * D1 * sp.Pp;
-        for (int i = 0; i < n; ++i) f[i] = 0;
-        // Horner: f = P~(w(t)) mod t^n, multiplying by w(t) with its recurrence
-        for (int d = min(D1 - 1, n - 1); d >= 0; --d) {
-            if (sp.lattice == CP_SQUARE) {  // * z/(1+z):  y_i = f_{i-1} - y_{i-1}
-                uint32_t prev = 0;
-                for (int i = 0; i < n; ++i) {
-                    uint32_t s = i ? f[i - 1] : 0;
-                    uint32_t y = sb(s, prev, p);
-                    h[i] = y;
-                    prev = y;
-                }
-            } else {  // * -x/(1-x)^2: shift, two prefix sums, negate
-                uint32_t u = 0, v = 0;
-                for (int i = 0; i < n; ++i) {
-                    uint32_t s = i ? f[i - 1] : 0;
-                    u = ad(u, s, p);
-                    v = ad(v, u, p);
-                    h[i] = sb(0, v, p);
-                }
+    const int n = sp.n, ld = n + 1;
+    for (int i = tid; i < n; i += blockDim.x) inv[i] = i ? pw((uint32_t)i, p - 2, M) : 0u;
+    // w = z/(1+z): (1+z) w^d = z w^(d-1);  w = -x/(1-x)^2: (1-x)^2 w^d = -x w^(d-1)
+    for (int i = 0; i < n; ++i) {
+        if (tid < n) {
+            const int d = tid;
+            const uint32_t up = i >= 1 ? B[(i - 1) * ld + d] : 0u, left = i >= 1 && d >= 1 ? B[(i - 1) * ld + d - 1] : 0u;
+            uint32_t x = i == 0 && d == 0 ? 1u : 0u;
+            if (d >= 1 && i >= 1) {
+                if (sp.lattice == CP_SQUARE) x = sb(left, up, p);
+                else x = sb(sb(ad(up, up, p), i >= 2 ? B[(i - 2) * ld + d] : 0u, p), left, p);
             }
-            for (int i = 0; i < n; ++i) f[i] = h[i];
-            uint32_t c = src[(size_t)d * sp.Pp + pk];  // a signed representative: its residue stays in its place
-            c = (int)c < 0 ? c + p : c;
-            src[(size_t)d * sp.Pp + pk] = c;
-            f[0] = ad(f[0], c, p);
+            B[i * ld + d] = x;
         }
-        if (f[0] != 1) atomicOr(err, 1);
-        // log f: h = f'/f, g_i = h_{i-1}/i
-        for (int i = 0; i + 1 < n; ++i) {
-            uint32_t a = mm(f[i + 1], (uint32_t)(i + 1), M);
-            for (int q = 1; q <= i; ++q) a = sb(a, mm(f[q], h[i - q], M), p);
-            h[i] = a;
-        }
-        uint32_t *g = logs + (size_t)j * n;
-        g[0] = 0;
-        for (int i = 1; i < n; ++i) g[i] = mm(h[i - 1], inv[i], M);
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        uint32_t a0 = 0, a1 = 0, a2 = 0;
-        for (int j = 0; j < sp.n_rects; ++j) {
-            const int r = rects[j].x, s = rects[j].y;
-            uint32_t g = logs[(size_t)j * n + i];
-            a0 = ad(a0, mm(from_int(flm_weight(0, sp.k, r, s), p), g, M), p);
-            a1 = ad(a1, mm(from_int(flm_weight(1, sp.k, r, s), p), g, M), p);
-            a2 = ad(a2, mm(from_int(flm_weight(2, sp.k, r, s), p), g, M), p);
+    const int j = blockIdx.x * kSeriesWarps + warp;
+    uint32_t *mine = work[warp];
+    if (j < sp.n_rects) {
+        uint32_t *src = ptilde + ((size_t)grp * sp.n_rects + j) * sp.D1 * sp.Pp + pk;
+        for (int d = lane; d < n; d += 32) {
+            uint32_t c = 0;
+            if (d < sp.D1) {
+                c = src[(size_t)d * sp.Pp];  // a signed representative: its residue stays in its place
+                c = (int)c < 0 ? c + p : c;
+                src[(size_t)d * sp.Pp] = c;
+            }
+            mine[d] = c;
         }
-        acc[0][i] = a0;
-        acc[1][i] = a1;
-        acc[2][i] = a2;
-    }
-    __syncthreads();
-    // E = exp(a): E_0 = 1, i E_i = sum_{q=1..i} q a_q E_{i-q}; warp x for series x
-    const int x = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (x < 3) {
-        if (lane == 0) E[x][0] = 1;
         __syncwarp();
-        for (int i = 1; i < n; ++i) {
-            uint32_t s = 0;
-            for (int q = 1 + lane; q <= i; q += 32) s = ad(s, mm(mm((uint32_t)q, acc[x][q], M), E[x][i - q], M), p);
-            for (int o = 16; o > 0; o >>= 1) s = ad(s, __shfl_xor_sync(0xffffffffu, s, o), p);
-            if (lane == 0) E[x][i] = mm(s, inv[i], M);
-            __syncwarp();
+        uint32_t f[kSeriesRegs], s[kSeriesRegs];
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m) {
+            const int i = lane + 32 * m;
+            uint32_t x = 0;
+            if (i < n)
+                for (int d = 0; d <= i; ++d) x = ad(x, mm(mine[d], B[i * ld + d], M), p);
+            f[m] = x;
         }
-        if (lane == 0) {
-            uint32_t *o = out + ((size_t)x * P + pi) * n;
-            if (x == 0) {
-                const bool sq = sp.lattice == CP_SQUARE;
-                for (int i = 0; i < n; ++i) {  // (1 +- t)^2 E
-                    uint32_t v = E[x][i];
-                    if (i >= 1) v = sq ? ad(v, mm(2, E[x][i - 1], M), p) : sb(v, mm(2, E[x][i - 1], M), p);
-                    if (i >= 2) v = ad(v, E[x][i - 2], p);
-                    o[i] = v;
-                }
-            } else {
-                for (int i = 0; i < n; ++i) o[i] = E[x][i];
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m)
+            if (lane + 32 * m < n) mine[lane + 32 * m] = f[m];
+        __syncwarp();
+        if (lane == 0 && f[0] != 1) atomicOr(err, 1);
+        // log f: h = f'/f with h_i = (i+1) f_{i+1} - sum_{q=1..i} f_q h_{i-q}; g_i = h_{i-1}/i
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m) {
+            const int i = lane + 32 * m;
+            s[m] = i + 1 < n ? mm(mine[i + 1], (uint32_t)(i + 1), M) : 0u;
+        }
+        for (int q = 0; q + 2 < n; ++q) {
+            const uint32_t h = lane_value(s, q);
+#pragma unroll
+            for (int m = 0; m < kSeriesRegs; ++m) {
+                const int i = lane + 32 * m;
+                if (32 * m < n && i > q && i + 1 < n) s[m] = sb(s[m], mm(mine[i - q], h, M), p);
             }
-            if (sp.add_mu && x < 2) {  // first-order: exp(f + c t^{n-1}) = exp(f) (1 + c t^{n-1}) mod t^n
-                const uint32_t mu = mu_mod(2 * sp.mmax, M);
-                const uint32_t c = x == 0 ? mu : sb(0, mm((uint32_t)sp.mmax, mu, M), p);
-                o[n - 1] = ad(o[n - 1], c, p);  // series 0 and 1 start with 1
+        }
+        uint32_t *g = logs + ((size_t)pi * sp.n_rects + j) * n;
+        if (lane == 0) g[0] = 0;
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m) {
+            const int i = lane + 32 * m;
+            if (i + 1 < n) g[i + 1] = mm(s[m], inv[i + 1], M);
+        }
+    }
+    // the prime's last block goes on
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicInc(finished + pi, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int r = tid; r < 3 * sp.n_rects; r += blockDim.x) {
+        const int x = r / sp.n_rects, k = r - x * sp.n_rects;
+        wgt[x][k] = from_int(flm_weight(x, sp.k, rects[k].x, rects[k].y), p);
+    }
+    __syncthreads();
+    for (int r = tid; r < 3 * n; r += blockDim.x) {  // work[x][q] = q a_q of series x
+        const int x = r / n, i = r - x * n;
+        uint32_t a = 0;
+        for (int k = 0; k < sp.n_rects; ++k)
+            a = ad(a, mm(wgt[x][k], __ldcg(logs + ((size_t)pi * sp.n_rects + k) * n + i), M), p);
+        work[x][i] = mm(a, (uint32_t)i, M);
+    }
+    __syncthreads();
+    const int x = warp;
+    if (x == 3 && sp.add_mu) {
+        const uint32_t mu = mu_mod(2 * sp.mmax, M, inv, tmp, lane);
+        if (lane == 0) work[3][0] = mu;
+    }
+    if (x < 3) {
+        // E = exp(a): E_0 = 1, i E_i = sum_{q=1..i} q a_q E_{i-q}
+        uint32_t s[kSeriesRegs];
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m) s[m] = lane + 32 * m < n ? mine[lane + 32 * m] : 0u;  // E_0's part of i E_i
+        if (lane == 0) s[0] = 1;  // E_0 itself
+        for (int q = 1; q < n; ++q) {
+            const uint32_t e = mm(lane_value(s, q), inv[q], M);
+#pragma unroll
+            for (int m = 0; m < kSeriesRegs; ++m) {
+                const int i = lane + 32 * m;
+                if (i == q) s[m] = e;
+                else if (32 * m < n && i > q && i < n) s[m] = ad(s[m], mm(mine[i - q], e, M), p);
             }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kSeriesRegs; ++m)
+            if (lane + 32 * m < n) mine[lane + 32 * m] = s[m];
+    }
+    __syncthreads();
+    if (x < 3) {
+        uint32_t *o = out + ((size_t)x * sp.P + pi) * n;
+        const bool sq = sp.lattice == CP_SQUARE;
+        for (int i = lane; i < n; i += 32) {
+            uint32_t v = mine[i];
+            if (x == 0) {  // (1 +- t)^2 E
+                if (i >= 1) v = sq ? ad(v, mm(2, mine[i - 1], M), p) : sb(v, mm(2, mine[i - 1], M), p);
+                if (i >= 2) v = ad(v, mine[i - 2], p);
+            }
+            // first-order: exp(f + c t^{n-1}) = exp(f) (1 + c t^{n-1}) mod t^n; series 0 and 1 start with 1
+            if (i == n - 1 && sp.add_mu && x < 2)
+                v = ad(v, x == 0 ? work[3][0] : sb(0, mm((uint32_t)sp.mmax, work[3][0], M), p), p);
+            o[i] = v;
         }
     }
 }
+
+size_t series_scratch_words(const SeriesParams &sp) { return (size_t)sp.P * sp.n_rects * sp.n + sp.P; }
 
 int launch_flm_series(uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
-                      uint32_t *out, int *err, cudaStream_t st) {
-    size_t shm = (size_t)sp.n_rects * sp.n * 4;
-    if (shm > 200 * 1024) return fail(CP_EINVAL, "too many rectangles for the series kernel");
-    if (shm > 48 * 1024)
-        CP_CUDA_TRY(cudaFuncSetAttribute(flm_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    flm_series_kernel<<<sp.P, 96, shm, st>>>(ptilde, rects, primes, sp, out, err);  // 3 warps: one per series
+                      uint32_t *scratch, uint32_t *out, int *err, cudaStream_t st) {
+    if (sp.n_rects > kMaxSeriesRects) return fail(CP_EINVAL, "too many rectangles for the series kernel");
+    const size_t shm = (size_t)sp.n * (sp.n + 1) * 4;
+    CP_CUDA_TRY(cudaFuncSetAttribute(flm_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kMaxSeries * (kMaxSeries + 1) * 4));
+    const dim3 grid((sp.n_rects + kSeriesWarps - 1) / kSeriesWarps, sp.P);
+    uint32_t *finished = scratch + (size_t)sp.P * sp.n_rects * sp.n;
+    flm_series_kernel<<<grid, 32 * kSeriesWarps, shm, st>>>(ptilde, rects, primes, sp, scratch, finished, out, err);
     CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }

@@ -7,6 +7,7 @@
 namespace cp {
 
 constexpr int kMaxSeries = 128;  // longest series (terms) handled
+constexpr int kMaxSeriesRects = 128;  // most rectangles of a band (4 per width)
 
 struct SeriesParams {
     int lattice;  // CP_SQUARE / CP_TRIANGULAR
@@ -23,7 +24,9 @@ struct SeriesParams {
 
 // ptilde [P/Pg][n_rects][D1][Pp] (signed representatives; each is replaced by its residue in [0, p)), rects (r, s),
 // primes: a prime block per group -> out [3][P][n].  err |= 1 if a P~ lacks constant term 1.
+// scratch: series_scratch_words(sp) words, the last P of them zero (left zero).
 int launch_flm_series(uint32_t *ptilde, const int2 *rects, const uint32_t *primes, const SeriesParams &sp,
-                      uint32_t *out, int *err, cudaStream_t st);
+                      uint32_t *scratch, uint32_t *out, int *err, cudaStream_t st);
+size_t series_scratch_words(const SeriesParams &sp);
 
 }  // namespace cp

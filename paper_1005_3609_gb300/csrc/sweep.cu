@@ -55,6 +55,7 @@ struct cp_sweep {
     int2 *rects_dev = nullptr;
     uint32_t *ptilde_dev = nullptr;  // [groups][n_rects][D1][Pp]
     uint32_t *series_dev = nullptr;  // [3][P][n]
+    uint32_t *logs_dev = nullptr;    // series kernel's scratch
     uint32_t *crt_dev = nullptr;     // cp_sweep_series_integers: limbs [3][n][limbs], then flags [3][n]
     size_t crt_words = 0;
     std::vector<uint32_t> primes_host;
@@ -80,6 +81,7 @@ struct cp_sweep {
         dev_free(rects_dev);
         dev_free(ptilde_dev);
         dev_free(series_dev);
+        dev_free(logs_dev);
         dev_free(crt_dev);
         dev_free(err_dev);
     }
@@ -211,6 +213,21 @@ static int build_program(cp_sweep *sw, int tile) {
     return CP_OK;
 }
 
+static SeriesParams series_params(const cp_sweep *sw) {
+    SeriesParams sp{};
+    sp.lattice = sw->lattice;
+    sp.k = sw->k;
+    sp.n = sw->n;
+    sp.D1 = sw->D1;
+    sp.P = sw->P;
+    sp.Pg = sw->Pg;
+    sp.Pp = sw->Pp;
+    sp.n_rects = (int)sw->rects.size();
+    sp.mmax = sw->k / 2;
+    sp.add_mu = (sw->lattice == CP_SQUARE && sw->k % 2 == 1) ? 1 : 0;
+    return sp;
+}
+
 // Every vector := e_0; at height 1 no other word is read (degree windows).
 static int enqueue_reset(cp_sweep *sw) {
     for (auto &st : sw->strips)
@@ -226,19 +243,8 @@ static int enqueue_program(cp_sweep *sw) {
         rc = launch_gather(sw->steps[t].data(), (int)sw->steps[t].size(), sw->step_blocks[t], sw->step_tile[t], sw->stream);
         if (rc) return rc;
     }
-    SeriesParams sp{};
-    sp.lattice = sw->lattice;
-    sp.k = sw->k;
-    sp.n = sw->n;
-    sp.D1 = sw->D1;
-    sp.P = sw->P;
-    sp.Pg = sw->Pg;
-    sp.Pp = sw->Pp;
-    sp.n_rects = (int)sw->rects.size();
-    sp.mmax = sw->k / 2;
-    sp.add_mu = (sw->lattice == CP_SQUARE && sw->k % 2 == 1) ? 1 : 0;
-    return launch_flm_series(sw->ptilde_dev, sw->rects_dev, sw->primes_dev, sp, sw->series_dev, sw->err_dev,
-                             sw->stream);
+    return launch_flm_series(sw->ptilde_dev, sw->rects_dev, sw->primes_dev, series_params(sw), sw->logs_dev,
+                             sw->series_dev, sw->err_dev, sw->stream);
 }
 
 // The primes as the strips hold them: a prime block per group.
@@ -293,6 +299,9 @@ static int sweep_build_lanes(int lattice, int k, const uint32_t *primes, int P, 
     if ((rc = dev_alloc((void **)&sw->err_dev, sizeof(int)))) return rc;
     CP_CUDA_TRY(cudaMemset(sw->err_dev, 0, sizeof(int)));
     if ((rc = build_strips(sw.get()))) return rc;
+    const size_t log_words = series_scratch_words(series_params(sw.get()));
+    if ((rc = dev_alloc((void **)&sw->logs_dev, 4 * log_words))) return rc;
+    CP_CUDA_TRY(cudaMemset(sw->logs_dev, 0, 4 * log_words));
     if ((rc = dev_alloc((void **)&sw->rects_dev, sizeof(int2) * n_rects))) return rc;
     CP_CUDA_TRY(cudaMemcpy(sw->rects_dev, sw->rects.data(), sizeof(int2) * n_rects, cudaMemcpyHostToDevice));
     if ((rc = build_program(sw.get(), tile))) return rc;
@@ -496,11 +505,9 @@ extern "C" int cp_sweep_series_integers(cp_sweep *sw, uint32_t *limbs_out, size_
         sw->crt_words = need;
     }
     uint32_t *limbs_d = sw->crt_dev, *flags_d = limbs_d + 3ull * n * limbs_per_coeff;
-    for (int x = 0; x < 3; ++x)
-        if ((rc = launch_crt(sw->series_dev + (size_t)x * P * n, sw->primes_host.data(), P, n,
-                             limbs_d + (size_t)x * n * limbs_per_coeff, limbs_per_coeff, nullptr, flags_d + (size_t)x * n,
-                             sw->stream)))
-            return rc;
+    if ((rc = launch_crt(sw->series_dev, sw->primes_host.data(), P, n, limbs_d, limbs_per_coeff, nullptr, flags_d,
+                         sw->stream, 3)))
+        return rc;
     std::vector<uint32_t> flags(3ull * n);
     CP_CUDA_TRY(cudaMemcpyAsync(limbs_out, limbs_d, 12ull * n * limbs_per_coeff, cudaMemcpyDeviceToHost, sw->stream));
     CP_CUDA_TRY(cudaMemcpyAsync(flags.data(), flags_d, 12ull * n, cudaMemcpyDeviceToHost, sw->stream));
