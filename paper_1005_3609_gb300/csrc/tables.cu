@@ -71,7 +71,6 @@ struct Term {
 };
 
 constexpr int kMaxTerms = 8;   // terms of one factor applied to one partition
-constexpr int kMaxFused = 64;  // terms of a two-site table before merging
 
 // H_{a,b} = 1 - J_{a,b} at v = -1: a term with a ~ b is killed (H s = s - s), otherwise
 // it splits into itself and the joined partition with -w.
@@ -197,33 +196,43 @@ __device__ __noinline__ int factor_terms(const OpDesc &op, const Labels &s, Term
     return n;
 }
 
-// Terms of a two-site table: the second factor applied to every term of the first.
-__device__ __noinline__ int fused_terms(const OpDesc &op, const Labels &s, Term *out) {
-    Term a[kMaxTerms];
-    const int na = factor_terms(op, s, a);
-    OpDesc ob = op;
-    ob.kind = op.kind_b;
-    ob.i = op.i_b;
-    int n = 0;
-    for (int j = 0; j < na; ++j) {
-        Term b[kMaxTerms];
-        const int nb = factor_terms(ob, a[j].s, b);
-        for (int q = 0; q < nb; ++q) {
-            out[n].s = b[q].s;
-            out[n].coef = a[j].coef * b[q].coef;
-            out[n].shift = a[j].shift + b[q].shift;
-            ++n;
-        }
+// Rank of a term's state in the output space, or ~0u with the error bit set.
+__device__ __forceinline__ uint32_t term_dst(const Labels &s, const Space &out, const RankTables &T, int *bad) {
+    if (!space_contains(s, out)) {
+        *bad |= 1;
+        return ~0u;
     }
-    return n;
+    const uint64_t r = space_rank(s, out, T);
+    if (r >= out.size) {
+        *bad |= 1;
+        return ~0u;
+    }
+    return (uint32_t)r;
+}
+
+// One packed edge into slot w of its source, if it fits (err bits below).
+__device__ __forceinline__ void put_term(const OpDesc &op, uint64_t src, uint32_t dst, int coef, int shift, int w, int K,
+                                         uint32_t *slot_dst, uint32_t *slot_edge, int *bad) {
+    const int sb = op.src_bits, cb = 30 - sb;  // coefficient bits
+    if (w >= K) {
+        *bad |= 2;
+        return;
+    }
+    if (coef < -(1 << (cb - 1)) || coef > (1 << (cb - 1)) - 1 || shift > 3) {
+        *bad |= 4;
+        slot_dst[src * K + w] = ~0u;
+        return;
+    }
+    slot_dst[src * K + w] = dst;
+    slot_edge[src * K + w] =
+        (uint32_t)src | ((uint32_t)shift << sb) | (((uint32_t)coef & ((1u << cb) - 1u)) << (sb + 2));
 }
 
 // One thread per source state.  slot_dst[src*K + t] = destination rank or ~0u,
 // slot_edge[...] = packed edge.  err bits: 1 bad rank / membership, 2 too many
 // terms, 4 coefficient out of range, 8 unrank/rank mismatch of the source.
-template <int NT>
-__global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *slot_dst, uint32_t *slot_edge,
-                                   int K, int *err) {
+__global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *slot_dst, uint32_t *slot_edge, int K,
+                                   int *err) {
     __shared__ RankTables T;
     stage_tables(T, Tg);
     uint64_t src = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,15 +241,10 @@ __global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *sl
     space_unrank(src, op.in, s, T);
     int bad = 0;
     if (!space_contains(s, op.in) || space_rank(s, op.in, T) != src) bad |= 8;
-    Term t[NT];
-    int n = op.fused ? fused_terms(op, s, t) : factor_terms(op, s, t);
-    uint32_t dst[NT];
-    for (int j = 0; j < n; ++j) {
-        if (!space_contains(t[j].s, op.out)) { bad |= 1; dst[j] = ~0u; continue; }
-        uint64_t r = space_rank(t[j].s, op.out, T);
-        if (r >= op.out.size) { bad |= 1; dst[j] = ~0u; continue; }
-        dst[j] = (uint32_t)r;
-    }
+    Term t[kMaxTerms];
+    const int n = factor_terms(op, s, t);
+    uint32_t dst[kMaxTerms];
+    for (int j = 0; j < n; ++j) dst[j] = term_dst(t[j].s, op.out, T, &bad);
     // merge equal (dst, shift)
     for (int j = 0; j < n; ++j) {
         if (t[j].coef == 0 || dst[j] == ~0u) continue;
@@ -250,19 +254,82 @@ __global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *sl
                 t[q].coef = 0;
             }
     }
-    const int sb = op.src_bits, cb = 30 - sb;  // coefficient bits
-    const int cmin = -(1 << (cb - 1)), cmax = (1 << (cb - 1)) - 1;
     int w = 0;
-    for (int j = 0; j < n; ++j) {
-        if (t[j].coef == 0 || dst[j] == ~0u) continue;
-        if (t[j].coef < cmin || t[j].coef > cmax || t[j].shift > 3) { bad |= 4; continue; }
-        if (w >= K) { bad |= 2; break; }
-        slot_dst[src * K + w] = dst[j];
-        slot_edge[src * K + w] = (uint32_t)src | ((uint32_t)t[j].shift << sb) |
-                                 (((uint32_t)t[j].coef & ((1u << cb) - 1u)) << (sb + 2));
-        ++w;
-    }
+    for (int j = 0; j < n; ++j)
+        if (t[j].coef != 0 && dst[j] != ~0u) put_term(op, src, dst[j], t[j].coef, t[j].shift, w++, K, slot_dst, slot_edge, &bad);
     for (; w < K; ++w) slot_dst[src * K + w] = ~0u;
+    if (bad) atomicOr(err, bad);
+}
+
+// A two-site table, the second factor applied to every term of the first: LANES threads
+// per source state, each for every LANES-th term of the first factor, which meet in
+// shared memory to merge equal (dst, shift).  Bound by the latency of unranking,
+// relabelling and ranking in local memory while a table has few states: one thread per
+// source took 170 us a table at width 12 (5 798 states), eight 95 us; a table that fills
+// the SMs anyway takes two (eight repeat too much of the first factor).
+template <int LANES>
+__global__ void __launch_bounds__(128)
+    build_fused_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *slot_dst, uint32_t *slot_edge, int K, int *err) {
+    constexpr int kSources = 128 / LANES, kAll = kMaxTerms * kMaxTerms;
+    __shared__ RankTables T;
+    __shared__ uint32_t s_dst[kSources][kAll + 1];
+    __shared__ int s_term[kSources][kAll + 1];  // coefficient << 4 | shift
+    stage_tables(T, Tg);
+    const int grp = threadIdx.x / LANES, lane = threadIdx.x % LANES;
+    const uint64_t src = (uint64_t)blockIdx.x * kSources + grp;
+    const bool have = src < op.in.size;
+    uint32_t *dst = s_dst[grp];
+    int *term = s_term[grp];
+    int bad = 0;
+    for (int k = lane; k < kAll; k += LANES) dst[k] = ~0u;
+    __syncwarp();
+    if (have) {
+        Labels s;
+        space_unrank(src, op.in, s, T);
+        if (lane == 0 && (!space_contains(s, op.in) || space_rank(s, op.in, T) != src)) bad |= 8;
+        Term a[kMaxTerms], t[kMaxTerms];
+        const int na = factor_terms(op, s, a);
+        OpDesc ob = op;
+        ob.kind = op.kind_b;
+        ob.i = op.i_b;
+        for (int j = lane; j < na; j += LANES) {
+            const int n = factor_terms(ob, a[j].s, t);
+            for (int q = 0; q < n; ++q) {
+                dst[j * kMaxTerms + q] = term_dst(t[q].s, op.out, T, &bad);
+                term[j * kMaxTerms + q] = ((t[q].coef * a[j].coef) << 4) | (t[q].shift + a[j].shift);
+            }
+        }
+    }
+    __syncwarp();
+    // of equal (dst, shift) the first stands for them all with the sum of their
+    // coefficients; the slots are the lanes' terms one after another, counted, then written
+    int w = 0;
+    for (int round = 0; round < 2; ++round) {
+        int c = 0;
+        for (int k = lane; k < kAll; k += LANES) {
+            const uint32_t d = dst[k];
+            if (d == ~0u) continue;
+            const int x = term[k];
+            int coef = x >> 4;
+            for (int m = k + 1; m < kAll; ++m)
+                if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef += term[m] >> 4;
+            for (int m = 0; m < k; ++m)
+                if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef = 0;
+            if (coef == 0) continue;
+            if (round) put_term(op, src, d, coef, x & 15, w + c, K, slot_dst, slot_edge, &bad);
+            ++c;
+        }
+        if (round) break;
+        w = c;
+        for (int o = 1; o < LANES; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o, LANES);
+            if (lane >= o) w += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, w, LANES - 1, LANES);
+        w -= c;
+        if (have)
+            for (int r = total + lane; r < K; r += LANES) slot_dst[src * K + r] = ~0u;
+    }
     if (bad) atomicOr(err, bad);
 }
 
@@ -368,19 +435,41 @@ __global__ void fill_kernel(const uint32_t *slot_dst, const uint32_t *slot_edge,
     }
 }
 
-// Deterministic order inside each destination: by packed value (src, then shift/coef).
+// Deterministic order inside each destination: by packed value (src, then shift/coef;
+// all different).  One warp per destination: every entry's place is the number of
+// smaller ones, up to kSortRegs entries a lane.  (An insertion sort by one thread per
+// destination took 62 us a table at width 12, for the few rows of a hundred entries.)
+constexpr int kSortRegs = 8;
 __global__ void sort_segments_kernel(const uint32_t *row_ptr, uint64_t n_dst, uint32_t *edges) {
-    uint64_t d = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t d = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t lane = threadIdx.x & 31;
     if (d >= n_dst) return;
-    uint32_t b = row_ptr[d], e = row_ptr[d + 1];
-    for (uint32_t i = b + 1; i < e; ++i) {
-        uint32_t x = edges[i];
-        uint32_t j = i;
-        while (j > b && edges[j - 1] > x) {
-            edges[j] = edges[j - 1];
-            --j;
+    const uint32_t b = row_ptr[d], n = row_ptr[d + 1] - b;
+    if (n <= 32) {
+        const uint32_t x = lane < n ? edges[b + lane] : 0xffffffffu;
+        uint32_t at = 0;
+        for (uint32_t i = 0; i < n; ++i) at += __shfl_sync(0xffffffffu, x, i) < x ? 1u : 0u;
+        if (lane < n) edges[b + at] = x;
+    } else if (n <= 32 * kSortRegs) {
+        uint32_t x[kSortRegs], at[kSortRegs] = {};
+#pragma unroll
+        for (int m = 0; m < kSortRegs; ++m) x[m] = lane + 32 * m < n ? edges[b + lane + 32 * m] : 0xffffffffu;
+        for (uint32_t i = 0; i < n; ++i) {
+            const uint32_t y = edges[b + i];
+#pragma unroll
+            for (int m = 0; m < kSortRegs; ++m) at[m] += y < x[m] ? 1u : 0u;
         }
-        edges[j] = x;
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kSortRegs; ++m)
+            if (lane + 32 * m < n) edges[b + at[m]] = x[m];
+    } else if (lane == 0) {
+        for (uint32_t i = 1; i < n; ++i) {
+            const uint32_t x = edges[b + i];
+            uint32_t j = i;
+            for (; j > 0 && edges[b + j - 1] > x; --j) edges[b + j] = edges[b + j - 1];
+            edges[b + j] = x;
+        }
     }
 }
 
@@ -571,6 +660,8 @@ __global__ void pack_units_kernel(const uint32_t *row_ptr, uint64_t n, uint32_t 
     if (!units) cnt[c] = k;
 }
 
+constexpr uint64_t kFusedManyLanes = 16384;  // two-site tables of up to so many source states take eight lanes each
+
 static uint64_t unit_runs(uint64_t n_dst) { return (n_dst + kPackRows - 1) / kPackRows; }
 
 // (in the room that build_table reserved)
@@ -627,12 +718,15 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
     if ((rc = dev_alloc((void **)&tab->row_ptr, (n_dst + 1) * 4))) return rc;
     CP_CUDA_TRY(cudaMemsetAsync(cnt, 0, (3 * n_dst + 3) * 4, st));
     const int bt = 128;
-    if (op.fused)
-        build_terms_kernel<kMaxFused><<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
-                                                                                            slot_edge, K, err);
-    else
-        build_terms_kernel<kMaxTerms><<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
-                                                                                            slot_edge, K, err);
+    if (op.fused) {
+        if (op.in.size <= kFusedManyLanes)
+            build_fused_terms_kernel<8><<<(unsigned)((op.in.size * 8 + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
+                                                                                                  slot_edge, K, err);
+        else
+            build_fused_terms_kernel<2><<<(unsigned)((op.in.size * 2 + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
+                                                                                                  slot_edge, K, err);
+    } else
+        build_terms_kernel<<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst, slot_edge, K, err);
     count_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, op.src_bits, cnt, csum, err + 2);
     max_count_kernel<<<608, 256, 0, st>>>(csum, n_dst, err + 1);
     CP_CUDA_TRY(cudaGetLastError());
@@ -659,7 +753,7 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
     tab->max_abs_coef = (uint32_t)herr[2];
     if ((rc = dev_alloc((void **)&tab->edges, (size_t)(nnz ? nnz : 1) * 4))) return rc;
     fill_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, tab->row_ptr, cursor, tab->edges);
-    sort_segments_kernel<<<(unsigned)((n_dst + 255) / 256), 256, 0, st>>>(tab->row_ptr, n_dst, tab->edges);
+    sort_segments_kernel<<<(unsigned)((n_dst + 7) / 8), 256, 0, st>>>(tab->row_ptr, n_dst, tab->edges);
     CP_CUDA_TRY(cudaGetLastError());
     return build_units(tab, sc);
 }
@@ -684,7 +778,7 @@ TableSet::~TableSet() {
 // Window words of every space of the two chains (cp_internal.h): the blocks by
 // unranking, lo by relaxing the row's tables from e_0 until a whole row changes
 // nothing (values only fall, a row per pass; a state needs about as many rows as
-// its blocks are nested, so L / 2 + 3 passes mostly do, each a no-op once
+// its blocks are nested, so L / 2 + 1 passes mostly do, each a no-op once
 // nothing changes), then the read-out's tables once.
 static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
     const cudaStream_t st = sc->st;
@@ -716,7 +810,7 @@ static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
         w = o;
     }
     constexpr int kMaxPasses = 64;
-    const int per_round = ts->L / 2 + 3;
+    const int per_round = ts->L / 2 + 1;
     if ((rc = sc->reset((kMaxPasses + 1) * sizeof(int)))) return rc;
     int *flags = sc->take<int>(kMaxPasses + 1);  // changed, one per pass; then the checks' flag
     cudaError_t e = cudaMemsetAsync(flags, 0, (kMaxPasses + 1) * sizeof(int), st);
