@@ -187,7 +187,7 @@ def table_layout(cp, args):
     if mode == 3:
         return ("two-site tables on both lattices: consecutive site factors composed in pairs (ceil(r/2) launches "
                 "per row, the intermediate vector never written); updates counted per site factor")
-    return ("rows >= 512 bytes: two-site tables, consecutive site factors composed in pairs (ceil(r/2) "
+    return ("rows >= 352 bytes: two-site tables, consecutive site factors composed in pairs (ceil(r/2) "
             "launches per row, the intermediate vector never written); otherwise one table per site factor; "
             "updates counted per site factor either way")
 

@@ -151,7 +151,8 @@ void cp_destroy(cp_strip *s);
  * of each pair is never written -- the same matrix product as the
  * factorisation of Sec. 3.2 with half the launches and vector traffic and as
  * many edge copies.  mode 1 (the default): two-site tables where a state's row,
- * (D+1) n_primes words, has at least 512 bytes (1024 from width 16 on); mode 2: for every square-lattice strip; mode 3: for every
+ * D+1 times n_primes (rounded up to a multiple of four) words, has at least 352
+ * bytes (on the square lattice from width 16 on: 1536); mode 2: for every square-lattice strip; mode 3: for every
  * strip of both lattices; mode 0: one table per factor, as in the paper.
  * Results are identical in every mode.  Returns the previous mode.  Not thread-safe
  * against concurrent strip creation.

@@ -296,7 +296,7 @@ class Strip:
 
 def set_factor_pairing(mode):
     """Layout of the tables built from now on (cp_set_factor_pairing): 0 one table per
-    site factor, 1 two-site tables for rows of at least 512 bytes (default), 2 two-site
+    site factor, 1 two-site tables for rows of at least 352 bytes (default), 2 two-site
     tables for every square strip, 3 for every strip.  Returns the previous mode."""
     return int(load().cp_set_factor_pairing(int(mode)))
 

@@ -143,11 +143,12 @@ int device_rank_tables(const RankTables **out_dev, RankTables *host_copy);
 // Build or fetch from the cache the tables of (lattice, L) on the current device
 // (chromatic polynomial: the projected factorisation of Sec. 3.2-3.3), paired
 // or not according to factor_pairing() and the row size.
-// row_bytes = bytes of one state's row, (D+1) * n_primes * 4, of the caller's vectors.
+// row_bytes = bytes of one state's row, (D+1) * padded_primes(n_primes) * 4, of the caller's vectors.
 int get_tables(int lattice, int L, size_t row_bytes, cudaStream_t stream, std::shared_ptr<TableSet> *out);
 // Library-wide choice for tables built from now on: 0 = one table per factor, 1 = two-site
-// tables for rows of at least kPairRowBytes (twice that from width kPairWide on; default), 2 = every square table, 3 = every table.
-constexpr size_t kPairRowBytes = 512;
+// tables for rows of at least kPairRowBytes (kPairWideRowBytes on the square lattice from
+// width kPairWide on; default), 2 = every square table, 3 = every table.
+constexpr size_t kPairRowBytes = 352, kPairWideRowBytes = 1536;
 constexpr int kPairWide = 16;
 int factor_pairing();
 int set_factor_pairing(int mode);

@@ -220,7 +220,7 @@ extern "C" int cp_create_strip(int lattice, int L, const uint32_t *primes, int n
     if ((rc = prepare_gather_kernels()) || (rc = crt_static_touch())) return rc;
     std::shared_ptr<TableSet> tabs;
     const long long D1 = max_degree >= 0 ? max_degree + 1 : (long long)L * max_rows;
-    if ((rc = get_tables(lattice, L, (size_t)D1 * n_primes * 4, (cudaStream_t)cuda_stream, &tabs))) return rc;
+    if ((rc = get_tables(lattice, L, (size_t)D1 * padded_primes(n_primes) * 4, (cudaStream_t)cuda_stream, &tabs))) return rc;
     return make_strip_padded(std::move(tabs), lattice, L, primes, n_primes, max_degree, max_rows, cuda_stream, out);
 }
 

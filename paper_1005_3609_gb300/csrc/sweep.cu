@@ -120,7 +120,7 @@ static int build_strips(cp_sweep *sw) {
             for (auto &rs : sw->rects)
                 if (rs.x == r) st.heights.push_back(rs.y);
             if (st.heights.empty()) continue;
-            if ((rc = get_tables(sw->lattice, r, (size_t)sw->D1 * Pg * 4, sw->stream, &st.tabs))) return rc;
+            if ((rc = get_tables(sw->lattice, r, (size_t)sw->D1 * padded_primes(Pg) * 4, sw->stream, &st.tabs))) return rc;
             const TableSet &ts = *st.tabs;
             sw->strips.push_back(st);
             SweepStrip &sp = sw->strips.back();

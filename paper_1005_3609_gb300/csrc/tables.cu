@@ -1072,11 +1072,13 @@ int get_tables(int lattice, int L, size_t row_bytes, cudaStream_t st, std::share
     // square width 16 D 63 on 16 primes 4.81 and 3.96 ms, width 14 on 4 primes 0.467 and
     // 0.327 ms, width 8 D 71 on 8 primes 62 and 35 us; triangular width 16 D 32 on 16
     // primes 1.42 and 1.36 ms, width 13 D 181 on 4 primes 0.274 and 0.247 ms, width 9
-    // D 80 on 8 primes 77 and 45 us.  Not on wide strips of short rows, where launches
-    // are long and there is little to reduce: square width 17 D 40 on 5 primes, four
-    // rows and the read-out, 6.76 and 7.08 ms.
+    // D 80 on 8 primes 77 and 45 us; and half the tables to build: a first square 11 x 10
+    // solve with D 30 on 4 primes (496-byte rows) 5.5 and 3.9 ms.  Not on wide square
+    // strips of short rows, where launches are long and there is little to reduce: square
+    // width 17 D 40 on 5 primes, four rows and the read-out, 6.76 and 7.08 ms.
+    const bool wide_short = lattice == CP_SQUARE && L >= kPairWide && row_bytes < kPairWideRowBytes;
     const int paired = g_pairing == 3 || (lattice == CP_SQUARE && g_pairing == 2) ||
-                       (g_pairing == 1 && row_bytes >= (L < kPairWide ? kPairRowBytes : 2 * kPairRowBytes));
+                       (g_pairing == 1 && row_bytes >= kPairRowBytes && !wide_short);
     auto key = std::make_tuple(lattice, L, paired);
     auto it = g_cache[dev].find(key);
     if (it != g_cache[dev].end()) {
