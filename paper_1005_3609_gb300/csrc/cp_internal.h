@@ -226,8 +226,8 @@ inline int padded_primes(int P) { return (P + 3) & ~3; }
 // accepted as cp_tm.h lists them and choose nothing.  A batch with rows that are
 // not 16-byte chunked, large coefficients or small primes uses the register kernel.
 constexpr int kTileChunk = 32;
-constexpr int kChunkWarps = 4;         // warps of a block of the chunk kernel
-constexpr int kChunkBlocksPerSM = 7;   // its launch bound
+constexpr int kChunkWarps = 2;         // warps of a block of the chunk kernel
+constexpr int kChunkBlocksPerSM = 14;   // its launch bound
 constexpr int kChunkSteps = 4;         // 32-chunk steps of a row held in registers
 // The encodings cp_strip_set_tile and cp_sweep_create accept (besides 0).
 bool tile_valid(int tile);

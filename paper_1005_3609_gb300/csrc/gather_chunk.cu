@@ -24,10 +24,15 @@
 // edges of a two-site table): 0.66 instructions per scheduler and cycle, 66% of the
 // shared-memory data path, DRAM at a quarter of its rate, 0.107 ms; the
 // producer/consumer kernel on whole rows that this one replaces took 0.155 ms.  One
-// row of the width-16 strip 7.73 -> 3.94 ms, triangular (D = 32) 5.32 -> 1.42 ms.
-// Seven blocks per SM (72 registers) beat six (4.31 ms) and five; two edges in flight
-// beat four (4.22 ms at six blocks); four steps beat six (4.26 ms) and eight (4.87 ms),
-// which hold wider rows in one pass but leave fewer warps.
+// row of the width-16 strip 7.73 -> 3.94 ms, triangular (D = 32) 5.32 -> 1.42 ms; with
+// the constants of a row's primes loaded once per row, the lane's prime group computed
+// once and an edge's first word kept from its copy, 3.73 and 1.28 ms; with two-warp
+// instead of four-warp blocks 3.67 and 1.25 ms (one-warp blocks 3.72, 1.30).
+// 28 warps per SM (72 registers) beat 24 (4.31 before the last two changes) and 20, and
+// 32, which spill (4.02 after them); two edges in flight beat four (4.22 at 24 warps);
+// four steps beat six (4.26) and eight (4.87), which hold wider rows in one pass but
+// leave fewer warps.  Bulk copies with an mbarrier per slot (5.1) and loads straight to
+// registers (5.8) halve the shared-memory traffic but wait longer.
 #include <cuda_runtime.h>
 
 #include <string>
@@ -146,6 +151,8 @@ struct Warp {
     uint32_t n;            // listed edges
     uint32_t nch, nk;      // chunks and steps of the current row segment
     uint4 *out;
+    uint32_t xa, xb;       // first words of the next two edges to add
+    uint32_t g0;           // lane % cpd
     Acc2 acc[kSteps][4];
 
     __device__ __forceinline__ Warp(const GatherTask &t_, uint4 *list_) : t(t_), list(list_) {}
@@ -164,11 +171,15 @@ struct Warp {
     // Reduce and store the current row segment.
     __device__ __forceinline__ void flush() {
         const uint4 *consts = reinterpret_cast<const uint4 *>(t.primes);
-        uint32_t g = lane % t.cpd;  // the primes of the lane's chunk
+        uint4 p = make_uint4(0, 0, 0, 0), m = p;
+        uint32_t g = g0;  // the primes of the lane's chunk
 #pragma unroll
         for (int k = 0; k < kSteps; ++k) {
             if (k >= (int)nk) break;
-            const uint4 p = __ldg(consts + g), m = __ldg(consts + CP_MAX_PRIMES / 4 + g);
+            if (k == 0 || t.r32) {
+                p = __ldg(consts + g);
+                m = __ldg(consts + CP_MAX_PRIMES / 4 + g);
+            }
             const uint4 v = make_uint4(fast_reduce(acc[k][0], p.x, m.x), fast_reduce(acc[k][1], p.y, m.y),
                                        fast_reduce(acc[k][2], p.z, m.z), fast_reduce(acc[k][3], p.w, m.w));
             stcs128_if(out + 32 * k, v, lane + 32 * k < nch ? 1u : 0u);
@@ -185,11 +196,13 @@ struct Warp {
         cp16_below(dst + 512u * k, ptr64(d.z, d.w) + lane + 32 * k, lane - (d.x & 0xffu) + 32u * k, d.y & 0xffffu);
     }
     // Any listed edge (an empty group past the list's end).
-    __device__ __forceinline__ void copy_any(uint32_t i) const {
+    __device__ __forceinline__ void copy_any(uint32_t i) {
+        xa = xb;
         if (i < n) {
             uint4 d;
             uint32_t dst;
             copy_begin(i, d, dst);
+            xb = d.x;
             const uint32_t steps = d.y >> 16;
 #pragma unroll
             for (int k = 0; k < kSteps; ++k) {
@@ -201,10 +214,12 @@ struct Warp {
     }
     // One of the current row, of NK steps.
     template <int NK>
-    __device__ __forceinline__ void copy_row(uint32_t i) const {
+    __device__ __forceinline__ void copy_row(uint32_t i) {
         uint4 d;
         uint32_t dst;
         copy_begin(i, d, dst);
+        xa = xb;
+        xb = d.x;
 #pragma unroll
         for (int k = 0; k < NK; ++k) copy_step(d, dst, k);
         cp_commit();
@@ -212,7 +227,7 @@ struct Warp {
     // Add listed edge i to the current row's sums.
     template <int NK>
     __device__ __forceinline__ void add_edge(uint32_t i) {
-        const uint32_t x = list[i].x, slot = slots + (i & (kDepth - 1)) * kSlotBytes;
+        const uint32_t x = xa, slot = slots + (i & (kDepth - 1)) * kSlotBytes;
         const int c = (int)x >> 24;
         cp_wait<kDepth - 1>();
 #pragma unroll
@@ -343,6 +358,7 @@ __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     const GatherTask &t = pack.t[find_task(pack, n_tasks, id)];
     Warp w(t, lists[warp]);
     w.lane = lane;
+    w.g0 = lane % t.cpd;
     w.slots = smem_addr(slots) + warp * kDepth * kSlotBytes + lane * 16u;
     w.unit(__ldg(t.units + (id - t.block_begin)), t.v_in + dv, t.v_out + dv, first || t.first ? 0 : t.cap);
 }
