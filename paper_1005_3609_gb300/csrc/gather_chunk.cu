@@ -36,6 +36,7 @@
 #include <cuda_runtime.h>
 
 #include <string>
+#include <type_traits>
 
 #include "cp_internal.h"
 #include "modred.cuh"
@@ -44,7 +45,6 @@ namespace cp {
 
 constexpr int kWarps = kChunkWarps;                      // warps per block
 constexpr int kSteps = kChunkSteps;                      // 32-chunk steps of a row held in registers
-constexpr uint32_t kDepth = 2;                         // edges whose copies are in flight per warp (a power of two)
 constexpr uint32_t kSlotBytes = kSteps * 512u;         // one edge's source words
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -144,6 +144,8 @@ __device__ __forceinline__ const uint4 *ptr64(uint32_t lo, uint32_t hi) {
     return reinterpret_cast<const uint4 *>(((uint64_t)hi << 32) | lo);
 }
 
+// kDepth: edges whose copies are in flight (a power of two).
+template <uint32_t kDepth>
 struct Warp {
     const GatherTask &t;
     uint4 *list;
@@ -227,7 +229,7 @@ struct Warp {
     // Add listed edge i to the current row's sums.
     template <int NK>
     __device__ __forceinline__ void add_edge(uint32_t i) {
-        const uint32_t x = xa, slot = slots + (i & (kDepth - 1)) * kSlotBytes;
+        const uint32_t x = kDepth == 2 ? xa : list[i].x, slot = slots + (i & (kDepth - 1)) * kSlotBytes;
         const int c = (int)x >> 24;
         cp_wait<kDepth - 1>();
 #pragma unroll
@@ -346,7 +348,7 @@ struct Warp {
 // dv is added to the tasks' vertex counts; first: as if every task's `first` were set.
 // Launches overlap: a launch's blocks may start while the one before it drains, load
 // their unit's tables (which no launch writes) and only then wait for it.
-template <int N>
+template <int N, uint32_t kDepth>
 __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, int dv, int first) {
     extern __shared__ __align__(128) uint8_t slots[];  // per warp: kDepth slots of kSegChunks chunks
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (id >= n_units) return;
     const GatherTask &t = pack.t[find_task(pack, n_tasks, id)];
-    Warp w(t, lists[warp]);
+    Warp<kDepth> w(t, lists[warp]);
     w.lane = lane;
     w.g0 = lane % t.cpd;
     w.slots = smem_addr(slots) + warp * kDepth * kSlotBytes + lane * 16u;
@@ -381,6 +383,14 @@ int debug_wait_timeout(long long cycles, cudaStream_t st) {
     return check_device_error(st);
 }
 
+// Launches of few units keep four edges in flight instead of two: there the chain of one
+// warp's edges is what they last, not the SMs' throughput.  Four take 16 KB a block, 12
+// blocks of two warps on each of the 152 SMs; up to two waves of those gain (k = 17 sweep
+// 457 -> 420 us, triangular 12x12 on one prime 793 -> 714, square 12x13 on 8 primes 1227 ->
+// 1180), a third, just begun, loses (Potts 10x10, 8 000 units: 1212 -> 1286).  Eight in
+// flight gain no more (429 us).
+constexpr uint32_t kFewUnits = 2 * 24 * 152;
+
 int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, cudaStream_t st, int dv, bool first) {
     return for_packs(tasks, n_tasks, n_units, [&](const auto &pack, int n, uint32_t units) -> int {
         constexpr int N = sizeof(pack.t) / sizeof(GatherTask);
@@ -391,11 +401,14 @@ int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, 
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((units + kWarps - 1) / kWarps);
         cfg.blockDim = dim3(32 * kWarps);
-        cfg.dynamicSmemBytes = kWarps * kDepth * kSlotBytes;
         cfg.stream = st;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        CP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N>, pack, n, units, dv, first ? 1 : 0));
+        auto go = [&](auto depth) -> cudaError_t {
+            cfg.dynamicSmemBytes = kWarps * decltype(depth)::value * kSlotBytes;
+            return cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N, decltype(depth)::value>, pack, n, units, dv, first ? 1 : 0);
+        };
+        CP_CUDA_TRY(units <= kFewUnits ? go(std::integral_constant<uint32_t, 4>()) : go(std::integral_constant<uint32_t, 2>()));
         return CP_OK;
     });
 }
