@@ -294,7 +294,14 @@ inline int for_packs(const GatherTask *tasks, int n_tasks, uint32_t total_blocks
 }
 // Set the kernels' shared-memory attributes (call outside stream capture).
 int prepare_gather_kernels();
-// Device error word set by bounded waits in kernels; check_device_error syncs
+// Error words that kernels set: pinned host memory mapped on the device.
+struct ErrorWord {
+    int *host = nullptr, *dev = nullptr;
+};
+int error_word_alloc(ErrorWord *w);
+void error_word_free(ErrorWord *w);
+int error_word_take(const ErrorWord &w);  // its value, cleared (after a synchronisation)
+// The device's word, set by bounded waits in kernels; check_device_error syncs
 // `st`, returns CP_ETIMEOUT (and clears the word) if it was set.
 int *device_error_flag();
 int check_device_error(cudaStream_t st);

@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <mutex>
 #include <string>
 
 #include "cp_internal.h"
@@ -260,31 +261,48 @@ int prepare_gather_kernels() {
     return device_error_flag() ? CP_OK : CP_ECUDA;
 }
 
-int *device_error_flag() {
-    static int *flags[64] = {};
+// An error word in pinned host memory, mapped on the device: the host reads it after a
+// synchronisation without a copy of its own (a blocking 4-byte copy took about 8 us of
+// every read-out and of every server step).
+int error_word_alloc(ErrorWord *w) {
+    CP_CUDA_TRY(cudaHostAlloc((void **)&w->host, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable));
+    *w->host = 0;
+    const cudaError_t e = cudaHostGetDevicePointer((void **)&w->dev, w->host, 0);
+    if (e != cudaSuccess) {
+        error_word_free(w);
+        return fail(CP_ECUDA, std::string("error word: ") + cudaGetErrorString(e));
+    }
+    return CP_OK;
+}
+
+void error_word_free(ErrorWord *w) {
+    if (w->host) cudaFreeHost(w->host);
+    *w = ErrorWord{};
+}
+
+int error_word_take(const ErrorWord &w) { return __atomic_exchange_n(w.host, 0, __ATOMIC_ACQ_REL); }
+
+static std::mutex g_err_mu;
+static ErrorWord *device_error_word() {
+    static ErrorWord words[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!flags[dev]) {
-        int *p = nullptr;
-        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) return nullptr;
-        cudaMemset(p, 0, sizeof(int));
-        cudaDeviceSynchronize();
-        flags[dev] = p;
-    }
-    return flags[dev];
+    std::lock_guard<std::mutex> lk(g_err_mu);
+    if (!words[dev].host && error_word_alloc(&words[dev])) return nullptr;
+    return &words[dev];
+}
+
+int *device_error_flag() {
+    ErrorWord *w = device_error_word();
+    return w ? w->dev : nullptr;
 }
 
 int check_device_error(cudaStream_t st) {
-    int *f = device_error_flag();
-    if (!f) return fail(CP_ECUDA, "device error word unavailable");
+    ErrorWord *w = device_error_word();
+    if (!w) return fail(CP_ECUDA, "device error word unavailable");
     CP_CUDA_TRY(cudaStreamSynchronize(st));
-    int h = 0;
-    CP_CUDA_TRY(cudaMemcpy(&h, f, sizeof(int), cudaMemcpyDeviceToHost));
-    if (h) {
-        CP_CUDA_TRY(cudaMemset(f, 0, sizeof(int)));
-        return fail(CP_ETIMEOUT, "a bounded wait in the chunk gather kernel ran out, or a block refused its "
-                                 "configuration (flags " + std::to_string(h) + ")");
-    }
+    const int h = error_word_take(*w);
+    if (h) return fail(CP_ETIMEOUT, "a bounded wait on the device ran out (flags " + std::to_string(h) + ")");
     return CP_OK;
 }
 

@@ -374,7 +374,7 @@ __global__ void wait_timeout_kernel(long long cycles, int *err) {
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) mbar_init(smem_addr(&bar), 1);
     __syncthreads();
-    if (threadIdx.x == 0 && !mbar_wait(smem_addr(&bar), 0, clock64() + cycles)) atomicOr(err, 1 << 16);
+    if (threadIdx.x == 0 && !mbar_wait(smem_addr(&bar), 0, clock64() + cycles)) atomicOr_system(err, 1 << 16);
 }
 
 int debug_wait_timeout(long long cycles, cudaStream_t st) {

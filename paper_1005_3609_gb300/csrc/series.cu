@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(32 * kSeriesWarps)
         for (int m = 0; m < kSeriesRegs; ++m)
             if (lane + 32 * m < n) mine[lane + 32 * m] = f[m];
         __syncwarp();
-        if (lane == 0 && f[0] != 1) atomicOr(err, 1);
+        if (lane == 0 && f[0] != 1) atomicOr_system(err, 1);
         // log f: h = f'/f with h_i = (i+1) f_{i+1} - sum_{q=1..i} f_q h_{i-q}; g_i = h_{i-1}/i
 #pragma unroll
         for (int m = 0; m < kSeriesRegs; ++m) {

@@ -83,6 +83,7 @@ struct cp_strip {
     cudaStream_t stream = nullptr;
     std::shared_ptr<TableSet> tabs;
     uint32_t *primes_dev = nullptr;  // prime block of Pp lanes
+    std::vector<uint32_t> primes;
     uint32_t *vec[2] = {nullptr, nullptr};
     int cur = 0;
     uint32_t *scratch[2] = {nullptr, nullptr};
@@ -149,6 +150,7 @@ static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const 
     s->Pp = Pp;
     s->D1 = (int)D + 1;
     s->max_rows = max_rows;
+    s->primes.assign(primes, primes + n_primes);
     s->stream = (cudaStream_t)cuda_stream;
     s->tabs = std::move(tabs);
     const TableSet &ts = *s->tabs;
@@ -310,20 +312,17 @@ extern "C" int cp_read_integers(cp_strip *s, uint32_t *limbs_out, size_t limbs_l
     uint32_t *limbs_d = s->crt_dev, *flags_d = limbs_d + (size_t)D1 * limbs_per_coeff, *bound_d = flags_d + D1;
     if ((rc = readout(s))) return rc;
     CP_CUDA_TRY(cudaMemcpyAsync(bound_d, bits.data(), 4ull * D1, cudaMemcpyHostToDevice, s->stream));
-    std::vector<uint32_t> primes(s->P);
-    CP_CUDA_TRY(cudaMemcpyAsync(primes.data(), s->primes_dev, 4ull * s->P, cudaMemcpyDeviceToHost, s->stream));
-    CP_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    if ((rc = launch_crt(s->row_out, primes.data(), s->P, D1, limbs_d, limbs_per_coeff, bound ? bound_d : nullptr,
+    if ((rc = launch_crt(s->row_out, s->primes.data(), s->P, D1, limbs_d, limbs_per_coeff, bound ? bound_d : nullptr,
                          flags_d, s->stream)))
         return rc;
-    std::vector<uint32_t> flags(D1);
-    CP_CUDA_TRY(cudaMemcpyAsync(limbs_out, limbs_d, 4ull * D1 * limbs_per_coeff, cudaMemcpyDeviceToHost, s->stream));
-    CP_CUDA_TRY(cudaMemcpyAsync(flags.data(), flags_d, 4ull * D1, cudaMemcpyDeviceToHost, s->stream));
+    std::vector<uint32_t> both((size_t)D1 * (limbs_per_coeff + 1));  // limbs, then flags: one copy
+    CP_CUDA_TRY(cudaMemcpyAsync(both.data(), limbs_d, both.size() * 4, cudaMemcpyDeviceToHost, s->stream));
     if ((rc = check_device_error(s->stream))) return rc;
-    if (flags_out)
-        for (int j = 0; j < D1; ++j) flags_out[j] = flags[j];
+    const uint32_t *flags = both.data() + (size_t)D1 * limbs_per_coeff;
+    std::copy((const uint32_t *)both.data(), flags, limbs_out);
+    if (flags_out) std::copy(flags, flags + D1, flags_out);
     if (height_out) *height_out = s->height;
-    return crt_outcome(flags.data(), D1);
+    return crt_outcome(flags, D1);
 }
 
 extern "C" int cp_strip_info(const cp_strip *s, uint64_t n_states[2], int *degree, int *height) {

@@ -59,7 +59,7 @@ struct cp_sweep {
     uint32_t *crt_dev = nullptr;     // cp_sweep_series_integers: limbs [3][n][limbs], then flags [3][n]
     size_t crt_words = 0;
     std::vector<uint32_t> primes_host;
-    int *err_dev = nullptr;
+    ErrorWord err;
     std::vector<std::vector<GatherTask>> steps;  // tasks of each batched launch
     std::vector<uint32_t> step_blocks;
     std::vector<int> step_tile;
@@ -83,7 +83,7 @@ struct cp_sweep {
         dev_free(series_dev);
         dev_free(logs_dev);
         dev_free(crt_dev);
-        dev_free(err_dev);
+        error_word_free(&err);
     }
 };
 
@@ -244,7 +244,7 @@ static int enqueue_program(cp_sweep *sw) {
         if (rc) return rc;
     }
     return launch_flm_series(sw->ptilde_dev, sw->rects_dev, sw->primes_dev, series_params(sw), sw->logs_dev,
-                             sw->series_dev, sw->err_dev, sw->stream);
+                             sw->series_dev, sw->err.dev, sw->stream);
 }
 
 // The primes as the strips hold them: a prime block per group.
@@ -296,8 +296,7 @@ static int sweep_build_lanes(int lattice, int k, const uint32_t *primes, int P, 
             if (r + s >= k - 3) ++n_rects;
     if ((rc = dev_alloc((void **)&sw->ptilde_dev, 4ull * n_rects * sw->D1 * Pp * groups))) return rc;
     if ((rc = dev_alloc((void **)&sw->series_dev, 4ull * 3 * P * sw->n))) return rc;
-    if ((rc = dev_alloc((void **)&sw->err_dev, sizeof(int)))) return rc;
-    CP_CUDA_TRY(cudaMemset(sw->err_dev, 0, sizeof(int)));
+    if ((rc = error_word_alloc(&sw->err))) return rc;
     if ((rc = build_strips(sw.get()))) return rc;
     const size_t log_words = series_scratch_words(series_params(sw.get()));
     if ((rc = dev_alloc((void **)&sw->logs_dev, 4 * log_words))) return rc;
@@ -395,12 +394,9 @@ extern "C" int cp_sweep_run(cp_sweep *sw) {
 
 extern "C" int cp_sweep_sync(cp_sweep *sw) {
     if (!sw) return fail(CP_EINVAL, "sweep is NULL");
-    CP_CUDA_TRY(cudaStreamSynchronize(sw->stream));
     int rc = check_device_error(sw->stream);
     if (rc) return rc;
-    int herr = 0;
-    CP_CUDA_TRY(cudaMemcpy(&herr, sw->err_dev, sizeof(int), cudaMemcpyDeviceToHost));
-    if (herr) return fail(CP_ESTATE, "a rectangle's P~ lacks constant term 1");
+    if (*(volatile int *)sw->err.host) return fail(CP_ESTATE, "a rectangle's P~ lacks constant term 1");
     return CP_OK;
 }
 
@@ -508,13 +504,13 @@ extern "C" int cp_sweep_series_integers(cp_sweep *sw, uint32_t *limbs_out, size_
     if ((rc = launch_crt(sw->series_dev, sw->primes_host.data(), P, n, limbs_d, limbs_per_coeff, nullptr, flags_d,
                          sw->stream, 3)))
         return rc;
-    std::vector<uint32_t> flags(3ull * n);
-    CP_CUDA_TRY(cudaMemcpyAsync(limbs_out, limbs_d, 12ull * n * limbs_per_coeff, cudaMemcpyDeviceToHost, sw->stream));
-    CP_CUDA_TRY(cudaMemcpyAsync(flags.data(), flags_d, 12ull * n, cudaMemcpyDeviceToHost, sw->stream));
+    std::vector<uint32_t> both(need);  // limbs, then flags: one copy
+    CP_CUDA_TRY(cudaMemcpyAsync(both.data(), limbs_d, need * 4, cudaMemcpyDeviceToHost, sw->stream));
     if ((rc = cp_sweep_sync(sw))) return rc;
-    if (flags_out)
-        for (size_t j = 0; j < flags.size(); ++j) flags_out[j] = flags[j];
-    return crt_outcome(flags.data(), 3 * n);
+    const uint32_t *flags = both.data() + 3ull * n * limbs_per_coeff;
+    std::copy((const uint32_t *)both.data(), flags, limbs_out);
+    if (flags_out) std::copy(flags, flags + 3ull * n, flags_out);
+    return crt_outcome(flags, 3 * n);
 }
 
 // The same program without the graph, with an event pair around every batched
