@@ -302,6 +302,13 @@ int cp_sweep_info(const cp_sweep *sw, int *n_rects, int *n_terms, int *tile, int
  * intermediate vectors of two-site tables included, plus the tables' CSR). */
 int cp_sweep_work(const cp_sweep *sw, uint64_t work[3]);
 
+/* Bytes one run has to move: of every table's input and output vector the words
+ * that can be non-zero (a state's coefficients start at the lowest power of w that
+ * reaches it and end at vertices - blocks), once each, and the tables.  For roofline
+ * figures: the gathers touch no other words, so the figures of cp_sweep_work, which
+ * count whole vectors, exceed what is moved.  Synchronises. */
+int cp_sweep_window_bytes(cp_sweep *sw, uint64_t *bytes);
+
 /* The rectangles, rs_host[2j] = r, rs_host[2j+1] = s. */
 int cp_sweep_rects(const cp_sweep *sw, int *rs_host, int max_rects);
 

@@ -54,6 +54,7 @@ SIGNATURES = {
     "cp_sweep_info": (ctypes.c_int, [vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                      ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int), u64p, u64p,
                                      ctypes.POINTER(ctypes.c_int)]),
+    "cp_sweep_window_bytes": (ctypes.c_int, [vp, u64p]),
     "cp_sweep_rects": (ctypes.c_int, [vp, ctypes.POINTER(ctypes.c_int), ctypes.c_int]),
     "cp_sweep_read_ptilde": (ctypes.c_int, [vp, u32p, ctypes.c_size_t]),
     "cp_sweep_read_series": (ctypes.c_int, [vp, u32p, ctypes.c_size_t]),
@@ -389,6 +390,12 @@ class Sweep:
 
     def sync(self):
         check("cp_sweep_sync", load().cp_sweep_sync(self._h))
+
+    def window_bytes(self):
+        """Bytes one run has to move (cp_sweep_window_bytes)."""
+        b = ctypes.c_uint64()
+        check("cp_sweep_window_bytes", load().cp_sweep_window_bytes(self._h, ctypes.byref(b)))
+        return int(b.value)
 
     def read_ptilde(self):
         """{(r, s): uint32 [n_primes][n_terms]}"""

@@ -311,6 +311,10 @@ int check_device_error(cudaStream_t st);
 int launch_transpose_row(const uint32_t *row, uint32_t *out, const uint32_t *primes_dev, int D1, int P, int Pp,
                          cudaStream_t st);
 
+// Adds to *sum_dev the degrees in the windows of n states of a vector of v vertices
+// capped at degree cap (first: of e_0 at height 1).
+int add_window_degrees(const uint16_t *win, uint64_t n, int v, int cap, unsigned long long *sum_dev, cudaStream_t st);
+
 // ------------------------------------------------------------------ CRT (crt.cu)
 // Device CRT of residues [P][n_coeffs] into limbs [n_coeffs][limbs]; with
 // flags_dev, per-coefficient flags (bit 0: bound_dev[j] + 2 > bit length of the

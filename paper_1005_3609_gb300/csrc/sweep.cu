@@ -62,6 +62,12 @@ struct cp_sweep {
     ErrorWord err;
     std::vector<std::vector<GatherTask>> steps;  // tasks of each batched launch
     std::vector<uint32_t> step_blocks;
+    struct Applied {
+        const SiteTable *tab;
+        int v_in;
+        bool first, final;
+    };
+    std::vector<Applied> applied;  // every table application of a run
     std::vector<int> step_tile;
     uint64_t updates = 0, bytes = 0, site_bytes = 0;
     cudaGraph_t graph = nullptr;
@@ -154,6 +160,7 @@ static int build_program(cp_sweep *sw, int tile) {
     const uint32_t pmin = *std::min_element(sw->primes_host.begin(), sw->primes_host.end());
     auto &steps = sw->steps;
     steps.clear();
+    sw->applied.clear();
     auto at = [&](size_t t) -> std::vector<GatherTask> & {
         if (steps.size() <= t) steps.resize(t + 1);
         return steps[t];
@@ -171,6 +178,7 @@ static int build_program(cp_sweep *sw, int tile) {
                 const size_t t = (size_t)row * nf + i;
                 append_gather_task(&at(t), ts.row[i], st.vec[t & 1], st.vec[(t & 1) ^ 1], pr, sw->D1, sw->Pp, v, pmin);
                 if (t == 0) at(t).back().first = 1;
+                sw->applied.push_back({&ts.row[i], v, t == 0, false});
                 v += ts.row[i].sites;
                 count_work(sw, ts.row[i], Pg);
             }
@@ -186,6 +194,7 @@ static int build_program(cp_sweep *sw, int tile) {
                 uint32_t *dst = final ? slot : st.scratch[sc];
                 append_gather_task(&at(t0 + i), ts.last[i], src, dst, pr, sw->D1, sw->Pp, v, pmin, final);
                 if (t0 + i == 0) at(0).back().first = 1;  // read out at height 1
+                sw->applied.push_back({&ts.last[i], v, t0 + i == 0, final});
                 v += ts.last[i].sites;
                 count_work(sw, ts.last[i], Pg);
                 src = dst;
@@ -405,6 +414,31 @@ extern "C" int cp_sweep_work(const cp_sweep *sw, uint64_t work[3]) {
     work[0] = sw->updates;
     work[1] = sw->bytes;
     work[2] = sw->site_bytes;
+    return CP_OK;
+}
+
+extern "C" int cp_sweep_window_bytes(cp_sweep *sw, uint64_t *bytes) {
+    if (!sw || !bytes) return fail(CP_EINVAL, "NULL argument");
+    unsigned long long *sum = nullptr, degrees = 0;
+    int rc = dev_alloc((void **)&sum, 8);
+    if (rc) return rc;
+    uint64_t tables = 0;
+    cudaError_t e = cudaMemsetAsync(sum, 0, 8, sw->stream);
+    const int cap = sw->D1 - 1;
+    for (auto &a : sw->applied) {
+        if (rc || e != cudaSuccess) break;
+        rc = add_window_degrees(a.tab->win_in, a.tab->n_src, a.v_in, a.first ? 0 : cap, sum, sw->stream);
+        if (!rc)
+            rc = add_window_degrees(a.tab->win_out, a.tab->n_dst, a.final ? kFinalVertices : a.v_in + a.tab->sites, cap, sum,
+                                    sw->stream);
+        tables += 8 * a.tab->nnz + 2 * a.tab->n_dst + 16ull * a.tab->n_units;
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&degrees, sum, 8, cudaMemcpyDeviceToHost, sw->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(sw->stream);
+    dev_free(sum);
+    if (rc) return rc;
+    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("window bytes: ") + cudaGetErrorString(e));
+    *bytes = 4ull * sw->Pp * degrees + tables;
     return CP_OK;
 }
 

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(128)
     const bool have = src < op.in.size;
     uint32_t *dst = s_dst[grp];
     int *term = s_term[grp];
-    int bad = 0;
+    int bad = 0, all = 0;  // all: end of the slots in use
     for (int k = lane; k < kAll; k += LANES) dst[k] = ~0u;
     __syncwarp();
     if (have) {
@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(128)
         if (lane == 0 && (!space_contains(s, op.in) || space_rank(s, op.in, T) != src)) bad |= 8;
         Term a[kMaxTerms], t[kMaxTerms];
         const int na = factor_terms(op, s, a);
+        all = na * kMaxTerms;
         OpDesc ob = op;
         ob.kind = op.kind_b;
         ob.i = op.i_b;
@@ -304,18 +305,24 @@ __global__ void __launch_bounds__(128)
     // of equal (dst, shift) the first stands for them all with the sum of their
     // coefficients; the slots are the lanes' terms one after another, counted, then written
     int w = 0;
+    uint32_t keep = ~0u;  // of this lane's slots, one bit each
+    static_assert(kAll / LANES <= 32, "a bit per slot of a lane");
     for (int round = 0; round < 2; ++round) {
         int c = 0;
-        for (int k = lane; k < kAll; k += LANES) {
+        for (int k = lane; k < all; k += LANES) {
             const uint32_t d = dst[k];
-            if (d == ~0u) continue;
+            if (d == ~0u || !(keep >> (k / LANES) & 1u)) continue;
             const int x = term[k];
             int coef = x >> 4;
-            for (int m = k + 1; m < kAll; ++m)
+            for (int m = k + 1; m < all; ++m)
                 if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef += term[m] >> 4;
-            for (int m = 0; m < k; ++m)
-                if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef = 0;
-            if (coef == 0) continue;
+            if (round == 0)
+                for (int m = 0; m < k; ++m)
+                    if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef = 0;
+            if (coef == 0) {
+                keep &= ~(1u << (k / LANES));
+                continue;
+            }
             if (round) put_term(op, src, d, coef, x & 15, w + c, K, slot_dst, slot_edge, &bad);
             ++c;
         }
@@ -353,18 +360,14 @@ __global__ void count_kernel(const uint32_t *slot_dst, const uint32_t *slot_edge
     if ((threadIdx.x & 31) == 0) atomicMax(max_coef, (int)m);
 }
 
-// Largest entry of cnt (warp maximum, one atomic per warp).
-__global__ void max_count_kernel(const uint32_t *cnt, uint64_t n, int *out) {
-    uint32_t m = 0;
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x)
-        m = max(m, cnt[k]);
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, (int)m);
-}
-
 constexpr int kScanThreads = 1024;
 
-// Exclusive scan, three passes: per-block sums, scan of the block sums, per-block scan + offset.
+// Exclusive scan, three launches: per-block sums, scan of the block sums, per-block
+// scan + offset.  Up to kScanAlone blocks the last launch does it alone, each block
+// adding up the words before its own: at most 31 loads a thread, all in flight at
+// once, against two launches more (a table of width 12 has 16 blocks; a launch there
+// is 2.3 us, and two scans a table make them a tenth of its build).
+constexpr uint64_t kScanAlone = 32;
 __device__ __forceinline__ uint32_t block_inclusive_scan(uint32_t v, uint32_t *warp_sums) {
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -414,14 +417,34 @@ __global__ void scan_sums_serial(uint32_t *sums, uint32_t n_blocks) {
     }
 }
 
-__global__ void scan_finish(const uint32_t *in, uint64_t n, const uint32_t *block_off, uint32_t *out) {
-    __shared__ uint32_t ws[32];
-    uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t v = k < n ? in[k] : 0;
-    uint32_t inc = block_inclusive_scan(v, ws);
-    uint32_t exc = block_off[blockIdx.x] + inc - v;
+// With `of`, also the largest of of[0..n) into *largest (a warp maximum, one atomic
+// per warp; on its own that was one more launch of 4.6 us a table).
+__global__ void scan_finish(const uint32_t *in, uint64_t n, const uint32_t *block_off, uint32_t *out, const uint32_t *of,
+                            int *largest) {
+    __shared__ uint32_t ws[32], before;
+    const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t off = 0;
+    if (block_off) {
+        off = block_off[blockIdx.x];
+    } else {
+        if (threadIdx.x == 0) before = 0;
+        __syncthreads();
+#pragma unroll 8
+        for (uint32_t b = 0; b < blockIdx.x; ++b) off += in[b * blockDim.x + threadIdx.x];
+        off = __reduce_add_sync(0xffffffffu, off);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&before, off);
+        __syncthreads();
+        off = before;
+    }
+    const uint32_t v = k < n ? in[k] : 0;
+    const uint32_t inc = block_inclusive_scan(v, ws);
+    const uint32_t exc = off + inc - v;
     if (k < n) out[k] = exc;
     if (k == n - 1) out[n] = exc + v;
+    if (of) {
+        const uint32_t m = __reduce_max_sync(0xffffffffu, k < n ? of[k] : 0u);
+        if ((threadIdx.x & 31) == 0) atomicMax(largest, (int)m);
+    }
 }
 
 __global__ void fill_kernel(const uint32_t *slot_dst, const uint32_t *slot_edge, uint64_t n_slots,
@@ -512,18 +535,26 @@ __global__ void copy_blocks_kernel(const uint16_t *win_row, uint16_t *win, uint6
 
 // One relaxation of the shortest paths over a table: lo_dst = min(lo_dst, lo_src + shift).
 // Skipped when *prev is given and zero (the pass before changed nothing); *changed
-// is set where a value fell.
+// is set where a value fell.  A small table's launch lasts as long as its longest
+// row's chain of dependent loads (rows of a hundred edges come up), so eight lanes
+// share a row there; a large one is bound by its instructions and takes a thread per
+// row (first triangular strips, cold: width 12 3.30 ms with one lane, 2.81 with eight;
+// width 16 29.9 and 34.3).
+constexpr uint64_t kWinManyLanes = 65536;  // rows up to which a row takes eight lanes
+template <uint32_t kLanes>
 __global__ void relax_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits,
                                  const uint16_t *win_in, uint16_t *win_out, const int *prev, int *changed) {
     if (prev && *prev == 0) return;
-    const uint64_t d = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (d >= n_dst) return;
-    const uint32_t mask = (1u << src_bits) - 1u;
+    const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, d = k / kLanes;
+    const uint32_t mask = (1u << src_bits) - 1u, lane = k % kLanes;
     uint32_t m = 255;
-    for (uint32_t e = row_ptr[d], e1 = row_ptr[d + 1]; e < e1; ++e) {
-        const uint32_t q = edges[e], lo = win_in[q & mask] & 0xffu;
-        if (lo != 255) m = min(m, min(lo + ((q >> src_bits) & 3u), 254u));
-    }
+    if (d < n_dst)
+        for (uint32_t e = row_ptr[d] + lane, e1 = row_ptr[d + 1]; e < e1; e += kLanes) {
+            const uint32_t q = edges[e], lo = win_in[q & mask] & 0xffu;
+            if (lo != 255) m = min(m, min(lo + ((q >> src_bits) & 3u), 254u));
+        }
+    for (uint32_t o = kLanes / 2; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (d >= n_dst || lane) return;
     const uint32_t w = win_out[d];
     if (m < (w & 0xffu)) {
         win_out[d] = (uint16_t)((w & 0xff00u) | m);
@@ -532,14 +563,15 @@ __global__ void relax_win_kernel(const uint32_t *row_ptr, const uint32_t *edges,
 }
 
 // Every transition keeps its source's window inside its destination's: lo_dst <=
-// lo_src + shift, and V_src - blocks_src + shift <= V_dst - blocks_dst.
+// lo_src + shift, and V_src - blocks_src + shift <= V_dst - blocks_dst.  (Lanes as above.)
+template <uint32_t kLanes>
 __global__ void check_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits, int sites,
                                  const uint16_t *win_in, const uint16_t *win_out, int *bad) {
-    const uint64_t d = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, d = k / kLanes;
     if (d >= n_dst) return;
     const uint32_t mask = (1u << src_bits) - 1u, w = win_out[d];
     bool ok = true;
-    for (uint32_t e = row_ptr[d], e1 = row_ptr[d + 1]; e < e1; ++e) {
+    for (uint32_t e = row_ptr[d] + (uint32_t)(k % kLanes), e1 = row_ptr[d + 1]; e < e1; e += kLanes) {
         const uint32_t q = edges[e], sh = (q >> src_bits) & 3u, x = win_in[q & mask];
         if ((x & 0xffu) == 255) continue;
         ok = ok && (w & 0xffu) <= min((x & 0xffu) + sh, 254u) && (w >> 8) + sh <= (x >> 8) + (uint32_t)sites;
@@ -592,14 +624,19 @@ struct Scratch {
 
 static size_t scan_bytes(uint64_t n) { return Scratch::span(((n + kScanThreads - 1) / kScanThreads + 1) * 4); }
 
-// out[0..n]: exclusive scan of cnt, with the total at the end (asynchronous on sc->st).
-static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *out, Scratch *sc) {
+// out[0..n]: exclusive scan of cnt, with the total at the end, and the largest of
+// of[0..n) into *largest (asynchronous on sc->st).
+static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *out, Scratch *sc, const uint32_t *of = nullptr,
+                          int *largest = nullptr) {
     uint64_t nb = (n + kScanThreads - 1) / kScanThreads;
     if (nb > (1u << 31)) return fail(CP_EINVAL, "scan too large");
-    uint32_t *sums = sc->take<uint32_t>(nb + 1);
-    scan_block_sums<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums);
-    scan_sums_serial<<<1, kScanThreads, 0, sc->st>>>(sums, (uint32_t)nb);
-    scan_finish<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums, out);
+    uint32_t *sums = nullptr;
+    if (nb > kScanAlone) {
+        sums = sc->take<uint32_t>(nb + 1);
+        scan_block_sums<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums);
+        scan_sums_serial<<<1, kScanThreads, 0, sc->st>>>(sums, (uint32_t)nb);
+    }
+    scan_finish<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums, out, of, largest);
     CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
@@ -728,9 +765,8 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
     } else
         build_terms_kernel<<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst, slot_edge, K, err);
     count_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, op.src_bits, cnt, csum, err + 2);
-    max_count_kernel<<<608, 256, 0, st>>>(csum, n_dst, err + 1);
     CP_CUDA_TRY(cudaGetLastError());
-    if ((rc = scan_exclusive(cnt, n_dst, tab->row_ptr, sc))) return rc;
+    if ((rc = scan_exclusive(cnt, n_dst, tab->row_ptr, sc, csum, err + 1))) return rc;
     int herr[3] = {0, 0, 0};
     uint32_t nnz = 0;
     CP_CUDA_TRY(cudaMemcpyAsync(herr, err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -815,8 +851,9 @@ static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
     int *flags = sc->take<int>(kMaxPasses + 1);  // changed, one per pass; then the checks' flag
     cudaError_t e = cudaMemsetAsync(flags, 0, (kMaxPasses + 1) * sizeof(int), st);
     auto relax = [&](const SiteTable &t, const int *prev, int *changed) {
-        relax_win_kernel<<<grid(t.n_dst), 128, 0, st>>>(t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.win_in,
-                                                       const_cast<uint16_t *>(t.win_out), prev, changed);
+        const bool many = t.n_dst <= kWinManyLanes;
+        (many ? relax_win_kernel<8> : relax_win_kernel<1>)<<<grid(t.n_dst * (many ? 8 : 1)), 128, 0, st>>>(
+            t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.win_in, const_cast<uint16_t *>(t.win_out), prev, changed);
     };
     int host[kMaxPasses + 1] = {}, pass = 0;
     bool done = false;
@@ -828,9 +865,11 @@ static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
         for (auto &t : ts->last) relax(t, nullptr, flags + kMaxPasses);
         e = cudaMemsetAsync(flags + kMaxPasses, 0, sizeof(int), st);
         for (auto *chain : {&ts->row, &ts->last})
-            for (auto &t : *chain)
-                check_win_kernel<<<grid(t.n_dst), 128, 0, st>>>(t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.sites,
-                                                               t.win_in, t.win_out, flags + kMaxPasses);
+            for (auto &t : *chain) {
+                const bool many = t.n_dst <= kWinManyLanes;
+                (many ? check_win_kernel<8> : check_win_kernel<1>)<<<grid(t.n_dst * (many ? 8 : 1)), 128, 0, st>>>(
+                    t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.sites, t.win_in, t.win_out, flags + kMaxPasses);
+            }
         check_e0_kernel<<<grid(ts->row[0].n_src), 128, 0, st>>>(win[0], ts->row[0].n_src, flags + kMaxPasses);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(host, flags, sizeof(host), cudaMemcpyDeviceToHost, st);
@@ -859,6 +898,22 @@ static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
             dev_free(t.edges);
             t.edges = nullptr;
         }
+    return CP_OK;
+}
+
+__global__ void window_degrees_kernel(const uint16_t *win, uint64_t n, int v, int cap, unsigned long long *sum) {
+    unsigned long long s = 0;
+    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) {
+        const int lo = win[k] & 0xff, hi = min(cap, v - (win[k] >> 8));
+        if (lo != 0xff && hi >= lo) s += hi - lo + 1;
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(sum, s);
+}
+
+int add_window_degrees(const uint16_t *win, uint64_t n, int v, int cap, unsigned long long *sum_dev, cudaStream_t st) {
+    window_degrees_kernel<<<304, 256, 0, st>>>(win, n, v, cap, sum_dev);
+    CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
 
