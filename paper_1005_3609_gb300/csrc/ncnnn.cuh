@@ -10,13 +10,20 @@
 namespace cp {
 
 constexpr int kMaxL = CP_MAX_L;
-constexpr uint8_t kFresh = 31;  // temporary label of a detached site (labels are < kMaxL)
-
-// A partition of the sites 0..m-1: block labels in first-occurrence order.
+// A partition of the sites 0..m-1: block labels in first-occurrence order.  Also as
+// words of four labels: the arrays live in local memory, where a byte at a time was a
+// chain of dependent accesses per operator (relabelling through a 32-entry map, about a
+// thousand cycles), so the operators below treat four labels at once and keep the
+// order of first occurrence without a map.  Bytes past the m-th mean nothing.
 struct Labels {
-    uint8_t v[kMaxL];
+    union {
+        uint8_t v[kMaxL];
+        uint32_t w[kMaxL / 4];
+    };
 };
+static_assert(kMaxL % 4 == 0 && kMaxL <= 32, "whole words; a bit per site or label");
 
+// Labels in first-occurrence order, from any (validation).
 __device__ __forceinline__ void canonicalise(Labels &s, int m) {
     uint8_t map[32];
 #pragma unroll
@@ -29,48 +36,91 @@ __device__ __forceinline__ void canonicalise(Labels &s, int m) {
     }
 }
 
-// J_{a,b} for a !~ b: merge the two blocks (the factor w is the caller's shift).
+// Number of blocks among the sites before i.
+__device__ __forceinline__ uint32_t blocks_before(const Labels &s, int i) {
+    uint32_t x = 0;  // largest label, byte by byte
+    for (int k = 0; k < i >> 2; ++k) x = __vmaxu4(x, s.w[k]);
+    if (i & 3) x = __vmaxu4(x, s.w[i >> 2] & ((1u << 8 * (i & 3)) - 1u));
+    x = __vmaxu4(x, x >> 16);
+    return i ? (max(x & 0xffu, (x >> 8) & 0xffu)) + 1 : 0;
+}
+
+// The smallest site t in (a, b) of site a's block, or -1.
+__device__ __forceinline__ int next_in_block(const Labels &s, int a, int b) {
+    if (a + 1 >= b) return -1;
+    const uint32_t x = s.v[a] * 0x01010101u;
+    int k = (a + 1) >> 2;
+    uint32_t eq = __vcmpeq4(s.w[k], x) & (~0u << 8 * ((a + 1) & 3));
+    while (eq == 0) {
+        if (4 * ++k >= b) return -1;
+        eq = __vcmpeq4(s.w[k], x);
+    }
+    const int t = 4 * k + (__ffs((int)eq) - 1) / 8;
+    return t < b ? t : -1;
+}
+
+// J_{a,b} for a !~ b: merge the two blocks (the factor w is the caller's shift).  The
+// later label goes, and the ones above it move down by one.
 __device__ __forceinline__ void join_blocks(Labels &s, int m, int a, int b) {
-    uint8_t la = s.v[a], lb = s.v[b];
-    for (int i = 0; i < m; ++i)
-        if (s.v[i] == lb) s.v[i] = la;
-    canonicalise(s, m);
+    const uint32_t la = min(s.v[a], s.v[b]) * 0x01010101u, lb = max(s.v[a], s.v[b]) * 0x01010101u;
+    for (int k = 0; 4 * k < m; ++k) {
+        const uint32_t x = s.w[k], eq = __vcmpeq4(x, lb);
+        s.w[k] = (eq & la) | (~eq & __vadd4(x, __vcmpgtu4(x, lb)));
+    }
 }
 
-// D_i: site i becomes a singleton.
+// D_i: site i becomes a singleton.  If its block x began before i, the singleton takes
+// the first label not seen before i; if it begins at i, the singleton keeps x and the rest
+// of the block takes the first label not seen before its next site.  The labels from
+// there on move up by one.
 __device__ __forceinline__ void detach_site(Labels &s, int m, int i) {
-    s.v[i] = kFresh;
-    canonicalise(s, m);
+    const uint32_t x = s.v[i], c = blocks_before(s, i);
+    uint32_t from = c;
+    if (x == c) {
+        const int f = next_in_block(s, i, m);
+        if (f < 0) return;
+        from = blocks_before(s, f);
+    }
+    const uint32_t x4 = x * 0x01010101u, from4 = from * 0x01010101u;
+    for (int k = i >> 2; 4 * k < m; ++k) {
+        const uint32_t y = s.w[k], eq = x == c ? __vcmpeq4(y, x4) : 0u;
+        s.w[k] = (eq & from4) | (~eq & __vsub4(y, __vcmpgeu4(y, from4)));
+    }
+    s.v[i] = (uint8_t)c;
 }
 
-// Non-crossing test in O(m): scanning left to right, a block that reappears
-// must be the innermost open one.
+// Non-crossing test in O(m): the blocks that may go on are open, a bit each; a block
+// that reappears must be one of them and closes the later ones (labels grow in the
+// order of first occurrence).
 __device__ __forceinline__ bool is_noncrossing(const Labels &s, int m) {
-    int8_t last[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) last[k] = -1;
-    for (int i = 0; i < m; ++i) last[s.v[i]] = (int8_t)i;
-    uint8_t stack[kMaxL];
-    int sp = 0;
-    uint32_t open = 0;  // bit set of open labels
+    uint32_t open = 0, next = 0;
+    bool ok = true;
     for (int i = 0; i < m; ++i) {
-        uint8_t b = s.v[i];
-        if (open >> b & 1u) {
-            if (sp == 0 || stack[sp - 1] != b) return false;
-            if (last[b] == i) { --sp; open &= ~(1u << b); }
-        } else if (last[b] != i) {
-            stack[sp++] = b;
-            open |= 1u << b;
+        const uint32_t x = s.v[i];
+        if (x == next) {
+            open |= 1u << next++;
+        } else {
+            ok = ok && x < next && (open >> x & 1u);
+            open &= (2u << (x & 31u)) - 1u;
         }
     }
-    return true;
+    return ok;
+}
+
+// Bit j: the sites j and j + 1 are in one block.
+__device__ __forceinline__ uint32_t adjacent_pairs(const Labels &s, int m) {
+    uint32_t bits = 0;
+    for (int k = 0; 4 * k < m - 1; ++k) {
+        const uint32_t x = s.w[k], y = k + 1 < kMaxL / 4 ? s.w[k + 1] : 0u;
+        const uint32_t eq = __vcmpeq4(x, __funnelshift_r(x, y, 8)) & 0x01010101u;
+        bits |= (eq * 0x01020408u >> 24 & 15u) << 4 * k;
+    }
+    return bits & ((1u << (m - 1)) - 1u);
 }
 
 // Neighbour rule: no (j, j+1) in one block, except the pair j == skip.
 __device__ __forceinline__ bool nn_ok(const Labels &s, int m, int skip) {
-    for (int j = 0; j + 1 < m; ++j)
-        if (j != skip && s.v[j] == s.v[j + 1]) return false;
-    return true;
+    return (adjacent_pairs(s, m) & ~(skip >= 0 ? 1u << skip : 0u)) == 0;
 }
 
 // Rank of an NCNNN partition of the points lo..hi-1 in the paper's order
@@ -89,9 +139,7 @@ __device__ __forceinline__ uint64_t ncnnn_rank(const Labels &s, int lo, int hi, 
         while (b - a > 2) {
             int n = b - a;
             if (s.v[a + 1] == s.v[a]) return ~0ull;
-            int j = -1;
-            for (int t = a + 2; t < b; ++t)
-                if (s.v[t] == s.v[a]) { j = t; break; }
+            const int j = next_in_block(s, a, b);
             if (j < 0) { ++a; continue; }
             int k = j - a - 2;
             uint64_t cr = T.cnt[b - j];
@@ -110,7 +158,8 @@ __device__ __forceinline__ uint64_t ncnnn_rank(const Labels &s, int lo, int hi, 
 // Inverse of ncnnn_rank on points lo..hi-1; labels are assigned in
 // first-occurrence order, so the result is canonical when lo == 0.
 __device__ __forceinline__ void ncnnn_unrank(uint64_t r, int lo, int hi, Labels &s, const RankTables &T) {
-    for (int i = lo; i < hi; ++i) s.v[i] = 0xFF;
+#pragma unroll
+    for (int k = 0; k < kMaxL / 4; ++k) s.w[k] = ~0u;
     uint8_t next = 0;
     int sa[kMaxL + 1], sb[kMaxL + 1];
     uint64_t sr[kMaxL + 1];
@@ -154,9 +203,7 @@ __device__ __forceinline__ uint64_t nc_rank(const Labels &s, int lo, int hi, con
     uint64_t mu = 1;
     for (;;) {
         while (b - a > 1) {
-            int n = b - a, j = -1;
-            for (int t = a + 1; t < b; ++t)
-                if (s.v[t] == s.v[a]) { j = t; break; }
+            const int n = b - a, j = next_in_block(s, a, b);
             if (j < 0) { ++a; continue; }
             int k = j - a - 1;
             r += mu * T.offc[n * kTblStride + k];
@@ -171,7 +218,8 @@ __device__ __forceinline__ uint64_t nc_rank(const Labels &s, int lo, int hi, con
 }
 
 __device__ __forceinline__ void nc_unrank(uint64_t r, int lo, int hi, Labels &s, const RankTables &T) {
-    for (int i = lo; i < hi; ++i) s.v[i] = 0xFF;
+#pragma unroll
+    for (int k = 0; k < kMaxL / 4; ++k) s.w[k] = ~0u;
     uint8_t next = 0;
     int sa[kMaxL + 1], sb[kMaxL + 1];
     uint64_t sr[kMaxL + 1];

@@ -108,14 +108,12 @@ __device__ int op_d(Term *t, int n, int m, int i) {
 }
 
 // P_{j,j+1} for j in [lo, hi) except `skip`.
-__device__ int op_p(Term *t, int n, int lo, int hi, int skip) {
+__device__ int op_p(Term *t, int n, int m, int lo, int hi, int skip) {
+    if (lo >= hi) return n;
+    const uint32_t pairs = ((1u << hi) - 1u) & ~((1u << lo) - 1u) & ~(skip >= 0 ? 1u << skip : 0u);
     int w = 0;
-    for (int j = 0; j < n; ++j) {
-        bool ok = true;
-        for (int q = lo; q < hi; ++q)
-            if (q != skip && t[j].s.v[q] == t[j].s.v[q + 1]) { ok = false; break; }
-        if (ok) t[w++] = t[j];
-    }
+    for (int j = 0; j < n; ++j)
+        if ((adjacent_pairs(t[j].s, m) & pairs) == 0) t[w++] = t[j];
     return w;
 }
 
@@ -164,18 +162,18 @@ __device__ __noinline__ int factor_terms(const OpDesc &op, const Labels &s, Term
         case OP_SQUARE:  // (prod_{j!=i} P) V_i H_{i,i+1};  T_m = (prod P) V_m      eq. (T_sq_proj)
             if (i < m - 1) n = op_h(t, n, m, i, i + 1);
             n = op_v(t, n, m, i);
-            n = op_p(t, n, 0, m - 1, i < m - 1 ? i : -1);
+            n = op_p(t, n, m, 0, m - 1, i < m - 1 ? i : -1);
             break;
         case OP_TRIANGULAR:  // (prod P) V_i H_{i-1,i} H_{i,i+1}                    Sec. 3.3
             if (i < m - 1) n = op_h(t, n, m, i, i + 1);
             if (i > 0) n = op_h(t, n, m, i - 1, i);
             n = op_v(t, n, m, i);
-            n = op_p(t, n, 0, m - 1, -1);
+            n = op_p(t, n, m, 0, m - 1, -1);
             break;
         case OP_LAST:  // (prod_{j>i} P) D_i H_{i,i+1}                                eq. (T_last_i)
             if (i < m - 1) n = op_h(t, n, m, i, i + 1);
             n = op_d(t, n, m, i);
-            n = op_p(t, n, i + 1, m - 1, -1);
+            n = op_p(t, n, m, i + 1, m - 1, -1);
             break;
         case OP_POTTS_SQUARE:  // V_i H_{i,i+1}: the rows of T = (prod V)(prod H), Sec. 3.2
             if (i < m - 1) n = op_hv(t, n, m, i, i + 1, op.v);
