@@ -20,7 +20,9 @@
 //              passes.  Per edge and step: one 16-byte shared load and two
 //              multiply-adds per word.
 //
-// What bounds it: instructions.  Width 14, D = 63, 16 primes (57 346 rows, 365 000
+// What bounds it: the shared-memory data path, each source word going through it twice
+// (copy and load; 83% of its rate in the middle launches of the square width-16 row, where
+// DRAM gives 3.0 TB/s and L2 is at 40%), with the issue slots next (64%).  Width 14, D = 63, 16 primes (57 346 rows, 365 000
 // edges of a two-site table): 0.66 instructions per scheduler and cycle, 66% of the
 // shared-memory data path, DRAM at a quarter of its rate, 0.107 ms; the
 // producer/consumer kernel on whole rows that this one replaces took 0.155 ms.  One
@@ -29,7 +31,7 @@
 // once and an edge's first word kept from its copy, 3.73 and 1.28 ms; with two-warp
 // instead of four-warp blocks 3.67 and 1.25 ms (one-warp blocks 3.72, 1.30).
 // 28 warps per SM (72 registers) beat 24 (4.31 before the last two changes) and 20, and
-// 32, which spill (4.02 after them); two edges in flight beat four (4.22 at 24 warps);
+// 32, which spill (4.02 after them); two edges in flight beat four (4.22 at 24 warps) in launches that fill the chip;
 // four steps beat six (4.26) and eight (4.87), which hold wider rows in one pass but
 // leave fewer warps.  Bulk copies with an mbarrier per slot (5.1) and loads straight to
 // registers (5.8) halve the shared-memory traffic but wait longer.

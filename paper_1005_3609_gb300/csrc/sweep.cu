@@ -10,7 +10,7 @@
 // row begins (both only read the current vector) and runs on two scratch
 // buffers while the strip moves on; its last factor writes the e_0 row
 // straight into the P~ array.  The primes are split into groups of Pg primes
-// (one strip per width and group).  The whole program -- vector resets, every
+// (one strip per width and group).  The whole program -- every
 // batched launch and the series kernel -- is captured once into a CUDA graph,
 // so a sweep is a single graph launch.  The prime grouping is picked by timing the
 // candidates (autotune) unless given.

@@ -261,10 +261,11 @@ __global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *sl
 
 // A two-site table, the second factor applied to every term of the first: LANES threads
 // per source state, each for every LANES-th term of the first factor, which meet in
-// shared memory to merge equal (dst, shift).  Bound by the latency of unranking,
-// relabelling and ranking in local memory while a table has few states: one thread per
-// source took 170 us a table at width 12 (5 798 states), eight 95 us; a table that fills
-// the SMs anyway takes two (eight repeat too much of the first factor).
+// shared memory to merge equal (dst, shift).  Bound by unranking, relabelling and ranking
+// in local memory: one thread per source took 170 us a table at width 12 (5 798 states),
+// eight 95 us, and with the labels as words 85 us (four lanes or a warp per source: the
+// cold tables of that width 2.91 or 2.71 ms against 2.55); a table that fills the SMs
+// anyway takes two (eight repeat too much of the first factor: width 14 8.4 against 5.6 ms).
 template <int LANES>
 __global__ void __launch_bounds__(128)
     build_fused_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *slot_dst, uint32_t *slot_edge, int K, int *err) {
