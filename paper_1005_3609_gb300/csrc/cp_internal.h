@@ -194,15 +194,23 @@ struct GatherTask {
 // first edge; one past the last edge}.  Rows differ a hundredfold in edges (the
 // states of many single sites collect most) and the heavy ones lie together, so
 // work is dealt out by edges and not by rows, and a heavy row's degrees are split
-// over kSplitParts warps.  A warp walks its edges one after another: tables too
-// small to give every resident warp 32 of them have smaller units.
+// over kSplitParts warps.  A warp walks its edges one after another, 32 listed at a time.
+// Large tables have units of 64 edges (start-up and draining per unit: square k = 33 sweep
+// 82.2 ms, triangular 29.9, width 17 on 5 primes 5.98, against 83.0, 31.8, 6.43 with 32 and
+// 85.8, 30.1, 5.74 with 128, whose last wave is long); tables of fewer than 8192 units
+// (two waves of resident warps) halve them, down to 4 edges (triangular 13 x 14 on 8
+// primes 2.80 ms, served mix 5.39, square sweep 86.4; the line at 4096 units 3.00, 5.56,
+// 85.9, at 16384 2.76, 5.39, 87.7: the last three with rows split from 24 or 32 edges).  Rows of
+// more than two units' edges are split (from one unit's on: square sweep 86.4, triangular
+// 34.0 ms, against 83.0 and 31.8), from 24 edges in the smallest units (16: triangular
+// 13 x 14 2.89), into four parts (two or eight: 1-3% slower solves).
 constexpr uint32_t kSplitParts = 4;
 inline uint32_t unit_edges(uint64_t nnz) {
-    uint32_t u = 32;
-    while (u > 4 && nnz < 4096ull * u) u /= 2;
+    uint32_t u = 64;
+    while (u > 4 && nnz < 8192ull * u) u /= 2;
     return u;
 }
-inline uint32_t split_edges(uint32_t unit) { return unit < 16 ? 16 : unit; }
+inline uint32_t split_edges(uint32_t unit) { return unit < 12 ? 24 : 2 * unit; }
 constexpr uint32_t kPackRows = 32;   // rows packed into units together
 
 // What a vector's primes are to the gathers: the prime lanes, then each lane's

@@ -5,7 +5,7 @@
 // by w a shift of the degree index), on the degree windows of cp_internal.h:
 // only the degrees that can be non-zero are read, computed and written.
 //
-// A warp takes one unit of work (a few consecutive destination rows with about 32
+// A warp takes one unit of work (a few consecutive destination rows with up to 64
 // edges, cp_internal.h) and works alone:
 //   front end  32 edges at a time, one per lane: the edge's word and its source's
 //              window, the window of its destination row, their intersection; the
@@ -21,7 +21,7 @@
 //              multiply-adds per word.
 //
 // What bounds it: the shared-memory data path, each source word going through it twice
-// (copy and load; 83% of its rate in the middle launches of the square width-16 row, where
+// (copy and load; 80% of its rate in the middle launches of the square width-16 row, where
 // DRAM gives 3.0 TB/s and L2 is at 40%), with the issue slots next (64%).  Width 14, D = 63, 16 primes (57 346 rows, 365 000
 // edges of a two-site table): 0.66 instructions per scheduler and cycle, 66% of the
 // shared-memory data path, DRAM at a quarter of its rate, 0.107 ms; the
@@ -29,7 +29,8 @@
 // row of the width-16 strip 7.73 -> 3.94 ms, triangular (D = 32) 5.32 -> 1.42 ms; with
 // the constants of a row's primes loaded once per row, the lane's prime group computed
 // once and an edge's first word kept from its copy, 3.73 and 1.28 ms; with two-warp
-// instead of four-warp blocks 3.67 and 1.25 ms (one-warp blocks 3.72, 1.30).
+// instead of four-warp blocks 3.67 and 1.25 ms (one-warp blocks 3.72, 1.30); units of 64
+// edges instead of 32 took the square k = 33 sweep from 86.4 to 82.2 ms (cp_internal.h).
 // 28 warps per SM (72 registers) beat 24 (4.31 before the last two changes) and 20, and
 // 32, which spill (4.02 after them); two edges in flight beat four (4.22 at 24 warps) in launches that fill the chip;
 // four steps beat six (4.26) and eight (4.87), which hold wider rows in one pass but
