@@ -340,7 +340,8 @@ int cp_sweep_set_primes(cp_sweep *sw, const uint32_t *primes_host, int n_primes)
 /* Run the sweep's batched gather launches once WITHOUT the graph, with a CUDA event
  * pair around each batched gather launch on the sweep's stream: *gather_ms =
  * summed gather kernel time, *n_gather = launches, *total_ms = whole pass
- * (no series kernel).  Synchronises.  For roofline measurements. */
+ * (no series kernel: the series of the last run stay; P~ is this pass's).
+ * Synchronises.  For roofline measurements. */
 int cp_sweep_profile(cp_sweep *sw, float *gather_ms, int *n_gather, float *total_ms);
 
 void cp_sweep_destroy(cp_sweep *sw);

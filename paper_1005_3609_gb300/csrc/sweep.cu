@@ -547,6 +547,23 @@ extern "C" int cp_sweep_series_integers(cp_sweep *sw, uint32_t *limbs_out, size_
     return crt_outcome(flags, 3 * n);
 }
 
+// The gathers store signed representatives; a run's series kernel puts residues in
+// their place, and this does where it does not follow.  words: per prime group.
+__global__ void ptilde_residues_kernel(uint32_t *ptilde, const uint32_t *primes, size_t words, int Pp) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    uint32_t *x = ptilde + blockIdx.y * words + i;
+    if ((int)*x < 0) *x += primes[blockIdx.y * kPrimeWords + i % Pp];
+}
+
+static int launch_ptilde_residues(cp_sweep *sw) {
+    const size_t words = sw->rects.size() * (size_t)sw->D1 * sw->Pp;
+    ptilde_residues_kernel<<<dim3((unsigned)((words + 255) / 256), sw->groups), 256, 0, sw->stream>>>(
+        sw->ptilde_dev, sw->primes_dev, words, sw->Pp);
+    CP_CUDA_TRY(cudaGetLastError());
+    return CP_OK;
+}
+
 // The same program without the graph, with an event pair around every batched
 // gather launch: sum of gather kernel times and number of gather launches.
 extern "C" int cp_sweep_profile(cp_sweep *sw, float *gather_ms, int *n_gather, float *total_ms) {
@@ -562,7 +579,9 @@ extern "C" int cp_sweep_profile(cp_sweep *sw, float *gather_ms, int *n_gather, f
         cudaEventRecord(ev[2 * t + 1], sw->stream);
     }
     CP_CUDA_TRY(cudaEventRecord(ev[2 * nst + 1], sw->stream));
-    cudaError_t e = cudaEventSynchronize(ev[2 * nst + 1]);
+    const int rr = launch_ptilde_residues(sw);
+    if (!rc) rc = rr;
+    cudaError_t e = cudaStreamSynchronize(sw->stream);
     float sum = 0, tot = 0;
     for (size_t t = 0; t < nst && e == cudaSuccess; ++t) {
         float ms = 0;
