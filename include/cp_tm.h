@@ -273,8 +273,9 @@ typedef struct cp_sweep cp_sweep;
  *       16, 32, 64, 128 = chunk gather kernel (rows of 16-byte chunks, dealt to the
  *       warps by edges).  With the latter the bits above, (16..192 << 12),
  *       (1, 2, 4, 8 << 20), (1, 2, 4 << 24) and (1, 2 << 28), are accepted and
- *       choose nothing.  Launches that the chunk kernel cannot take (large
- *       coefficients, small primes) run on the register kernel;
+ *       choose nothing.  Launches that the chunk kernel cannot take (Potts
+ *       coefficients beyond a byte, rows that are not whole 16-byte chunks) run on
+ *       the register kernel;
  * prime_groups: number of strips per width, dividing n_primes, or 0 = autotune.
  * cuda_stream must be a non-default stream (the program is graph-captured on it).
  * Errors: CP_EINVAL (k < 4, k/2 > CP_MAX_L, series longer than 128 terms, bad
@@ -334,7 +335,9 @@ int cp_sweep_series_integers(cp_sweep *sw, uint32_t *limbs_host, size_t limbs_le
 int cp_sweep_read_series_device(cp_sweep *sw, uint32_t *out_dev, size_t out_len);
 
 /* Replace the sweep's primes (same count) for the next run: a host-to-device
- * copy of n_primes words on the sweep's stream; the tables and the graph stay. */
+ * copy on the sweep's stream; the tables stay.  So does the graph, except where the
+ * smallest prime crosses the bound of the gathers' shorter reduction (about 10^7):
+ * then the call synchronises and captures the program again. */
 int cp_sweep_set_primes(cp_sweep *sw, const uint32_t *primes_host, int n_primes);
 
 /* Run the sweep's batched gather launches once WITHOUT the graph, with a CUDA event

@@ -181,7 +181,8 @@ struct GatherTask {
     uint32_t src_bits;        // edge format of the table
     uint32_t seg;             // chunk kernel: degrees of one pass over a row
     uint32_t r32;             // 32 modulo cpd
-    uint32_t fast;            // 1: the coefficients and primes suit the chunk kernel's sums (fast_ok, modred.cuh)
+    uint32_t chunk;           // 1: rows and coefficients suit the chunk kernel
+    uint32_t fast;            // 1: the coefficients and primes suit its 32-bit reduction (fast_ok, modred.cuh)
     uint32_t fast_k0;         // their offset
     int32_t v_in, v_out;      // vertices of the input and of the output vector (window bound V - blocks)
     int32_t cap;              // highest degree kept, D
@@ -214,7 +215,7 @@ inline uint32_t split_edges(uint32_t unit) { return unit < 12 ? 24 : 2 * unit; }
 constexpr uint32_t kPackRows = 32;   // rows packed into units together
 
 // What a vector's primes are to the gathers: the prime lanes, then each lane's
-// multiplier of the chunk kernel's reduction (256 bytes).
+// multiplier of the chunk kernel's reductions (256 bytes).
 constexpr int kPrimeWords = 2 * CP_MAX_PRIMES;
 void fill_prime_block(const uint32_t *primes, int n_primes, int lanes, uint32_t *block);
 
@@ -232,7 +233,7 @@ inline int padded_primes(int P) { return (P + 3) & ~3; }
 // Gather tile (low 12 bits): 1, 2, 4, 8 = register kernel with that many rows
 // per warp (8 warps per block); 16, 32, 64, 128 = chunk kernel.  The other bits are
 // accepted as cp_tm.h lists them and choose nothing.  A batch with rows that are
-// not 16-byte chunked, large coefficients or small primes uses the register kernel.
+// not 16-byte chunked or with large coefficients uses the register kernel.
 constexpr int kTileChunk = 32;
 constexpr int kChunkWarps = 2;         // warps of a block of the chunk kernel
 constexpr int kChunkBlocksPerSM = 14;   // its launch bound
@@ -246,7 +247,8 @@ uint32_t task_blocks(const GatherTask &t, int items);
 uint32_t assign_blocks(std::vector<GatherTask> &tasks, int items);
 // Effective tile for a batch (falls back to the register kernel when needed).
 int effective_tile(const std::vector<GatherTask> &tasks, int items);
-// The chunk kernel takes coefficients as signed bytes; fast_ok (modred.cuh) bounds their sums.
+// The chunk kernel takes coefficients as signed bytes, with sums below kChunkMaxSum; of
+// which fast_ok (modred.cuh) says for which primes the 32-bit reduction is exact.
 constexpr uint32_t kChunkMaxCoef = 127;
 bool table_fast(const SiteTable &tab, uint32_t min_prime);
 // Launch a batch of tasks (block_begin assigned for `items`), by value in the

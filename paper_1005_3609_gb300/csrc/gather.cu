@@ -193,7 +193,7 @@ static uint32_t magic_for(uint32_t d) { return d <= 1 ? 0u : (uint32_t)(((1ull <
 void fill_prime_block(const uint32_t *primes, int n_primes, int lanes, uint32_t *block) {
     for (int k = 0; k < lanes; ++k) {
         block[k] = primes[std::min(k, n_primes - 1)];
-        block[CP_MAX_PRIMES + k] = fast_magic(block[k]);
+        block[CP_MAX_PRIMES + k] = chunk_magic(block[k]);
     }
 }
 
@@ -223,6 +223,7 @@ void append_gather_task(std::vector<GatherTask> *tasks, const SiteTable &tab, co
     t.r32 = 32u % t.cpd;
     t.n_primes = (uint32_t)P;
     t.src_bits = (uint32_t)tab.op.src_bits;
+    t.chunk = v4 && tab.max_abs_coef <= kChunkMaxCoef && tab.max_coef_sum < kChunkMaxSum ? 1u : 0u;
     t.fast = table_fast(tab, min_prime) ? 1u : 0u;
     t.fast_k0 = fast_offset(tab.max_coef_sum);
     t.v_in = v_in;

@@ -113,6 +113,24 @@ __device__ __forceinline__ uint32_t fast_reduce(const Acc2 &a, uint32_t p, uint3
     return a.lo - (uint32_t)q1 * p;
 }
 
+// The same for any prime, and sums of coefficients S < 2^15 (kChunkMaxSum): h = hi + k0 =
+// sum c xh, l = lo - h 2^16 = sum c xl as a signed word (|l| < S 2^16 < 2^31), so
+// v = sum c x = h 2^16 + l exactly and u = v + p 2^15 lies in (0, p 2^16).  With t =
+// chunk_shift(p), m = floor(2^(32 + t) / p) and q = floor(floor(u / 2^t) m / 2^32),
+//   u / p >= q > u / p - u / 2^(32 + t) - 2^t / p - 1 > u / p - 2:
+// for p >= 2^17, t = 16, the terms are below p / 2^32 < 1/2 and 1/2, for smaller p of b
+// bits, t = b - 2, below 2^-14 and 1/2.  So r = u - q p lies in [0, 2p), and the word
+// stored, r - p, in [-p, p).  A few times the instructions of the 32-bit reduction, once a
+// row and word: square 12 x 13 on 8 primes near 10^6 1.28 ms, near 2^31 with the 32-bit one
+// 1.14; square width 16, D 63, 16 primes, eight rows 19.5 ms (on the register kernel 13.2
+// and 64.7).
+__device__ __forceinline__ uint32_t any_reduce(const Acc2 &a, uint32_t k0, uint32_t p, uint32_t m, uint32_t t) {
+    const int h = a.hi + (int)k0;
+    const int l = (int)(a.lo - ((uint32_t)h << 16));
+    const unsigned long long u = (unsigned long long)((long long)h * 65536 + l + ((long long)p << 15));
+    return (uint32_t)u - (__umulhi((uint32_t)(u >> t), m) + 1u) * p;
+}
+
 // Asynchronous 16-byte copy to shared memory where t < len (unsigned), zeros written elsewhere.
 __device__ __forceinline__ void cp16_below(uint32_t dst, const uint4 *src, uint32_t t, uint32_t len) {
     asm volatile(
@@ -147,8 +165,8 @@ __device__ __forceinline__ const uint4 *ptr64(uint32_t lo, uint32_t hi) {
     return reinterpret_cast<const uint4 *>(((uint64_t)hi << 32) | lo);
 }
 
-// kDepth: edges whose copies are in flight (a power of two).
-template <uint32_t kDepth>
+// kDepth: edges whose copies are in flight (a power of two); kAny: any_reduce.
+template <uint32_t kDepth, bool kAny>
 struct Warp {
     const GatherTask &t;
     uint4 *list;
@@ -185,8 +203,11 @@ struct Warp {
                 p = __ldg(consts + g);
                 m = __ldg(consts + CP_MAX_PRIMES / 4 + g);
             }
-            const uint4 v = make_uint4(fast_reduce(acc[k][0], p.x, m.x), fast_reduce(acc[k][1], p.y, m.y),
-                                       fast_reduce(acc[k][2], p.z, m.z), fast_reduce(acc[k][3], p.w, m.w));
+            auto reduced = [&](const Acc2 &a, uint32_t pi, uint32_t mi) {
+                return kAny ? any_reduce(a, t.fast_k0, pi, mi, chunk_shift(pi)) : fast_reduce(a, pi, mi);
+            };
+            const uint4 v = make_uint4(reduced(acc[k][0], p.x, m.x), reduced(acc[k][1], p.y, m.y),
+                                       reduced(acc[k][2], p.z, m.z), reduced(acc[k][3], p.w, m.w));
             stcs128_if(out + 32 * k, v, lane + 32 * k < nch ? 1u : 0u);
             g += t.r32;
             g = g >= t.cpd ? g - t.cpd : g;
@@ -351,7 +372,7 @@ struct Warp {
 // dv is added to the tasks' vertex counts; first: as if every task's `first` were set.
 // Launches overlap: a launch's blocks may start while the one before it drains, load
 // their unit's tables (which no launch writes) and only then wait for it.
-template <int N, uint32_t kDepth>
+template <int N, uint32_t kDepth, bool kAny>
 __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, int dv, int first) {
     extern __shared__ __align__(128) uint8_t slots[];  // per warp: kDepth slots of kSegChunks chunks
@@ -361,14 +382,14 @@ __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (id >= n_units) return;
     const GatherTask &t = pack.t[find_task(pack, n_tasks, id)];
-    Warp<kDepth> w(t, lists[warp]);
+    Warp<kDepth, kAny> w(t, lists[warp]);
     w.lane = lane;
     w.g0 = lane % t.cpd;
     w.slots = smem_addr(slots) + warp * kDepth * kSlotBytes + lane * 16u;
     w.unit(__ldg(t.units + (id - t.block_begin)), t.v_in + dv, t.v_out + dv, first || t.first ? 0 : t.cap);
 }
 
-bool chunk_usable(const GatherTask &t) { return t.vec4 && t.fast; }
+bool chunk_usable(const GatherTask &t) { return t.chunk != 0; }
 
 // Diagnostic: a wait that can never complete (an mbarrier nothing arrives on),
 // bounded by `cycles`; on expiry it sets bit 16 of *err and returns, like the
@@ -407,11 +428,16 @@ int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, 
         cfg.stream = st;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        auto go = [&](auto depth) -> cudaError_t {
+        bool any = false;
+        for (int k = 0; k < n; ++k) any = any || !pack.t[k].fast;
+        auto go = [&](auto depth, auto any_prime) -> cudaError_t {
             cfg.dynamicSmemBytes = kWarps * decltype(depth)::value * kSlotBytes;
-            return cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N, decltype(depth)::value>, pack, n, units, dv, first ? 1 : 0);
+            return cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N, decltype(depth)::value, decltype(any_prime)::value>, pack,
+                                      n, units, dv, first ? 1 : 0);
         };
-        CP_CUDA_TRY(units <= kFewUnits ? go(std::integral_constant<uint32_t, 4>()) : go(std::integral_constant<uint32_t, 2>()));
+        auto pick = [&](auto depth) { return any ? go(depth, std::true_type()) : go(depth, std::false_type()); };
+        CP_CUDA_TRY(units <= kFewUnits ? pick(std::integral_constant<uint32_t, 4>())
+                                       : pick(std::integral_constant<uint32_t, 2>()));
         return CP_OK;
     });
 }

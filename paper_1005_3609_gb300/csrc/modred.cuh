@@ -51,18 +51,6 @@ __host__ __device__ __forceinline__ ModRed modred_make(uint32_t p) {
 // The bias every accumulator of prime p starts from: p 2^21.
 __host__ __device__ __forceinline__ long long modred_bias(uint32_t p) { return (long long)p << 21; }
 
-// A signed representative of u mod p in [-p, p), as its 32-bit two's
-// complement: r - p with r = u - q p in [0, 2p) (one instruction fewer than
-// the full reduction).  The gathers read every input word as a signed 32-bit
-// value, so inputs in [-p, p) still give |v| < p S and the bias above covers
-// them; a gather whose output only feeds further gathers may store this.
-__device__ __forceinline__ uint32_t modred_reduce_signed(long long acc, uint32_t p, uint32_t m, uint32_t s) {
-    const unsigned long long u = (unsigned long long)acc;
-    const uint32_t h = (uint32_t)(u >> s);
-    const uint32_t q = __umulhi(h, m);
-    return (uint32_t)u - q * p - p;  // r - p, r in [0, 2p); exact modulo 2^32
-}
-
 // u mod p for an accumulator u = p 2^21 + v, |v| < p 2^20.
 __device__ __forceinline__ uint32_t modred_reduce(long long acc, uint32_t p, uint32_t m, uint32_t s) {
     const unsigned long long u = (unsigned long long)acc;
@@ -72,14 +60,27 @@ __device__ __forceinline__ uint32_t modred_reduce(long long acc, uint32_t p, uin
     return min(r, r - p);
 }
 
-// The chunk gather's sums (gather_chunk.cu): offset k0 of the upper halves for a
-// coefficient sum s, whether a prime suits it, and the prime's multiplier (below
-// 2^31, as such primes are above 2^17).
+// The chunk gather's sums (gather_chunk.cu), for coefficient sums below kChunkMaxSum:
+// offset k0 of the upper halves for a coefficient sum s, and whether a prime suits the
+// 32-bit reduction with it (such primes are above 2^17).
+constexpr uint32_t kChunkMaxSum = 1u << 15;
 constexpr uint32_t kFastMaxSum = 8192;
 __host__ __device__ __forceinline__ uint32_t fast_offset(uint32_t s) { return (3 * s + 1) / 2; }
 __host__ __device__ __forceinline__ bool fast_ok(uint32_t s, uint32_t p) {
     return s <= kFastMaxSum && (uint64_t)s * 163840u + 65536u + (((uint64_t)p * (s + 2)) >> 17) + 2u < p;
 }
-__host__ __device__ __forceinline__ uint32_t fast_magic(uint32_t p) { return (uint32_t)((1ull << 48) / p); }
+// A prime's multiplier floor(2^(32 + t) / p) there (at most 2^31), and its t: 16, for p below
+// 2^17 its bit length minus 2.
+__host__ __device__ __forceinline__ uint32_t chunk_shift(uint32_t p) {
+    if (p >= (1u << 17)) return 16;
+#ifdef __CUDA_ARCH__
+    return 30 - __clz((int)p);
+#else
+    uint32_t b = 2;
+    while ((p >> b) != 0) ++b;  // bit length
+    return b - 2;
+#endif
+}
+inline uint32_t chunk_magic(uint32_t p) { return (uint32_t)((1ull << (32 + chunk_shift(p))) / p); }
 
 }  // namespace cp

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import gpu_util
-from oracle import modp, tm_exact
+from oracle import tm_exact, tm_generic
 
 pytestmark = pytest.mark.gpu
 
@@ -68,3 +68,60 @@ def test_ptilde_keeps_its_primes_until_the_next_run():
                 want = tm_exact.ptilde("square", r, s)[:sw.n_terms]
                 want += [0] * (sw.n_terms - len(want))
                 assert res.tolist() == gpu_util.residues_of(want, one), (step, r, s)
+
+
+def solve(lattice, L, N, primes, D=-1, v=None, tile=0):
+    with cp.Strip(lattice, L, primes, max_degree=D, max_rows=N, v=v) as s:
+        s.set_tile(tile)
+        s.advance(N - 1)
+        return s.read()
+
+
+def solve_ms(lattice, L, N, primes, tile=0, D=-1):
+    """Median time of reset, rows and read-out, in ms."""
+    import time
+
+    import torch
+    with cp.Strip(lattice, L, primes, max_degree=D, max_rows=N) as s:
+        s.set_tile(tile)
+        ms = []
+        for _ in range(9):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            s.reset()
+            s.advance(N - 1)
+            s.read()
+            ms.append((time.perf_counter() - t) * 1e3)
+    return sorted(ms[2:])[3]
+
+
+# below the bound of the chunk kernel's 32-bit reduction the sums are put together to 64 bits: both shifts of its
+# quotient (2^17), the smallest primes, and large ones beside them
+@pytest.mark.parametrize("primes", [[2], [3, 2], [2, 3, 5, 7, 11], primes_from(65500, 4), primes_from(131000, 9),
+                                    primes_from(1 << 17, 4), primes_from(1000003, 6), primes_from(15 * 163840, 4),
+                                    [2, 2147483647, 131071, 131101, 1073741827]],
+                         ids=lambda p: "%d_%d" % (p[0], len(p)))
+@pytest.mark.parametrize("lattice", ["square", "triangular"])
+def test_small_primes(lattice, primes):
+    L, N = 6, 8
+    want = gpu_util.residues_of(tm_exact.ptilde(lattice, L, N), primes)
+    assert solve(lattice, L, N, primes).tolist() == want
+    assert solve(lattice, L, N, primes, D=7).tolist() == [w[:8] for w in want]
+    for L, N, D in ((12, 4, 40), (13, 5, -1)):  # heavy rows, split and in several passes
+        assert np.array_equal(solve(lattice, L, N, primes, D=D), solve(lattice, L, N, primes, D=D, tile=4)), L
+
+
+@pytest.mark.parametrize("lattice,v", [("square", 8), ("square", -9), ("square", 10), ("triangular", 4), ("triangular", -3)])
+def test_potts_sums_beyond_the_fast_bound(lattice, v):
+    # coefficients within a byte, their sums into one state in the hundreds and thousands: no prime below is fast
+    for primes in (primes_from(10007, 4), gpu_util.seed_primes(4, seed=43)):
+        want = gpu_util.residues_of(tm_generic.ztilde(lattice, 5, 4, v), primes)
+        assert solve(lattice, 5, 4, primes, v=v).tolist() == want
+        assert np.array_equal(solve(lattice, 9, 5, primes, v=v), solve(lattice, 9, 5, primes, v=v, tile=4))
+
+
+@pytest.mark.parametrize("lattice", ["square", "triangular"])
+def test_small_primes_are_no_slow_case(lattice):
+    # the same kernel with a longer reduction (the register kernel took 11 times as long here)
+    big, small = gpu_util.seed_primes(8, seed=44), primes_from(1000003, 8)
+    assert solve_ms(lattice, 12, 13, small) < 2.5 * solve_ms(lattice, 12, 13, big)
