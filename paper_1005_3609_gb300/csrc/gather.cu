@@ -16,7 +16,7 @@
 // are read, computed and written.
 //
 // One launch processes a batch of independent tasks (factors of different
-// strips); each block belongs to one task and covers 8 * RPW consecutive
+// strips); each block belongs to one task and covers 8 * rpw consecutive
 // destination rows of it, one warp per row at a time.
 #include <cuda_runtime.h>
 
@@ -51,28 +51,48 @@ __device__ __forceinline__ EdgeWin edge_window(const GatherTask &t, const uint2 
     return lo == 0xff ? EdgeWin{0, 0} : EdgeWin{lo + sh, hi + sh};
 }
 
-// acc += coef * in[src][chunk c - shift*cpd], for the edges held one per lane
-// in `my` and `win` (edge j in lane j), up to four loads in flight per lane.
+// 16 (4) bytes from global memory where pred != 0, else zero, without a branch.
 template <bool V4>
+__device__ __forceinline__ uint4 load_if(const uint32_t *in, size_t off, uint32_t pred) {
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (V4)
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+            : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
+            : "l"(reinterpret_cast<const uint4 *>(in) + off), "r"(pred));
+    else
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.global.nc.u32 %0, [%1];\n\t}"
+            : "+r"(v.x)
+            : "l"(in + off), "r"(pred));
+    return v;
+}
+
+// acc += coef * in[src][chunk c - shift*cpd], for the edges held one per lane
+// in `my` and `win` (edge j in lane j), kFlight loads in flight per lane.
+// deg0, deg1: the lowest and the highest degree of the warp's chunks; edges that
+// reach none of them are passed over.  A launch lasts as long as its heaviest row, a
+// chain of dependent steps of kFlight edges: with a branch per load instead of a
+// predicate and every edge walked, square 12 x 13 on 8 primes with one and eight rows a
+// warp took 7.3 and 18.9 ms (on whole rows, before degree windows, 6.0 and 12.3), now 3.8
+// and 8.9.
+template <int kFlight, bool V4>
 __device__ __forceinline__ void gather_edges(const GatherTask &t, uint32_t my, const EdgeWin &win, int n, uint32_t c,
-                                             int deg, bool active, long long *acc) {
-    for (int e = 0; e < n; e += 4) {
-        uint32_t q[4];
-        uint4 x[4];
+                                             int deg, int deg0, int deg1, bool active, long long *acc) {
+    uint32_t left = __ballot_sync(kFull, (int)(threadIdx.x & 31) < n && win.lo <= deg1 && win.hi > deg0);
+    while (left) {
+        uint32_t q[kFlight];
+        uint4 x[kFlight];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            q[j] = __shfl_sync(kFull, my, min(e + j, 31));
-            const int lo = __shfl_sync(kFull, win.lo, min(e + j, 31)), hi = __shfl_sync(kFull, win.hi, min(e + j, 31));
+        for (int j = 0; j < kFlight; ++j) {
+            const int e = left ? __ffs((int)left) - 1 : 0;
+            q[j] = __shfl_sync(kFull, my, e);
+            const int lo = __shfl_sync(kFull, win.lo, e), hi = __shfl_sync(kFull, win.hi, e);
             const uint32_t sh = edge_shift(q[j], t.src_bits);
-            x[j] = make_uint4(0, 0, 0, 0);
-            if (e + j < n && active && deg >= lo && deg < hi) {
-                const size_t off = (size_t)edge_src(q[j], t.src_bits) * t.C + (c - sh * t.cpd);
-                if (V4) x[j] = __ldg(reinterpret_cast<const uint4 *>(t.in) + off);
-                else x[j].x = __ldg(t.in + off);
-            }
+            const size_t off = (size_t)edge_src(q[j], t.src_bits) * t.C + (c - sh * t.cpd);
+            x[j] = load_if<V4>(t.in, off, left && active && deg >= lo && deg < hi ? 1u : 0u);
+            left &= left - 1;
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kFlight; ++j) {
             const long long cf = edge_coef(q[j], t.src_bits);  // absent edges loaded zero
             acc[0] += (long long)(int)x[j].x * cf;
             if (V4) {
@@ -89,8 +109,9 @@ __device__ __forceinline__ void gather_edges(const GatherTask &t, uint32_t my, c
 // window) and broadcast with shuffles; the lanes sweep the chunks of the row's
 // window 32 at a time.  The next row's CSR is fetched while the current row is
 // computed.
-template <int RPW, bool V4>
-__device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, const ModRed *s_mr, int dv, int first) {
+template <int kFlight, bool V4>
+__device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, int rpw, const ModRed *s_mr, int dv,
+                                            int first) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int dcap_in = first || t.first ? 0 : t.cap;
     uint32_t row = row0 + warp;
@@ -98,10 +119,10 @@ __device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, 
     uint32_t e0 = __shfl_sync(kFull, rp, 0), ne = __shfl_sync(kFull, rp, 1) - e0;
     uint2 my = (row < t.rows && lane < ne) ? __ldg(t.edges + e0 + lane) : make_uint2(0, 0);
 #pragma unroll 1
-    for (int k = 0; k < RPW; ++k) {
+    for (int k = 0; k < rpw; ++k) {
         if (row >= t.rows) return;
         const uint32_t nrow = row + kWarps;
-        uint32_t nrp = (k + 1 < RPW && nrow < t.rows && lane < 2) ? __ldg(t.row_ptr + nrow + lane) : 0;
+        uint32_t nrp = (k + 1 < rpw && nrow < t.rows && lane < 2) ? __ldg(t.row_ptr + nrow + lane) : 0;
         const uint32_t w = __ldg(t.win_out + row);
         const int lo = (int)(w & 0xffu);
         const int end = lo == 0xff ? 0 : min(t.cap, t.v_out + dv - (int)(w >> 8)) + 1;
@@ -112,14 +133,15 @@ __device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, 
             const uint32_t c = j + lane;
             const bool active = c < c_end;
             const uint32_t deg = fast_div(c, t.magic_cpd);
+            const int deg0 = (int)fast_div(j, t.magic_cpd), deg1 = (int)fast_div(min(j + 32, c_end) - 1, t.magic_cpd);
             const uint32_t pc = (c - deg * t.cpd) * (V4 ? 4 : 1);  // prime of the first word
             long long acc[4] = {modred_bias(s_mr[pc].p), V4 ? modred_bias(s_mr[pc + 1].p) : 0,
                                 V4 ? modred_bias(s_mr[pc + 2].p) : 0, V4 ? modred_bias(s_mr[pc + 3].p) : 0};
-            gather_edges<V4>(t, my.x, win, (int)min(ne, 32u), c, (int)deg, active, acc);
+            gather_edges<kFlight, V4>(t, my.x, win, (int)min(ne, 32u), c, (int)deg, deg0, deg1, active, acc);
             for (uint32_t eb = 32; eb < ne; eb += 32) {  // rows with more than 32 edges
                 const uint2 mb = (eb + lane < ne) ? __ldg(t.edges + e0 + eb + lane) : make_uint2(0, 0);
                 const EdgeWin wb = (eb + lane < ne) ? edge_window(t, mb, dcap_in, dv) : EdgeWin{0, 0};
-                gather_edges<V4>(t, mb.x, wb, (int)min(ne - eb, 32u), c, (int)deg, active, acc);
+                gather_edges<kFlight, V4>(t, mb.x, wb, (int)min(ne - eb, 32u), c, (int)deg, deg0, deg1, active, acc);
             }
             if (active) {
                 const size_t o = (size_t)row * t.C + c;
@@ -139,19 +161,19 @@ __device__ __forceinline__ void gather_rows(const GatherTask &t, uint32_t row0, 
     }
 }
 
-template <int RPW, int N>
+template <int kFlight, int N>
 __global__ void __launch_bounds__(kGatherThreads)
-    gather_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, int dv, int first) {
+    gather_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, int rpw, int dv, int first) {
     __shared__ ModRed s_mr[CP_MAX_PRIMES];
     const GatherTask &t = pack.t[find_task(pack, n_tasks, blockIdx.x)];
     if (threadIdx.x < t.n_primes) {
         s_mr[threadIdx.x] = modred_make(__ldg(t.primes + threadIdx.x));
     }
     __syncthreads();
-    // rows of the block: row0 + warp + 8 k, k < RPW
-    const uint32_t row0 = (blockIdx.x - t.block_begin) * (uint32_t)(kWarps * RPW);
-    if (t.vec4) gather_rows<RPW, true>(t, row0, s_mr, dv, first);
-    else gather_rows<RPW, false>(t, row0, s_mr, dv, first);
+    // rows of the block: row0 + warp + 8 k, k < rpw
+    const uint32_t row0 = (blockIdx.x - t.block_begin) * (uint32_t)(kWarps * rpw);
+    if (t.vec4) gather_rows<kFlight, true>(t, row0, rpw, s_mr, dv, first);
+    else gather_rows<kFlight, false>(t, row0, rpw, s_mr, dv, first);
 }
 
 bool tile_is_chunk(int items) { return (items & 0xFFF) >= 16; }
@@ -234,12 +256,20 @@ void append_gather_task(std::vector<GatherTask> *tasks, const SiteTable &tab, co
 
 int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, cudaStream_t st, int dv, bool first);
 
-template <int RPW>
-static int launch_gather_rows(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, cudaStream_t st, int dv,
+// Launches of up to three waves of resident blocks (two of them per SM with 98 registers,
+// 152 SMs) keep eight loads in flight instead of four: there the heaviest row's chain is
+// what they last.  Four and eight: square 12 x 12 on 8 primes, two rows a warp (499 blocks)
+// 4.60 and 3.87 ms, width 13, two rows (1332 blocks) 1.64 and 1.67, one row (2664) 1.35 and
+// 1.71; short rows of one-factor tables lose 3 to 10% below the line.
+constexpr uint32_t kFewBlocks = 3 * 2 * 152;
+
+static int launch_gather_rows(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, int rpw, cudaStream_t st, int dv,
                               bool first) {
     return for_packs(tasks, n_tasks, total_blocks, [&](const auto &pack, int n, uint32_t blocks) -> int {
         constexpr int N = sizeof(pack.t) / sizeof(GatherTask);
-        if (blocks) gather_kernel<RPW, N><<<blocks, kGatherThreads, 0, st>>>(pack, n, dv, first ? 1 : 0);
+        if (!blocks) return CP_OK;
+        if (blocks <= kFewBlocks) gather_kernel<8, N><<<blocks, kGatherThreads, 0, st>>>(pack, n, rpw, dv, first ? 1 : 0);
+        else gather_kernel<4, N><<<blocks, kGatherThreads, 0, st>>>(pack, n, rpw, dv, first ? 1 : 0);
         CP_CUDA_TRY(cudaGetLastError());
         return CP_OK;
     });
@@ -249,13 +279,10 @@ int launch_gather(const GatherTask *tasks, int n_tasks, uint32_t total_blocks, i
                   bool first) {
     if (n_tasks <= 0 || total_blocks == 0) return CP_OK;
     if (tile_is_chunk(items)) return launch_gather_chunk(tasks, n_tasks, total_blocks, st, dv, first);
-    switch (items & 0xFFF) {
-        case 1: return launch_gather_rows<1>(tasks, n_tasks, total_blocks, st, dv, first);
-        case 2: return launch_gather_rows<2>(tasks, n_tasks, total_blocks, st, dv, first);
-        case 4: return launch_gather_rows<4>(tasks, n_tasks, total_blocks, st, dv, first);
-        case 8: return launch_gather_rows<8>(tasks, n_tasks, total_blocks, st, dv, first);
-    }
-    return fail(CP_EINVAL, "gather tile must be 1, 2, 4, 8, 16, 32, 64 or 128");
+    const int rpw = items & 0xFFF;
+    if (rpw != 1 && rpw != 2 && rpw != 4 && rpw != 8)
+        return fail(CP_EINVAL, "gather tile must be 1, 2, 4, 8, 16, 32, 64 or 128");
+    return launch_gather_rows(tasks, n_tasks, total_blocks, rpw, st, dv, first);
 }
 
 int prepare_gather_kernels() {

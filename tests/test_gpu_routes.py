@@ -125,3 +125,18 @@ def test_small_primes_are_no_slow_case(lattice):
     # the same kernel with a longer reduction (the register kernel took 11 times as long here)
     big, small = gpu_util.seed_primes(8, seed=44), primes_from(1000003, 8)
     assert solve_ms(lattice, 12, 13, small) < 2.5 * solve_ms(lattice, 12, 13, big)
+
+
+# both depths of the register kernel (launches of fewer and of more blocks), whole and padded prime lanes
+@pytest.mark.parametrize("tile", [1, 2, 4, 8])
+@pytest.mark.parametrize("lattice", ["square", "triangular"])
+def test_register_tiles_agree(lattice, tile):
+    for L, N, D, P in ((13, 4, 40, 1), (13, 4, -1, 8), (11, 5, -1, 20), (7, 8, 30, 5)):
+        primes = gpu_util.seed_primes(P, seed=45)
+        assert np.array_equal(solve(lattice, L, N, primes, D=D, tile=tile), solve(lattice, L, N, primes, D=D)), (L, P)
+
+
+@pytest.mark.parametrize("tile,ms", [(1, 6.0), (2, 7.5), (4, 9.6), (8, 12.3)])
+def test_register_tiles_keep_their_speed(tile, ms):
+    # ms: what the tile took on whole rows, before degree windows
+    assert solve_ms("square", 12, 13, gpu_util.seed_primes(8, seed=46), tile=tile) < ms
