@@ -56,9 +56,14 @@ typedef struct cp_strip cp_strip;
  * cp_create_strip -- a strip of width L, height 1, state vector = e_0.
  * Builds (or reuses from the per-device cache) the rank tables and the CSR
  * tables of every per-site factor T_i and T_i^last on the GPU, and allocates
- * the two state vectors [S][D+1][n_primes, rounded up to a multiple of four where
- * that fits] (S = M_{L-1} + M_{L-2} on the
+ * the two state vectors [S][D+1][n_primes] (S = M_{L-1} + M_{L-2} on the
  * square lattice, M_{L-1} on the triangular one; Sec. 3.2-3.3).
+ * Memory: n_primes is rounded up to a multiple of four there (one prime takes the
+ * memory of four), as the faster gather kernel reads four primes at a time, unless that
+ * does not fit: all strips and sweeps on a device together spend at most an eighth of
+ * its memory on the added lanes, and those beyond have rows of their primes alone
+ * (slower, same results).  The tables take 8 bytes per transition (12 while they are
+ * built) and stay cached until cp_clear_table_cache.
  *   lattice    CP_SQUARE or CP_TRIANGULAR
  *   L          1..CP_MAX_L sites per row (strip width m of the paper)
  *   primes_host, n_primes   1..CP_MAX_PRIMES distinct primes < 2^31 (copied)

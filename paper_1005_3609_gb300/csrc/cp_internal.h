@@ -344,4 +344,22 @@ int crt_static_touch();
 int dev_alloc(void **p, size_t bytes);
 void dev_free(void *p);
 
+// What an object's padding lanes take beyond the rows of its primes alone.  The lanes of
+// all objects on a device together get at most 1 / kPadFraction of its memory, so that
+// strips of one prime, four times as large with them, still leave room for the next ones;
+// an object whose lanes do not fit in that has rows of its primes alone (the register
+// kernel; results are the same).  Given back with the object.
+constexpr size_t kPadFraction = 8;
+class PadShare {
+    int dev_ = -1;
+    size_t bytes_ = 0;
+
+  public:
+    PadShare() = default;
+    PadShare(const PadShare &) = delete;
+    PadShare &operator=(const PadShare &) = delete;
+    ~PadShare();
+    bool take(size_t bytes);  // on the current device, in addition to what it holds
+};
+
 }  // namespace cp

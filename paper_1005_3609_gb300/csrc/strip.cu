@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -34,6 +35,31 @@ int dev_alloc(void **p, size_t bytes) {
 
 void dev_free(void *p) {
     if (p) cudaFree(p);
+}
+
+static std::mutex g_pad_mu;
+static size_t g_pad_used[64], g_pad_limit[64];  // per device
+
+bool PadShare::take(size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || (dev_ >= 0 && dev_ != dev)) return false;
+    std::lock_guard<std::mutex> lk(g_pad_mu);
+    if (!g_pad_limit[dev]) {
+        size_t free_bytes = 0, total = 0;
+        if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) return false;
+        g_pad_limit[dev] = total / kPadFraction;
+    }
+    if (bytes > g_pad_limit[dev] - g_pad_used[dev]) return false;
+    g_pad_used[dev] += bytes;
+    dev_ = dev;
+    bytes_ += bytes;
+    return true;
+}
+
+PadShare::~PadShare() {
+    if (dev_ < 0) return;
+    std::lock_guard<std::mutex> lk(g_pad_mu);
+    g_pad_used[dev_] -= bytes_;
 }
 
 // Deterministic Miller-Rabin for n < 2^32 (bases 2, 7, 61).
@@ -99,6 +125,7 @@ struct cp_strip {
     };
     std::vector<Launch> row_l[2], last_l[2];
     const uint32_t *last_result[2] = {nullptr, nullptr};
+    PadShare pad;
 
     ~cp_strip() {
         dev_free(primes_dev);
@@ -160,10 +187,12 @@ static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const 
     const uint32_t min_prime = *std::min_element(primes, primes + n_primes);
     if ((rc = dev_alloc((void **)&s->primes_dev, sizeof(block)))) return rc;
     CP_CUDA_TRY(cudaMemcpy(s->primes_dev, block, sizeof(block), cudaMemcpyHostToDevice));
-    for (int k = 0; k < 2; ++k)
-        if ((rc = dev_alloc((void **)&s->vec[k], ts.S_max * row_words * 4))) return rc;
     // read-out scratch: T_1^last writes cnt[L-1] rows, T_2^last cnt[L-2], ...
     uint64_t sA = ts.last[0].n_dst, sB = ts.last.size() >= 2 ? ts.last[1].n_dst : 1;
+    if (Pp != n_primes && !s->pad.take((2 * ts.S_max + sA + sB) * s->D1 * (Pp - n_primes) * 4))
+        return fail(CP_ENOMEM, "the padding lanes' share of the device memory is taken");
+    for (int k = 0; k < 2; ++k)
+        if ((rc = dev_alloc((void **)&s->vec[k], ts.S_max * row_words * 4))) return rc;
     if ((rc = dev_alloc((void **)&s->scratch[0], sA * row_words * 4))) return rc;
     if ((rc = dev_alloc((void **)&s->scratch[1], sB * row_words * 4))) return rc;
     if ((rc = dev_alloc((void **)&s->row_out, row_words * 4))) return rc;
@@ -204,8 +233,8 @@ static int make_strip(std::shared_ptr<TableSet> tabs, int lattice, int L, const 
     return CP_OK;
 }
 
-// Rows padded to 16-byte chunks (the chunk kernel); where the vectors do not fit
-// that way, rows of the given primes alone (the register kernel).
+// Rows padded to 16-byte chunks (the chunk kernel); where the vectors or the padding's
+// share (PadShare) do not fit that way, rows of the given primes alone (the register kernel).
 static int make_strip_padded(std::shared_ptr<TableSet> tabs, int lattice, int L, const uint32_t *primes, int n_primes,
                              int max_degree, int max_rows, void *cuda_stream, cp_strip **out) {
     const int Pp = padded_primes(n_primes);

@@ -72,6 +72,7 @@ struct cp_sweep {
     uint64_t updates = 0, bytes = 0, site_bytes = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    PadShare pad;
 
     ~cp_sweep() {
         if (exec) cudaGraphExecDestroy(exec);
@@ -130,9 +131,11 @@ static int build_strips(cp_sweep *sw) {
             const TableSet &ts = *st.tabs;
             sw->strips.push_back(st);
             SweepStrip &sp = sw->strips.back();
+            uint64_t sA = ts.last[0].n_dst, sB = ts.last.size() >= 2 ? ts.last[1].n_dst : 1;
+            if (sw->Pp != Pg && !sw->pad.take((2 * ts.S_max + sA + sB) * sw->D1 * (sw->Pp - Pg) * 4))
+                return fail(CP_ENOMEM, "the padding lanes' share of the device memory is taken");
             for (int b = 0; b < 2; ++b)
                 if ((rc = dev_alloc((void **)&sp.vec[b], ts.S_max * row_words * 4))) return rc;
-            uint64_t sA = ts.last[0].n_dst, sB = ts.last.size() >= 2 ? ts.last[1].n_dst : 1;
             if ((rc = dev_alloc((void **)&sp.scratch[0], sA * row_words * 4))) return rc;
             if ((rc = dev_alloc((void **)&sp.scratch[1], sB * row_words * 4))) return rc;
         }
@@ -268,8 +271,8 @@ static std::vector<uint32_t> prime_blocks(const cp_sweep *sw) {
 static int sweep_build_lanes(int lattice, int k, const uint32_t *primes, int P, int tile, int groups, int Pp,
                              cudaStream_t stream, cp_sweep **out);
 
-// Rows padded to 16-byte chunks (the chunk kernel); where the vectors do not fit that way, rows of
-// the given primes alone (the register kernel).
+// Rows padded to 16-byte chunks (the chunk kernel); where the vectors or the padding's share
+// (PadShare) do not fit that way, rows of the given primes alone (the register kernel).
 static int sweep_build(int lattice, int k, const uint32_t *primes, int P, int tile, int groups, cudaStream_t stream,
                        cp_sweep **out) {
     const int Pg = P / groups, Pp = padded_primes(Pg);

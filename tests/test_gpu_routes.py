@@ -140,3 +140,92 @@ def test_register_tiles_agree(lattice, tile):
 def test_register_tiles_keep_their_speed(tile, ms):
     # ms: what the tile took on whole rows, before degree windows
     assert solve_ms("square", 12, 13, gpu_util.seed_primes(8, seed=46), tile=tile) < ms
+
+
+def gb_used():
+    import torch
+    free, total = torch.cuda.mem_get_info()
+    return (total - free) / 1e9
+
+
+STATES_12 = 2 * 7986 + 835 + 127  # square width 12, two-site tables: two vectors and the read-out's two
+
+
+def lane_gb(D):
+    """Memory of one prime lane of a square width-12 strip's vectors."""
+    return STATES_12 * (D + 1) * 4 / 1e9
+
+
+class Padding:
+    """Two strips of one prime whose padding lanes take all but a thousandth of the share that padding may have."""
+
+    def __enter__(self):
+        import torch
+        prime = gpu_util.seed_primes(1, seed=48)
+        share = torch.cuda.mem_get_info()[1] / 8
+        self.D = int(0.4995 * share / (3 * lane_gb(0) * 1e9)) - 1
+        self.strips = [cp.Strip("square", 12, prime, max_degree=self.D, max_rows=3) for _ in range(2)]
+        return self
+
+    def __exit__(self, *a):
+        for s in self.strips:
+            s.close()
+
+
+def test_padding_lanes_leave_room_for_other_strips():
+    primes = gpu_util.seed_primes(3, seed=48)
+    want = solve("square", 12, 3, primes[:1])[0].tolist()
+    with Padding() as pad:
+        D, lane = pad.D, lane_gb(pad.D)
+        for n, lanes in ((1, 1), (3, 3)):  # the share is taken: their primes alone
+            before = gb_used()
+            with cp.Strip("square", 12, primes[:n], max_degree=D, max_rows=3) as s:
+                assert abs(gb_used() - before - lanes * lane) < 0.1 * lane
+                s.advance(2)
+                got = s.read()[0]
+                assert got[:len(want)].tolist() == want and not got[len(want):].any()
+        pad.strips.pop().close()
+        before = gb_used()
+        with cp.Strip("square", 12, primes[:1], max_degree=D, max_rows=3):  # given back: four lanes again
+            assert abs(gb_used() - before - 4 * lane) < 0.1 * lane
+
+
+@pytest.mark.parametrize("lattice,n_primes,groups", [("square", 5, 1), ("triangular", 2, 2), ("square", 1, 0)])
+def test_sweeps_of_unpadded_rows(lattice, n_primes, groups):
+    import torch
+    primes, stream, out = gpu_util.seed_primes(n_primes, seed=49), torch.cuda.Stream(), []
+
+    def sweep(k):
+        before = gb_used()
+        with cp.Sweep(lattice, k, primes, stream, prime_groups=groups) as sw:
+            used = gb_used() - before
+            sw.run()
+            return used, sw.read_series(), sw.read_ptilde()
+
+    sweep(31)  # (tables and kernels are there)
+    padded = sweep(31)
+    with Padding():
+        alone = sweep(31)
+    Pg = n_primes // max(groups, 1)
+    assert alone[0] < padded[0] * (Pg / (Pg + 3 & ~3) + 0.15)
+    assert np.array_equal(padded[1], alone[1])
+    assert padded[2].keys() == alone[2].keys() and all(np.array_equal(padded[2][x], alone[2][x]) for x in padded[2])
+
+
+def test_rows_of_the_primes_alone_where_padded_ones_do_not_fit():
+    import torch
+    primes, D = gpu_util.seed_primes(5, seed=50), 13000
+    want = solve("square", 12, 4, primes, D=60)
+    torch.cuda.empty_cache()
+    lane = lane_gb(D)
+    hold = torch.empty(int((torch.cuda.mem_get_info()[0] / 1e9 - 6.5 * lane) * 1e9), dtype=torch.uint8, device="cuda")
+    try:
+        before = gb_used()
+        with cp.Strip("square", 12, primes, max_degree=D, max_rows=4) as s:
+            assert abs(gb_used() - before - 5 * lane) < 0.2 * lane
+            s.advance(3)
+            got = s.read()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(got[:, :61], want) and not got[:, 61:].any()
