@@ -427,20 +427,32 @@ int cp_debug_check_space(int kind, int m, int e, uint64_t *n_bad, uint64_t *size
  * timeout path without faulting or hanging the GPU. */
 int cp_debug_wait_timeout(long long cycles);
 
-/* The modular reduction of the gather kernels (Sec. 3.5: arithmetic modulo
+/* The modular reduction of the register gather (Sec. 3.5: arithmetic modulo
  * primes below 2^31), run on the GPU on given values: out_host[k] =
- * v_host[k] mod p_host[k] in [0, p), computed exactly as the kernels reduce an
- * accumulator (integer Barrett step from the bias p 2^21, see the kernels'
+ * v_host[k] mod p_host[k] in [0, p), computed exactly as the kernel reduces an
+ * accumulator (integer Barrett step from the bias p 2^21, see the kernel's
  * source).  Requires 2 <= p_host[k] < 2^31 and |v_host[k]| < p_host[k] * 2^20
  * (the bound the table build enforces on every destination); CP_EINVAL
  * otherwise.  Synchronous. */
 int cp_debug_reduce(const int64_t *v_host, const uint32_t *p_host, int n, uint32_t *out_host);
 
+/* The sums and reductions of the chunk gather (Sec. 3.5), run on the GPU on given
+ * values: out_host[k] in [-p, p) is congruent to sum_e coefs_host[k*n_edges + e] *
+ * words_host[k*n_edges + e] modulo p = p_host[k], by the 32-bit reduction or, with
+ * any_prime, by the one for every prime.  s_host[k]: the bound on the sum of
+ * |coefficient| that the kernel's offset is chosen for.  Requires |coefficient| <= 127,
+ * sum of |coefficient| <= s_host[k] < 2^15, |word| <= p, 2 <= p < 2^31 and, without
+ * any_prime, s and p within the 32-bit reduction's bound (5 s 2^15 + 2^16 + (s + 2)
+ * p / 2^17 + 2 < p, s <= 8192); CP_EINVAL otherwise.  A diagnostic (it allocates device
+ * buffers).  Synchronous. */
+int cp_debug_chunk_sum(const int32_t *coefs_host, const int32_t *words_host, int n_edges, const uint32_t *s_host,
+                       const uint32_t *p_host, int n, int any_prime, int32_t *out_host);
+
 /* A 32-bit reduction (Sec. 3.5) of a word's sum kept as two 32-bit halves, u =
- * hi_host[k] 2^16 + lo_host[k], for primes of at least 2^17:
+ * hi_host[k] 2^16 + lo_host[k], for primes of at least 2^17 (of its own: the gathers'
+ * are cp_debug_chunk_sum's and cp_debug_reduce's):
  * out_host[k] = u mod p_host[k] in [0, p) when full != 0,
- * else (u mod p) or (u mod p) - p, a signed representative in [-p, p), as the
- * gathers store.  Requires
+ * else (u mod p) or (u mod p) - p, a signed representative in [-p, p).  Requires
  * 2^17 <= p_host[k] < 2^31 and 0 < u < p_host[k] 2^16; CP_EINVAL otherwise.
  * A diagnostic (it allocates device buffers).  Synchronous. */
 int cp_debug_reduce_halves(const int32_t *lo_host, const int32_t *hi_host, const uint32_t *p_host, int n, int full,

@@ -76,6 +76,8 @@ SIGNATURES = {
     "cp_debug_table": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, u32p,
                                       ctypes.c_uint64, u32p, ctypes.c_uint64, u64p]),
     "cp_debug_reduce": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int64), u32p, ctypes.c_int, u32p]),
+    "cp_debug_chunk_sum": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32), ctypes.c_int,
+                                          u32p, u32p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int32)]),
     "cp_debug_reduce_halves": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32), u32p,
                                               ctypes.c_int, ctypes.c_int, u32p]),
     "cp_server_stats": (ctypes.c_int, [vp, u64p, u64p, u64p, ctypes.POINTER(ctypes.c_size_t)]),
@@ -316,6 +318,20 @@ def debug_reduce(values, primes):
     check("cp_debug_reduce", load().cp_debug_reduce(v.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), pp, len(v),
                                                     out.ctypes.data_as(u32p)))
     return [int(x) for x in out]
+
+
+def debug_chunk_sum(coefs, words, bounds, primes, any_prime=False):
+    """The chunk gather's sums of coefs[k][e] * words[k][e] and their reduction modulo
+    primes[k] on the GPU, as signed representatives in [-p, p) (cp_debug_chunk_sum)."""
+    c = np.ascontiguousarray(np.asarray(coefs, dtype=np.int32))
+    x = np.ascontiguousarray(np.asarray(words, dtype=np.int32))
+    s, sp = _u32(bounds)
+    p, pp = _u32(primes)
+    out = np.zeros(len(p), dtype=np.int32)
+    i32p = ctypes.POINTER(ctypes.c_int32)
+    check("cp_debug_chunk_sum", load().cp_debug_chunk_sum(c.ctypes.data_as(i32p), x.ctypes.data_as(i32p), c.shape[1], sp,
+                                                          pp, len(p), 1 if any_prime else 0, out.ctypes.data_as(i32p)))
+    return [int(v) for v in out]
 
 
 def debug_reduce_halves(lo, hi, primes, full=True):

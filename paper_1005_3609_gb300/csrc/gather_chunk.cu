@@ -444,7 +444,66 @@ int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, 
 
 }  // namespace cp
 
-// Diagnostic: a 32-bit reduction of two-halves sums on given values (one thread per value).
+// Diagnostic: the kernel's sums and reductions on given values (one thread per value).
+namespace cp {
+__global__ void debug_chunk_sum_kernel(const int *coefs, const int *words, int n_edges, const uint32_t *s,
+                                       const uint32_t *pr, int n, int any_prime, int *out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const uint32_t p = pr[k], k0 = fast_offset(s[k]), t = chunk_shift(p);
+    const uint32_t m = (uint32_t)((1ull << (32 + t)) / p);  // chunk_magic
+    Acc2 a{0u, -(int)k0};
+    for (int e = 0; e < n_edges; ++e) {
+        const size_t i = (size_t)k * n_edges + e;
+        add_word(a, (uint32_t)words[i], coefs[i], (uint32_t)coefs[i] << 24);
+    }
+    out[k] = (int)(any_prime ? any_reduce(a, k0, p, m, t) : fast_reduce(a, p, m));
+}
+}  // namespace cp
+
+extern "C" int cp_debug_chunk_sum(const int32_t *coefs_host, const int32_t *words_host, int n_edges,
+                                  const uint32_t *s_host, const uint32_t *p_host, int n, int any_prime,
+                                  int32_t *out_host) {
+    using namespace cp;
+    if (n < 0 || n_edges < 0 || (n > 0 && (!coefs_host || !words_host || !s_host || !p_host || !out_host)))
+        return fail(CP_EINVAL, "bad arguments");
+    for (int k = 0; k < n; ++k) {
+        const uint32_t p = p_host[k];
+        if (p < 2 || p >= (1u << 31)) return fail(CP_EINVAL, "p must be in [2, 2^31)");
+        if (s_host[k] >= kChunkMaxSum || (!any_prime && !fast_ok(s_host[k], p)))
+            return fail(CP_EINVAL, "the coefficient sum's bound does not suit the reduction");
+        uint64_t sum = 0;
+        for (int e = 0; e < n_edges; ++e) {
+            const long long c = coefs_host[(size_t)k * n_edges + e], x = words_host[(size_t)k * n_edges + e];
+            if (c < -(int)kChunkMaxCoef || c > (int)kChunkMaxCoef) return fail(CP_EINVAL, "|coefficient| must be at most 127");
+            if (x < -(long long)p || x > (long long)p) return fail(CP_EINVAL, "|word| must be at most p");
+            sum += (uint64_t)(c < 0 ? -c : c);
+        }
+        if (sum > s_host[k]) return fail(CP_EINVAL, "sum of |coefficient| exceeds its bound");
+    }
+    if (n == 0) return CP_OK;
+    const size_t words = (size_t)n * n_edges;
+    uint32_t *d = nullptr;  // coefficients, words, bounds, primes, results
+    int rc = dev_alloc((void **)&d, 4 * (2 * words + 3 * (size_t)n));
+    if (rc) return rc;
+    int *c_d = (int *)d, *x_d = c_d + words, *o_d = x_d + words;
+    uint32_t *s_d = (uint32_t *)(o_d + n), *p_d = s_d + n;
+    cudaError_t e = cudaMemcpy(c_d, coefs_host, 4 * words, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(x_d, words_host, 4 * words, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(s_d, s_host, 4ull * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(p_d, p_host, 4ull * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        debug_chunk_sum_kernel<<<(n + 255) / 256, 256>>>(c_d, x_d, n_edges, s_d, p_d, n, any_prime, o_d);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(out_host, o_d, 4ull * n, cudaMemcpyDeviceToHost);
+    dev_free(d);
+    if (e != cudaSuccess) return fail(CP_ECUDA, std::string("cp_debug_chunk_sum: ") + cudaGetErrorString(e));
+    return CP_OK;
+}
+
+// Diagnostic: a 32-bit reduction of two-halves sums on given values (one thread per
+// value), for an entry point alone: no gather uses it.
 namespace cp {
 // For primes p >= 2^17 the sums start at B = p 2^15 (a multiple of p above
 // |sum c x| <= S p), so u = hi 2^16 + lo lies in (0, p 2^16), and the quotient
