@@ -123,14 +123,18 @@ __device__ __forceinline__ bool nn_ok(const Labels &s, int m, int skip) {
     return (adjacent_pairs(s, m) & ~(skip >= 0 ? 1u << skip : 0u)) == 0;
 }
 
+// The parts of a partition that a ranking (unranking) puts off are disjoint, with a point
+// of a block before each, so kMaxL / 2 entries hold those of an NCNNN partition, whose
+// parts have a point at least; ranks are below 2^32 (M_19, Catalan(16)).
+
 // Rank of an NCNNN partition of the points lo..hi-1 in the paper's order
 // (Sec. 3.4): a point alone first (rank of the rest), then by the smallest
 // partner lo+2+k of point lo, inner points as the most significant digit and
 // the right part (from the partner on) as the least significant one.
 // Returns ~0ull if the partition violates the neighbour rule at the first point.
 __device__ __forceinline__ uint64_t ncnnn_rank(const Labels &s, int lo, int hi, const RankTables &T) {
-    int sa[kMaxL + 1], sb[kMaxL + 1];
-    uint64_t smul[kMaxL + 1];
+    uint8_t sa[kMaxL / 2], sb[kMaxL / 2];
+    uint32_t smul[kMaxL / 2];
     int sp = 0;
     uint64_t r = 0;
     int a = lo, b = hi;
@@ -144,7 +148,7 @@ __device__ __forceinline__ uint64_t ncnnn_rank(const Labels &s, int lo, int hi, 
             int k = j - a - 2;
             uint64_t cr = T.cnt[b - j];
             r += mu * T.off[n * kTblStride + k];
-            sa[sp] = a + 1; sb[sp] = j; smul[sp] = mu * cr; ++sp;   // inner part, later
+            sa[sp] = (uint8_t)(a + 1); sb[sp] = (uint8_t)j; smul[sp] = (uint32_t)(mu * cr); ++sp;   // inner part, later
             a = j;                                                   // right part, now
         }
         if (b - a == 2 && s.v[a] == s.v[a + 1]) return ~0ull;
@@ -161,8 +165,8 @@ __device__ __forceinline__ void ncnnn_unrank(uint64_t r, int lo, int hi, Labels 
 #pragma unroll
     for (int k = 0; k < kMaxL / 4; ++k) s.w[k] = ~0u;
     uint8_t next = 0;
-    int sa[kMaxL + 1], sb[kMaxL + 1];
-    uint64_t sr[kMaxL + 1];
+    uint8_t sa[kMaxL / 2], sb[kMaxL / 2];
+    uint32_t sr[kMaxL / 2];
     int sp = 0;
     int a = lo, b = hi;
     for (;;) {
@@ -181,7 +185,7 @@ __device__ __forceinline__ void ncnnn_unrank(uint64_t r, int lo, int hi, Labels 
             uint64_t inner = r / cr, right = r - inner * cr;
             int j = a + 2 + k;
             s.v[j] = s.v[a];
-            sa[sp] = j; sb[sp] = b; sr[sp] = right; ++sp;   // right part after the inner one
+            sa[sp] = (uint8_t)j; sb[sp] = (uint8_t)b; sr[sp] = (uint32_t)right; ++sp;   // right part after the inner one
             a = a + 1; b = j; r = inner;
         }
         if (sp == 0) break;
@@ -195,8 +199,8 @@ __device__ __forceinline__ void ncnnn_unrank(uint64_t r, int lo, int hi, Labels 
 // as the most significant digit and the right part (from the partner on) as
 // the least significant one.  The count recursion is Catalan's.
 __device__ __forceinline__ uint64_t nc_rank(const Labels &s, int lo, int hi, const RankTables &T) {
-    int sa[kMaxL + 1], sb[kMaxL + 1];
-    uint64_t smul[kMaxL + 1];
+    uint8_t sa[kMaxL + 1], sb[kMaxL + 1];
+    uint32_t smul[kMaxL + 1];
     int sp = 0;
     uint64_t r = 0;
     int a = lo, b = hi;
@@ -207,7 +211,7 @@ __device__ __forceinline__ uint64_t nc_rank(const Labels &s, int lo, int hi, con
             if (j < 0) { ++a; continue; }
             int k = j - a - 1;
             r += mu * T.offc[n * kTblStride + k];
-            sa[sp] = a + 1; sb[sp] = j; smul[sp] = mu * T.cntc[b - j]; ++sp;  // inner part, later
+            sa[sp] = (uint8_t)(a + 1); sb[sp] = (uint8_t)j; smul[sp] = (uint32_t)(mu * T.cntc[b - j]); ++sp;  // inner part, later
             a = j;                                                              // right part, now
         }
         if (sp == 0) break;
@@ -221,8 +225,8 @@ __device__ __forceinline__ void nc_unrank(uint64_t r, int lo, int hi, Labels &s,
 #pragma unroll
     for (int k = 0; k < kMaxL / 4; ++k) s.w[k] = ~0u;
     uint8_t next = 0;
-    int sa[kMaxL + 1], sb[kMaxL + 1];
-    uint64_t sr[kMaxL + 1];
+    uint8_t sa[kMaxL + 1], sb[kMaxL + 1];
+    uint32_t sr[kMaxL + 1];
     int sp = 0;
     int a = lo, b = hi;
     for (;;) {
@@ -238,7 +242,7 @@ __device__ __forceinline__ void nc_unrank(uint64_t r, int lo, int hi, Labels &s,
             uint64_t inner = r / cr, right = r - inner * cr;
             int j = a + 1 + k;
             s.v[j] = s.v[a];
-            sa[sp] = j; sb[sp] = b; sr[sp] = right; ++sp;  // right part after the inner one
+            sa[sp] = (uint8_t)j; sb[sp] = (uint8_t)b; sr[sp] = (uint32_t)right; ++sp;  // right part after the inner one
             a = a + 1; b = j; r = inner;
         }
         if (sp == 0) break;

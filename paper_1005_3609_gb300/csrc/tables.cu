@@ -261,68 +261,85 @@ __global__ void build_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *sl
 
 // A two-site table, the second factor applied to every term of the first: LANES threads
 // per source state, each for every LANES-th term of the first factor, which meet in
-// shared memory to merge equal (dst, shift).  Bound by unranking, relabelling and ranking
-// in local memory: one thread per source took 170 us a table at width 12 (5 798 states),
-// eight 95 us, and with the labels as words 85 us (four lanes or a warp per source: the
-// cold tables of that width 2.91 or 2.71 ms against 2.55); a table that fills the SMs
-// anyway takes two (eight repeat too much of the first factor: width 14 8.4 against 5.6 ms).
-template <int LANES>
+// shared memory to merge equal (dst, shift).  A source has at most 14 terms before that
+// on the square lattice (8 a lane of two) and 23 on the triangular one (15 a lane of
+// two), at every width, as a factor changes little beyond the sites beside its own; a
+// lane has room for kLane, and the build fails if one needs more.  Bound by unranking,
+// relabelling and ranking in local memory: one thread per source took 170 us a table at
+// width 12 (5 798 states), eight 95 us, and with the labels as words 85 us (four lanes or
+// a warp per source: the cold tables of that width 2.91 or 2.71 ms against 2.55).  Tables
+// that fill the SMs anyway take fewer lanes, as each repeats the first factor, and live
+// on the L1 that the shared slots leave to local memory: cold tables (without padding
+// slots to 64 a source, and with small stacks in the ranking), square width 17 two lanes
+// 56.1 ms (64 slots 61.6, one lane 60.2), triangular width 14 two lanes 5.6 (one 6.1),
+// width 16 one 15.9 (two 17.3), width 18 one 107.8 (two 130.9, 64 slots 175).
+template <int LANES, int kLane>
 __global__ void __launch_bounds__(128)
     build_fused_terms_kernel(OpDesc op, const RankTables *Tg, uint32_t *slot_dst, uint32_t *slot_edge, int K, int *err) {
-    constexpr int kSources = 128 / LANES, kAll = kMaxTerms * kMaxTerms;
+    constexpr int kSources = 128 / LANES, kAll = LANES * kLane;
     __shared__ RankTables T;
-    __shared__ uint32_t s_dst[kSources][kAll + 1];
-    __shared__ int s_term[kSources][kAll + 1];  // coefficient << 4 | shift
+    __shared__ uint32_t s_key[kSources][kAll + 1];  // destination << 3 | shift
+    __shared__ int s_coef[kSources][kAll + 1];
     stage_tables(T, Tg);
     const int grp = threadIdx.x / LANES, lane = threadIdx.x % LANES;
     const uint64_t src = (uint64_t)blockIdx.x * kSources + grp;
     const bool have = src < op.in.size;
-    uint32_t *dst = s_dst[grp];
-    int *term = s_term[grp];
-    int bad = 0, all = 0;  // all: end of the slots in use
-    for (int k = lane; k < kAll; k += LANES) dst[k] = ~0u;
-    __syncwarp();
+    uint32_t *key = s_key[grp];
+    int *coef = s_coef[grp];
+    int bad = 0, mine = 0;  // mine: this lane's terms, the first of its kLane slots
     if (have) {
         Labels s;
         space_unrank(src, op.in, s, T);
         if (lane == 0 && (!space_contains(s, op.in) || space_rank(s, op.in, T) != src)) bad |= 8;
         Term a[kMaxTerms], t[kMaxTerms];
         const int na = factor_terms(op, s, a);
-        all = na * kMaxTerms;
         OpDesc ob = op;
         ob.kind = op.kind_b;
         ob.i = op.i_b;
         for (int j = lane; j < na; j += LANES) {
             const int n = factor_terms(ob, a[j].s, t);
             for (int q = 0; q < n; ++q) {
-                dst[j * kMaxTerms + q] = term_dst(t[q].s, op.out, T, &bad);
-                term[j * kMaxTerms + q] = ((t[q].coef * a[j].coef) << 4) | (t[q].shift + a[j].shift);
+                const uint32_t d = term_dst(t[q].s, op.out, T, &bad);
+                if (d == ~0u) continue;
+                if (mine == kLane) {
+                    bad |= 2;
+                    break;
+                }
+                const int k = lane * kLane + mine++;
+                key[k] = d << 3 | (uint32_t)(t[q].shift + a[j].shift);
+                coef[k] = t[q].coef * a[j].coef;
             }
         }
     }
+    int end[LANES];  // end of each lane's terms
+#pragma unroll
+    for (int l = 0; l < LANES; ++l) end[l] = l * kLane + __shfl_sync(0xffffffffu, mine, l, LANES);
     __syncwarp();
     // of equal (dst, shift) the first stands for them all with the sum of their
     // coefficients; the slots are the lanes' terms one after another, counted, then written
     int w = 0;
-    uint32_t keep = ~0u;  // of this lane's slots, one bit each
-    static_assert(kAll / LANES <= 32, "a bit per slot of a lane");
+    uint32_t keep = ~0u;  // of this lane's terms, one bit each
+    static_assert(kLane <= 32, "a bit per slot of a lane");
     for (int round = 0; round < 2; ++round) {
         int c = 0;
-        for (int k = lane; k < all; k += LANES) {
-            const uint32_t d = dst[k];
-            if (d == ~0u || !(keep >> (k / LANES) & 1u)) continue;
-            const int x = term[k];
-            int coef = x >> 4;
-            for (int m = k + 1; m < all; ++m)
-                if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef += term[m] >> 4;
-            if (round == 0)
-                for (int m = 0; m < k; ++m)
-                    if (dst[m] == d && ((term[m] ^ x) & 15) == 0) coef = 0;
-            if (coef == 0) {
-                keep &= ~(1u << (k / LANES));
+        for (int i = 0; i < mine; ++i) {
+            if (!(keep >> i & 1u)) continue;
+            const int k = lane * kLane + i;
+            const uint32_t x = key[k];
+            int sum = 0;
+            bool first = true;
+#pragma unroll
+            for (int l = 0; l < LANES; ++l)
+                for (int m = l * kLane; m < end[l]; ++m)
+                    if (key[m] == x) {
+                        sum += coef[m];
+                        first = first && m >= k;
+                    }
+            if (!first || sum == 0) {
+                keep &= ~(1u << i);
                 continue;
             }
-            if (round) put_term(op, src, d, coef, x & 15, w + c, K, slot_dst, slot_edge, &bad);
+            if (round) put_term(op, src, x >> 3, sum, (int)(x & 7u), w + c, K, slot_dst, slot_edge, &bad);
             ++c;
         }
         if (round) break;
@@ -696,7 +713,8 @@ __global__ void pack_units_kernel(const uint32_t *row_ptr, uint64_t n, uint32_t 
     if (!units) cnt[c] = k;
 }
 
-constexpr uint64_t kFusedManyLanes = 16384;  // two-site tables of up to so many source states take eight lanes each
+// Source states up to which a two-site table takes eight lanes each, and a triangular one two.
+constexpr uint64_t kFusedManyLanes = 16384, kFusedTwoLanes = 65536;
 
 static uint64_t unit_runs(uint64_t n_dst) { return (n_dst + kPackRows - 1) / kPackRows; }
 
@@ -755,12 +773,13 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
     CP_CUDA_TRY(cudaMemsetAsync(cnt, 0, (3 * n_dst + 3) * 4, st));
     const int bt = 128;
     if (op.fused) {
-        if (op.in.size <= kFusedManyLanes)
-            build_fused_terms_kernel<8><<<(unsigned)((op.in.size * 8 + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
-                                                                                                  slot_edge, K, err);
-        else
-            build_fused_terms_kernel<2><<<(unsigned)((op.in.size * 2 + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst,
-                                                                                                  slot_edge, K, err);
+        auto go = [&](auto kernel, int lanes) {
+            kernel<<<(unsigned)((op.in.size * lanes + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst, slot_edge, K, err);
+        };
+        if (op.in.size <= kFusedManyLanes) go(build_fused_terms_kernel<8, kMaxTerms>, 8);
+        else if (op.kind != OP_TRIANGULAR) go(build_fused_terms_kernel<2, 8>, 2);
+        else if (op.in.size <= kFusedTwoLanes) go(build_fused_terms_kernel<2, 16>, 2);
+        else go(build_fused_terms_kernel<1, 24>, 1);
     } else
         build_terms_kernel<<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst, slot_edge, K, err);
     count_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, op.src_bits, cnt, csum, err + 2);

@@ -229,3 +229,31 @@ def test_rows_of_the_primes_alone_where_padded_ones_do_not_fit():
         del hold
         torch.cuda.empty_cache()
     assert np.array_equal(got[:, :61], want) and not got[:, 61:].any()
+
+
+def test_wide_two_site_tables_keep_their_build_time():
+    # triangular width 17 with two-site tables: one table per factor, as before them, took 47.5 to 48.3 ms
+    import time
+
+    import torch
+    primes, ms = gpu_util.seed_primes(12, seed=51), []
+    for _ in range(4):
+        cp.load().cp_clear_table_cache()
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        cp.Strip("triangular", 17, primes, max_degree=40, max_rows=3).close()
+        ms.append((time.perf_counter() - t) * 1e3)
+    assert min(ms) < 52
+
+
+@pytest.mark.parametrize("lattice,L", [("square", 14), ("triangular", 13), ("triangular", 14), ("triangular", 15)])
+def test_wide_two_site_tables_are_the_product(lattice, L):
+    # every way a two-site table is built (eight, two or one thread a source), against one table per factor
+    primes, out = gpu_util.seed_primes(4, seed=52), []
+    for mode in (3, 0):
+        old = cp.set_factor_pairing(mode)
+        try:
+            out.append(solve(lattice, L, 3, primes, D=12))
+        finally:
+            cp.set_factor_pairing(old)
+    assert np.array_equal(*out)
