@@ -38,6 +38,7 @@
 // registers (5.8) halve the shared-memory traffic but wait longer.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 #include <type_traits>
 
@@ -306,8 +307,8 @@ struct Warp {
         __syncwarp();
     }
 
-    // One unit of work.
-    __device__ __forceinline__ void unit(const uint4 &u, int v_in, int v_out, int cap_in) {
+    // One unit of work: its part `part` of `parts` by degrees.
+    __device__ __forceinline__ void unit(const uint4 &u, uint32_t part, uint32_t parts, int v_in, int v_out, int cap_in) {
         const uint32_t row0 = u.x, nrows = u.y & 63u, e_end = u.w;
         uint2 q = u.z + lane < e_end ? __ldg(t.edges + u.z + lane) : make_uint2(0, 0xff);
         uint32_t a = 0, hi = 0;
@@ -316,10 +317,19 @@ struct Warp {
             a = w & 0xffu;
             const int e = min(t.cap, v_out - (int)(w >> 8)) + 1;
             hi = (a == 0xffu || e <= (int)a) ? a : (uint32_t)e;
-            if ((u.y >> 6) & 1u) {  // a part of a heavy row: an equal share of its degrees, one step of them at least
-                const uint32_t part = u.y >> 8, len = hi - a;
-                const uint32_t share = max((len + kSplitParts - 1) / kSplitParts, t.seg / kSteps);
-                a = min(a + part * share, hi);
+            const bool heavy = (u.y >> 6) & 1u;
+            if (parts > 1 || heavy) {
+                // equal shares of the degrees for the launch's parts, one pass of them at least, and
+                // for the parts of a heavy row, one step of them at least
+                const uint32_t len = hi - a, least = heavy ? t.seg / kSteps : t.seg;
+                uint32_t i = u.y >> 8, share = (len + kSplitParts - 1) / kSplitParts;
+                if (parts > 1) {
+                    const uint32_t all = heavy ? kSplitParts * parts : parts;
+                    i = (heavy ? i * parts : 0) + part;
+                    share = (len + all - 1) / all;
+                }
+                share = max(share, least);
+                a = min(a + i * share, hi);
                 hi = min(a + share, hi);
             }
         }
@@ -369,24 +379,30 @@ struct Warp {
     }
 };
 
-// dv is added to the tasks' vertex counts; first: as if every task's `first` were set.
+// dv is added to the tasks' vertex counts; first: as if every task's `first` were set;
+// parts: warps per unit (degree_parts).
 // Launches overlap: a launch's blocks may start while the one before it drains, load
 // their unit's tables (which no launch writes) and only then wait for it.
 template <int N, uint32_t kDepth, bool kAny>
 __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
-    gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, int dv, int first) {
+    gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, uint32_t parts, int dv,
+                        int first) {
     extern __shared__ __align__(128) uint8_t slots[];  // per warp: kDepth slots of kSegChunks chunks
     __shared__ uint4 lists[kWarps][32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t id = blockIdx.x * kWarps + warp;
+    uint32_t id = blockIdx.x * kWarps + warp, part = 0;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (id >= n_units) return;
+    if (id >= n_units * parts) return;
+    if (parts > 1) {
+        part = id / n_units;
+        id -= part * n_units;
+    }
     const GatherTask &t = pack.t[find_task(pack, n_tasks, id)];
     Warp<kDepth, kAny> w(t, lists[warp]);
     w.lane = lane;
     w.g0 = lane % t.cpd;
     w.slots = smem_addr(slots) + warp * kDepth * kSlotBytes + lane * 16u;
-    w.unit(__ldg(t.units + (id - t.block_begin)), t.v_in + dv, t.v_out + dv, first || t.first ? 0 : t.cap);
+    w.unit(__ldg(t.units + (id - t.block_begin)), part, parts, t.v_in + dv, t.v_out + dv, first || t.first ? 0 : t.cap);
 }
 
 bool chunk_usable(const GatherTask &t) { return t.chunk != 0; }
@@ -415,6 +431,20 @@ int debug_wait_timeout(long long cycles, cudaStream_t st) {
 // flight gain no more (429 us).
 constexpr uint32_t kFewUnits = 2 * 24 * 152;
 
+// Parts that the degrees of a launch's rows are dealt out in, a warp for each part of a
+// unit: as many as the longest row has passes, where that leaves the launch below
+// kFewUnits.  A warp walks its passes one after another, so a strip of few states and
+// long rows (square 4 x 200 on 32 primes as integers: up to 50 passes a row) took 20.2 ms on one
+// part, 4.4 with a block for the columns of a row, and takes 1.4 on these.
+static uint32_t degree_parts(const GatherTask *tasks, int n_tasks, uint32_t n_units, int dv) {
+    uint32_t passes = 1;
+    for (int k = 0; k < n_tasks; ++k) {
+        const uint32_t degrees = (uint32_t)std::min(tasks[k].cap, std::max(tasks[k].v_out + dv, 0)) + 1;
+        passes = std::max(passes, (degrees + tasks[k].seg - 1) / tasks[k].seg);
+    }
+    return std::min(passes, std::max(1u, kFewUnits / std::max(1u, n_units)));
+}
+
 int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, cudaStream_t st, int dv, bool first) {
     return for_packs(tasks, n_tasks, n_units, [&](const auto &pack, int n, uint32_t units) -> int {
         constexpr int N = sizeof(pack.t) / sizeof(GatherTask);
@@ -423,7 +453,8 @@ int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, 
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((units + kWarps - 1) / kWarps);
+        const uint32_t parts = degree_parts(pack.t, n, units, dv);
+        cfg.gridDim = dim3((units * parts + kWarps - 1) / kWarps);
         cfg.blockDim = dim3(32 * kWarps);
         cfg.stream = st;
         cfg.attrs = &attr;
@@ -433,10 +464,10 @@ int launch_gather_chunk(const GatherTask *tasks, int n_tasks, uint32_t n_units, 
         auto go = [&](auto depth, auto any_prime) -> cudaError_t {
             cfg.dynamicSmemBytes = kWarps * decltype(depth)::value * kSlotBytes;
             return cudaLaunchKernelEx(&cfg, gather_chunk_kernel<N, decltype(depth)::value, decltype(any_prime)::value>, pack,
-                                      n, units, dv, first ? 1 : 0);
+                                      n, units, parts, dv, first ? 1 : 0);
         };
         auto pick = [&](auto depth) { return any ? go(depth, std::true_type()) : go(depth, std::false_type()); };
-        CP_CUDA_TRY(units <= kFewUnits ? pick(std::integral_constant<uint32_t, 4>())
+        CP_CUDA_TRY(units * parts <= kFewUnits ? pick(std::integral_constant<uint32_t, 4>())
                                        : pick(std::integral_constant<uint32_t, 2>()));
         return CP_OK;
     });

@@ -257,3 +257,29 @@ def test_wide_two_site_tables_are_the_product(lattice, L):
         finally:
             cp.set_factor_pairing(old)
     assert np.array_equal(*out)
+
+
+# rows of one pass of a warp (512 / lanes degrees) and around whole numbers of passes, dealt out by degrees; widths
+# without and with heavy rows, whose parts are dealt out again
+@pytest.mark.parametrize("lattice", ["square", "triangular"])
+@pytest.mark.parametrize("L,N,P", [(1, 300, 32), (2, 90, 12), (4, 60, 32), (7, 40, 16), (10, 30, 32), (11, 20, 28)])
+def test_long_rows_dealt_out_by_degrees(lattice, L, N, P):
+    primes, span = gpu_util.seed_primes(P, seed=53), 512 // (P + 3 & ~3)
+    whole = None
+    for D in (-1, span - 1, span, 2 * span - 2, 2 * span, 7 * span, 7 * span + 1):
+        got = solve(lattice, L, N, primes, D=D)
+        assert np.array_equal(got, solve(lattice, L, N, primes, D=D, tile=4)), D
+        if D == -1:
+            whole = got
+        else:
+            n = min(D + 1, whole.shape[1])
+            assert np.array_equal(got[:, :n], whole[:, :n]) and not got[:, n:].any(), D
+    if L <= 4 and N <= 90:
+        want = tm_exact.ptilde(lattice, L, N)
+        assert whole.tolist() == gpu_util.residues_of(want, primes)
+
+
+@pytest.mark.parametrize("L,N,P,ms", [(4, 200, 32, 4.2), (3, 400, 4, 5.7), (7, 171, 16, 12.9), (8, 150, 32, 16.4)])
+def test_tall_strips_keep_their_speed(L, N, P, ms):
+    # ms: what the rows and the read-out took with a block for the columns of a row (before the chunk kernel)
+    assert solve_ms("square", L, N, gpu_util.seed_primes(P, seed=54)) < ms
