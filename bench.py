@@ -187,8 +187,8 @@ def table_layout(cp, args):
     if mode == 3:
         return ("two-site tables on both lattices: consecutive site factors composed in pairs (ceil(r/2) launches "
                 "per row, the intermediate vector never written); updates counted per site factor")
-    return ("rows >= 352 bytes: two-site tables, consecutive site factors composed in pairs (ceil(r/2) "
-            "launches per row, the intermediate vector never written); otherwise one table per site factor; "
+    return ("rows >= 352 bytes (square from width 16 on: 1536): two-site tables, consecutive site factors composed "
+            "in pairs (ceil(r/2) launches per row, the intermediate vector never written); otherwise one table per site factor; "
             "updates counted per site factor either way")
 
 

@@ -103,7 +103,10 @@ int cp_create_strip_potts(int lattice, int L, int v, const uint32_t *primes_host
 /*
  * cp_advance_rows -- apply T = T_L ... T_1 n_rows times (eq. (T_sq_decomp));
  * height += n_rows.  Asynchronous on the strip's stream (one gather launch per
- * table: per site, or per pair of sites with two-site tables).
+ * table: per site, or per pair of sites with two-site tables).  Recorded by a stream
+ * capture, the launches are those of the heights they were recorded at (a strip's
+ * coefficients are computed up to what its height can reach): replay them from there,
+ * for instance with a cp_strip_reset recorded before.
  * Errors: CP_EINVAL (height would exceed max_rows), CP_ECUDA.
  */
 int cp_advance_rows(cp_strip *s, int n_rows);
@@ -128,7 +131,7 @@ int cp_strip_info(const cp_strip *s, uint64_t n_states[2], int *degree, int *hei
  * work[0] = updates of one row advance (output words of T_1 .. T_L: sum of
  * S_out (D+1) n_primes over the per-site factors), work[1] = the bytes its
  * launched tables need (each reads its input vector and writes its output
- * vector once, 4 (S_in + S_out)(D+1) n_primes, plus its CSR table,
+ * vector once, 4 (S_in + S_out)(D+1) n_primes, plus its CSR table of packed edges,
  * 4 (S_out + 1 + nnz); a two-site table skips the intermediate vector),
  * work[2], work[3] = the same for one read-out (T_1^last .. T_{L-1}^last),
  * work[4], work[5] = the bytes of the row and of the read-out done one factor

@@ -15,7 +15,7 @@ namespace cp {
 // ------------------------------------------------------------------ errors
 void set_error(const std::string &msg);
 int fail(int code, const std::string &msg);
-// Distinct primes in [2, 2^31), 1..CP_MAX_PRIMES of them (trial division on the host).
+// Distinct primes in [2, 2^31), 1..CP_MAX_PRIMES of them (Miller-Rabin on the host).
 int check_primes(const uint32_t *primes, int n);
 
 #define CP_CUDA_TRY(expr)                                                                \
@@ -190,8 +190,8 @@ struct GatherTask {
 };
 
 // Units of work of the chunk kernel, in row order: consecutive destination rows with
-// at most unit_edges(nnz) edges together and at most 32 rows, or a part of one row
-// with more than split_edges of them.  {first row; rows | heavy << 6 | part << 8;
+// at most unit_edges(nnz) edges together and at most 32 rows, one row of up to
+// split_edges, or a part of one row with more.  {first row; rows | heavy << 6 | part << 8;
 // first edge; one past the last edge}.  Rows differ a hundredfold in edges (the
 // states of many single sites collect most) and the heavy ones lie together, so
 // work is dealt out by edges and not by rows, and a heavy row's degrees are split
@@ -302,7 +302,8 @@ inline int for_packs(const GatherTask *tasks, int n_tasks, uint32_t total_blocks
     }
     return CP_OK;
 }
-// Set the kernels' shared-memory attributes (call outside stream capture).
+// Create what the gathers and their checks need on the device (its error word; call
+// outside stream capture).
 int prepare_gather_kernels();
 // Error words that kernels set: pinned host memory mapped on the device.
 struct ErrorWord {
@@ -311,8 +312,9 @@ struct ErrorWord {
 int error_word_alloc(ErrorWord *w);
 void error_word_free(ErrorWord *w);
 int error_word_take(const ErrorWord &w);  // its value, cleared (after a synchronisation)
-// The device's word, set by bounded waits in kernels; check_device_error syncs
-// `st`, returns CP_ETIMEOUT (and clears the word) if it was set.
+// The device's word, set by a bounded wait that ran out (of the kernels only
+// cp_debug_wait_timeout's waits); check_device_error syncs `st`, returns CP_ETIMEOUT (and
+// clears the word) if it was set.
 int *device_error_flag();
 int check_device_error(cudaStream_t st);
 

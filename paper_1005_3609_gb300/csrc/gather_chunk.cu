@@ -6,7 +6,8 @@
 // only the degrees that can be non-zero are read, computed and written.
 //
 // A warp takes one unit of work (a few consecutive destination rows with up to 64
-// edges, cp_internal.h) and works alone:
+// edges together, or one heavier row or a part of it, cp_internal.h), all its degrees or a
+// share of them, and works alone:
 //   front end  32 edges at a time, one per lane: the edge's word and its source's
 //              window, the window of its destination row, their intersection; the
 //              edges that contribute are listed in shared memory;
@@ -53,30 +54,6 @@ constexpr uint32_t kSlotBytes = kSteps * 512u;         // one edge's source word
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-// The suspend-time hint (ns) lets a waiting warp sleep in the barrier instead of
-// re-issuing the test, leaving the issue slots to the warps that have work.
-constexpr uint32_t kWaitHintNs = 20000;
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t a, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity), "r"(kWaitHintNs)
-        : "memory");
-    return ok != 0;
-}
-// Wait for the phase of parity `parity` to complete; false once the deadline passes.
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, long long deadline) {
-    while (!mbar_try_wait(a, parity))
-        if (clock64() > deadline) return false;
-    return true;
-}
 // Streaming 16-byte global store where pred != 0, without a branch.
 __device__ __forceinline__ void stcs128_if(uint4 *ptr, uint4 v, uint32_t pred) {
     asm volatile(
@@ -387,7 +364,7 @@ template <int N, uint32_t kDepth, bool kAny>
 __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
     gather_chunk_kernel(const __grid_constant__ TaskPack<N> pack, int n_tasks, uint32_t n_units, uint32_t parts, int dv,
                         int first) {
-    extern __shared__ __align__(128) uint8_t slots[];  // per warp: kDepth slots of kSegChunks chunks
+    extern __shared__ __align__(128) uint8_t slots[];  // per warp: kDepth slots of kSlotBytes
     __shared__ uint4 lists[kWarps][32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t id = blockIdx.x * kWarps + warp, part = 0;
@@ -407,9 +384,30 @@ __global__ void __launch_bounds__(32 * kWarps, kChunkBlocksPerSM)
 
 bool chunk_usable(const GatherTask &t) { return t.chunk != 0; }
 
+__device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(uint32_t a, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Wait for the phase of parity `parity` to complete; false once the deadline passes.
+__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, long long deadline) {
+    while (!mbar_try_wait(a, parity))
+        if (clock64() > deadline) return false;
+    return true;
+}
+
 // Diagnostic: a wait that can never complete (an mbarrier nothing arrives on),
-// bounded by `cycles`; on expiry it sets bit 16 of *err and returns, like the
-// gather kernels' waits.
+// bounded by `cycles`; on expiry it sets bit 16 of *err and returns.  (The gathers
+// themselves wait for nothing but their own copies and the launch before.)
 __global__ void wait_timeout_kernel(long long cycles, int *err) {
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) mbar_init(smem_addr(&bar), 1);

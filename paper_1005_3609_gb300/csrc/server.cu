@@ -164,8 +164,9 @@ static size_t request_bytes_estimate(int lattice, int L, int D1, int P) {
     return 2 * al(Smax * RB) + al(sA * RB) + al(sB * RB) + 2 * al(RB) + al(4 * kPrimeWords);
 }
 
-// Largest padded prime count of a job on D1 coefficients: the row must stay a
-// row of at most 1536 16-byte chunks and within CP_MAX_PRIMES.
+// Largest padded prime count of a job on D1 coefficients: rows of at most 1536 16-byte
+// chunks (24 KB) and CP_MAX_PRIMES.  Requests beyond that become further jobs, which share
+// the step's launches but not rows; no kernel needs the line.
 static int job_prime_limit(int D1) {
     int lim = (6144 / D1) & ~3;
     if (lim > CP_MAX_PRIMES) lim = CP_MAX_PRIMES;

@@ -1146,9 +1146,22 @@ int get_tables(int lattice, int L, size_t row_bytes, cudaStream_t st, std::share
     // 0.327 ms, width 8 D 71 on 8 primes 62 and 35 us; triangular width 16 D 32 on 16
     // primes 1.42 and 1.36 ms, width 13 D 181 on 4 primes 0.274 and 0.247 ms, width 9
     // D 80 on 8 primes 77 and 45 us; and half the tables to build: a first square 11 x 10
-    // solve with D 30 on 4 primes (496-byte rows) 5.5 and 3.9 ms.  Not on wide square
-    // strips of short rows, where launches are long and there is little to reduce: square
-    // width 17 D 40 on 5 primes, four rows and the read-out, 6.76 and 7.08 ms.
+    // solve with D 30 on 4 primes (496-byte rows) 5.5 and 3.9 ms.  Four or eight rows and the
+    // read-out, time with one table per factor over time with two-site tables:
+    //   row bytes            176        352        496        1312       2624
+    //   width 4 to 8       1.1-1.7    1.2-1.7    1.2-1.7    1.3-1.7    1.5-1.6
+    //   width 10 square      1.06       1.10       1.10       1.21       1.38
+    //   width 12 square      0.94       0.93       0.98       1.05       1.11
+    //   width 12 triangular  1.03       1.00       1.09       1.18       1.23
+    //   width 14, 15       1.4-2.1    1.3-1.5    1.25-1.4   1.2-1.3    1.2-1.3
+    //   width 16 square      0.97       1.30       1.27       1.28       1.27
+    //   width 16 triangular  1.00       1.24       1.18       1.18       1.18
+    //   width 17, 18       0.8-0.9    0.9-1.0    1.04-1.1   1.07-1.15  1.08-1.15
+    // so at 352 bytes the widest strips break even.  Wide square strips wait for rows of 1536
+    // bytes: with units of 32 edges shorter rows lost there (width 17 D 40 on 5 primes, four
+    // rows and the read-out, 6.76 and 7.08 ms); with units of 64 they gain (8 primes 5.95 and
+    // 5.19 ms), but two-site tables take longer to build (width 17 44 and 56 ms, width 19
+    // 277 and 433), which takes some sixty such rows to pay back.
     const bool wide_short = lattice == CP_SQUARE && L >= kPairWide && row_bytes < kPairWideRowBytes;
     const int paired = g_pairing == 3 || (lattice == CP_SQUARE && g_pairing == 2) ||
                        (g_pairing == 1 && row_bytes >= kPairRowBytes && !wide_short);
