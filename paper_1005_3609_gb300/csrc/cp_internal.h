@@ -25,6 +25,27 @@ int check_primes(const uint32_t *primes, int n);
             return ::cp::fail(CP_ECUDA, std::string(#expr) + ": " + cudaGetErrorString(_e)); \
     } while (0)
 
+// Device allocation helpers (library-owned memory).
+int dev_alloc(void **p, size_t bytes);
+void dev_free(void *p);
+
+// Device memory handed out in pieces of 256-byte multiples and given back as a whole.
+// Small pieces come from common blocks, which grow from 64 KB to 1 MB; one of kPoolPiece
+// bytes or more has an allocation of its own.
+constexpr size_t kPoolPiece = 256 << 10;
+class DevPool {
+    std::vector<void *> blocks_;
+    char *at_ = nullptr;
+    size_t left_ = 0, next_ = 64 << 10;
+
+  public:
+    DevPool() = default;
+    DevPool(const DevPool &) = delete;
+    DevPool &operator=(const DevPool &) = delete;
+    ~DevPool();
+    int alloc(void **p, size_t bytes);
+};
+
 // ------------------------------------------------------------------ state spaces
 // Point counts go up to CP_MAXN in the rank tables (contracted spaces use L-1).
 constexpr int kMaxN = 24;
@@ -112,7 +133,7 @@ struct SiteTable {
     uint64_t n_src = 0, n_dst = 0, nnz = 0;
     uint64_t n_site_out = 0;  // output states of the per-site factors it stands for (n_dst, or mid + n_dst)
     uint32_t *row_ptr = nullptr;  // [n_dst + 1]
-    uint32_t *edges = nullptr;    // [nnz] while the table is built
+    uint32_t *edges = nullptr;    // [nnz] while the table is built (of its own from kBigTable edges on)
     uint2 *wedges = nullptr;      // [nnz] the edges as the gathers read them (GatherTask::edges)
     uint4 *units = nullptr;           // [n_units] units of work of the chunk kernel (GatherTask::units)
     uint32_t n_units = 0;
@@ -121,6 +142,10 @@ struct SiteTable {
     uint32_t max_coef_sum = 0;        // largest sum of |coefficient| into one destination (an upper bound)
     uint32_t max_abs_coef = 0;        // largest |coefficient|
 };
+
+// A wide strip's tables take gigabytes: edges of such a table are freed as soon as its
+// wedges are there, so that there is no second copy of more than one of them.
+constexpr uint64_t kBigTable = 1u << 24;
 
 // All tables of one (lattice, L) on one device; shared between strips.
 struct TableSet {
@@ -132,7 +157,7 @@ struct TableSet {
     std::vector<SiteTable> row;
     std::vector<SiteTable> last;
     std::vector<uint32_t *> x_prefix;  // square lattice: prefix table of X_e, e = 0..L-2
-    std::vector<uint16_t *> wins;      // window words of every space of the two chains
+    DevPool pool;                      // what the tables, prefixes and windows lie in
     size_t bytes = 0;
     ~TableSet();
 };
@@ -341,10 +366,6 @@ uint64_t rectangle_edges(int lattice, int L, int N);
 int crt_outcome(const uint32_t *flags, int n_coeffs);
 // Load the CRT module (and the static array of cp_crt_static) on the current device.
 int crt_static_touch();
-
-// Device allocation helpers (library-owned memory).
-int dev_alloc(void **p, size_t bytes);
-void dev_free(void *p);
 
 // What an object's padding lanes take beyond the rows of its primes alone.  The lanes of
 // all objects on a device together get at most 1 / kPadFraction of its memory, so that

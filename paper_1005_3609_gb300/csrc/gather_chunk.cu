@@ -22,8 +22,8 @@
 //              multiply-adds per word.
 //
 // What bounds it: the shared-memory data path, each source word going through it twice
-// (copy and load; 80% of its rate in the middle launches of the square width-16 row, where
-// DRAM gives 3.0 TB/s and L2 is at 40%), with the issue slots next (64%).  Width 14, D = 63, 16 primes (57 346 rows, 365 000
+// (copy and load; 78% of its rate in the middle launches of the square width-16 row, where
+// DRAM gives 3.8 TB/s and L2 is at 46%), with the issue slots next (66%).  Width 14, D = 63, 16 primes (57 346 rows, 365 000
 // edges of a two-site table): 0.66 instructions per scheduler and cycle, 66% of the
 // shared-memory data path, DRAM at a quarter of its rate, 0.107 ms; the
 // producer/consumer kernel on whole rows that this one replaces took 0.155 ms.  One

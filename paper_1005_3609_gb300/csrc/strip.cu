@@ -37,6 +37,30 @@ void dev_free(void *p) {
     if (p) cudaFree(p);
 }
 
+DevPool::~DevPool() {
+    for (auto p : blocks_) dev_free(p);
+}
+
+int DevPool::alloc(void **p, size_t bytes) {
+    bytes = ((bytes ? bytes : 1) + 255) & ~(size_t)255;
+    const bool own = bytes >= kPoolPiece;
+    if (!own && bytes <= left_) {
+        *p = at_;
+    } else {
+        const size_t size = own ? bytes : std::max(bytes, next_);
+        const int rc = dev_alloc(p, size);
+        if (rc) return rc;
+        blocks_.push_back(*p);
+        if (own) return CP_OK;
+        at_ = (char *)*p;
+        left_ = size;
+        next_ = std::min<size_t>(4 * next_, 1 << 20);
+    }
+    at_ += bytes;
+    left_ -= bytes;
+    return CP_OK;
+}
+
 static std::mutex g_pad_mu;
 static size_t g_pad_used[64], g_pad_limit[64];  // per device
 

@@ -434,9 +434,9 @@ __global__ void scan_sums_serial(uint32_t *sums, uint32_t n_blocks) {
 }
 
 // With `of`, also the largest of of[0..n) into *largest (a warp maximum, one atomic
-// per warp; on its own that was one more launch of 4.6 us a table).
+// per warp; on its own that was one more launch of 4.6 us a table); with `total`, the sum there too.
 __global__ void scan_finish(const uint32_t *in, uint64_t n, const uint32_t *block_off, uint32_t *out, const uint32_t *of,
-                            int *largest) {
+                            int *largest, uint32_t *total) {
     __shared__ uint32_t ws[32], before;
     const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t off = 0;
@@ -456,7 +456,10 @@ __global__ void scan_finish(const uint32_t *in, uint64_t n, const uint32_t *bloc
     const uint32_t inc = block_inclusive_scan(v, ws);
     const uint32_t exc = off + inc - v;
     if (k < n) out[k] = exc;
-    if (k == n - 1) out[n] = exc + v;
+    if (k == n - 1) {
+        out[n] = exc + v;
+        if (total) *total = exc + v;
+    }
     if (of) {
         const uint32_t m = __reduce_max_sync(0xffffffffu, k < n ? of[k] : 0u);
         if ((threadIdx.x & 31) == 0) atomicMax(largest, (int)m);
@@ -554,9 +557,9 @@ __global__ void copy_blocks_kernel(const uint16_t *win_row, uint16_t *win, uint6
 // is set where a value fell.  A small table's launch lasts as long as its longest
 // row's chain of dependent loads (rows of a hundred edges come up), so eight lanes
 // share a row there; a large one is bound by its instructions and takes a thread per
-// row (first triangular strips, cold: width 12 3.30 ms with one lane, 2.81 with eight;
-// width 16 29.9 and 34.3).
-constexpr uint64_t kWinManyLanes = 65536;  // rows up to which a row takes eight lanes
+// row (cold tables of square strips with rows of 336 bytes, one lane and eight: width 14,
+// 57 346 rows, 6.7 and 7.6 ms, width 16 18.1 and 27.6; width 13, 21 309 rows, 4.9 and 4.8).
+constexpr uint64_t kWinManyLanes = 32768;  // rows up to which a row takes eight lanes
 template <uint32_t kLanes>
 __global__ void relax_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits,
                                  const uint16_t *win_in, uint16_t *win_out, const int *prev, int *changed) {
@@ -579,14 +582,15 @@ __global__ void relax_win_kernel(const uint32_t *row_ptr, const uint32_t *edges,
 }
 
 // Every transition keeps its source's window inside its destination's: lo_dst <=
-// lo_src + shift, and V_src - blocks_src + shift <= V_dst - blocks_dst.  (Lanes as above.)
+// lo_src + shift, and V_src - blocks_src + shift <= V_dst - blocks_dst.  With e0 (a row's
+// last table), no state but e_0 (rank 0) has degree 0.  (Lanes as above.)
 template <uint32_t kLanes>
 __global__ void check_win_kernel(const uint32_t *row_ptr, const uint32_t *edges, uint64_t n_dst, int src_bits, int sites,
-                                 const uint16_t *win_in, const uint16_t *win_out, int *bad) {
+                                 const uint16_t *win_in, const uint16_t *win_out, int e0, int *bad) {
     const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, d = k / kLanes;
     if (d >= n_dst) return;
     const uint32_t mask = (1u << src_bits) - 1u, w = win_out[d];
-    bool ok = true;
+    bool ok = !e0 || ((w & 0xffu) == 0) == (d == 0);
     for (uint32_t e = row_ptr[d] + (uint32_t)(k % kLanes), e1 = row_ptr[d + 1]; e < e1; e += kLanes) {
         const uint32_t q = edges[e], sh = (q >> src_bits) & 3u, x = win_in[q & mask];
         if ((x & 0xffu) == 255) continue;
@@ -595,26 +599,28 @@ __global__ void check_win_kernel(const uint32_t *row_ptr, const uint32_t *edges,
     if (!ok) *bad = 1;
 }
 
-// States of degree 0 other than e_0 (rank 0): none in a row space.
-__global__ void check_e0_kernel(const uint16_t *win, uint64_t n, int *bad) {
-    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n && ((win[r] & 0xffu) == 0) != (r == 0)) *bad = 1;
-}
-
 // ------------------------------------------------------------------ host side
 
 // Working memory of one table set's build: one device allocation, handed out from
 // the start for each table (the build's kernels run on one stream, in order) and
 // freed with the object, instead of a dozen allocations and frees, each a
-// synchronisation, per table.
+// synchronisation, per table.  What stays of a set and its plain edges lie in pools for
+// the same reason, and a table stops the host once (for its edges' number): with four
+// allocations and two stops a table, small sets of one table per factor took longer
+// than without degree windows (cold, square Potts width 7 1.97 ms, 1.66 without, now 1.44;
+// square width 9, 336-byte rows, 2.94, 2.72 and 2.20).
 struct Scratch {
     char *base = nullptr;
     size_t cap = 0, used = 0;
     cudaStream_t st;
+    DevPool edges;                // plain edges of the set's tables, below kBigTable of them
+    uint32_t *counts = nullptr;   // units of each table (kMaxTables words), then the windows' flags (kWinFlags)
+    int n_counts = 0;
+    bool idle = false;            // nothing of the build is in flight any more
     explicit Scratch(cudaStream_t s) : st(s) {}
     Scratch(const Scratch &) = delete;
     ~Scratch() {
-        if (base) cudaStreamSynchronize(st);
+        if (!idle) cudaStreamSynchronize(st);
         dev_free(base);
     }
     // Start over with at least `bytes` bytes.
@@ -643,7 +649,7 @@ static size_t scan_bytes(uint64_t n) { return Scratch::span(((n + kScanThreads -
 // out[0..n]: exclusive scan of cnt, with the total at the end, and the largest of
 // of[0..n) into *largest (asynchronous on sc->st).
 static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *out, Scratch *sc, const uint32_t *of = nullptr,
-                          int *largest = nullptr) {
+                          int *largest = nullptr, uint32_t *total = nullptr) {
     uint64_t nb = (n + kScanThreads - 1) / kScanThreads;
     if (nb > (1u << 31)) return fail(CP_EINVAL, "scan too large");
     uint32_t *sums = nullptr;
@@ -652,12 +658,12 @@ static int scan_exclusive(const uint32_t *cnt, uint64_t n, uint32_t *out, Scratc
         scan_block_sums<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums);
         scan_sums_serial<<<1, kScanThreads, 0, sc->st>>>(sums, (uint32_t)nb);
     }
-    scan_finish<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums, out, of, largest);
+    scan_finish<<<(unsigned)nb, kScanThreads, 0, sc->st>>>(cnt, n, sums, out, of, largest, total);
     CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
 
-static int build_x_prefix(int m, int e, Scratch *sc, uint32_t **out) {
+static int build_x_prefix(int m, int e, Scratch *sc, DevPool *pool, uint32_t **out) {
     const RankTables *T_dev = nullptr;
     RankTables T;
     int rc = device_rank_tables(&T_dev, &T);
@@ -665,7 +671,7 @@ static int build_x_prefix(int m, int e, Scratch *sc, uint32_t **out) {
     const uint64_t Sb = T.cnt[m];
     if ((rc = sc->reset(Scratch::span(Sb * 4) + scan_bytes(Sb)))) return rc;
     uint32_t *flag = sc->take<uint32_t>(Sb), *pre = nullptr;
-    if ((rc = dev_alloc((void **)&pre, (Sb + 1) * 4))) return rc;
+    if ((rc = pool->alloc((void **)&pre, (Sb + 1) * 4))) return rc;
     x_partner_kernel<<<(unsigned)((Sb + 127) / 128), 128, 0, sc->st>>>(m, e, T_dev, flag);
     rc = scan_exclusive(flag, Sb, pre, sc);
     uint32_t total = 0;
@@ -673,18 +679,14 @@ static int build_x_prefix(int m, int e, Scratch *sc, uint32_t **out) {
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(sc->st);
     if (!rc && ce != cudaSuccess) rc = fail(CP_ECUDA, std::string("x_partner: ") + cudaGetErrorString(ce));
     if (!rc && total != T.cnt[m - 1]) rc = fail(CP_ESTATE, "excepted space has the wrong size");
-    if (rc) {
-        dev_free(pre);
-        return rc;
-    }
-    *out = pre;
-    return CP_OK;
+    if (!rc) *out = pre;
+    return rc;
 }
 
 // Packs the rows of one run of kPackRows into units (cp_internal.h), in order: one
 // thread per run.  Without `units` it only counts them.
 __global__ void pack_units_kernel(const uint32_t *row_ptr, uint64_t n, uint32_t most, uint32_t split, uint32_t *cnt,
-                                  const uint32_t *pos, uint4 *units) {
+                                  const uint32_t *pos, uint4 *units, uint32_t *total) {
     const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, r0 = c * kPackRows;
     if (r0 >= n) return;
     const uint64_t r1 = min(n, r0 + kPackRows);
@@ -711,26 +713,41 @@ __global__ void pack_units_kernel(const uint32_t *row_ptr, uint64_t n, uint32_t 
         b = e;
     }
     if (!units) cnt[c] = k;
+    else if (r1 == n) *total = k;
 }
 
 // Source states up to which a two-site table takes eight lanes each, and a triangular one two.
 constexpr uint64_t kFusedManyLanes = 16384, kFusedTwoLanes = 65536;
 
+constexpr int kMaxTables = 2 * CP_MAX_L;  // of a set: a row's and the read-out's
+// Of the windows: changed, one per pass; the checks' flag; what the read-out's tables changed (not used).
+constexpr int kMaxPasses = 64, kWinFlags = kMaxPasses + 2;
+
 static uint64_t unit_runs(uint64_t n_dst) { return (n_dst + kPackRows - 1) / kPackRows; }
 
-// (in the room that build_table reserved)
-static int build_units(SiteTable *tab, Scratch *sc) {
+// Units of a table, in the room that build_table reserved; n_units is read back with the
+// windows' flags (build_windows), so a small table has room for the most there can be: a
+// unit is closed by a run's end, by the next row's edges (two neighbours then have more
+// than `most` between them) or by a heavy row, which is kSplitParts itself.
+static int build_units(SiteTable *tab, Scratch *sc, DevPool *pool) {
     const uint64_t n = tab->n_dst, runs = unit_runs(n);
     uint32_t *cnt = sc->take<uint32_t>(runs), *pos = sc->take<uint32_t>(runs + 1);
     const unsigned grid = (unsigned)((runs + 63) / 64);
     const uint32_t most = unit_edges(tab->nnz), split = split_edges(most);
-    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, cnt, nullptr, nullptr);
+    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, cnt, nullptr, nullptr, nullptr);
     int rc = scan_exclusive(cnt, runs, pos, sc);
     if (rc) return rc;
-    CP_CUDA_TRY(cudaMemcpyAsync(&tab->n_units, pos + runs, 4, cudaMemcpyDeviceToHost, sc->st));
-    CP_CUDA_TRY(cudaStreamSynchronize(sc->st));
-    if ((rc = dev_alloc((void **)&tab->units, std::max<size_t>(1, tab->n_units) * sizeof(uint4)))) return rc;
-    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, nullptr, pos, tab->units);
+    uint64_t room = std::min<uint64_t>(n, runs + 2 * tab->nnz / most + 1 + tab->nnz / split) + kSplitParts * (tab->nnz / split);
+    if (room * sizeof(uint4) >= kPoolPiece) {
+        uint32_t units = 0;
+        CP_CUDA_TRY(cudaMemcpyAsync(&units, pos + runs, 4, cudaMemcpyDeviceToHost, sc->st));
+        CP_CUDA_TRY(cudaStreamSynchronize(sc->st));
+        room = units;
+    }
+    if ((rc = pool->alloc((void **)&tab->units, room * sizeof(uint4)))) return rc;
+    if (!sc->counts && (rc = sc->edges.alloc((void **)&sc->counts, (kMaxTables + kWinFlags) * 4))) return rc;
+    pack_units_kernel<<<grid, 64, 0, sc->st>>>(tab->row_ptr, n, most, split, nullptr, pos, tab->units,
+                                               sc->counts + sc->n_counts++);
     CP_CUDA_TRY(cudaGetLastError());
     return CP_OK;
 }
@@ -753,7 +770,7 @@ __global__ void fill_wedges_kernel(const uint4 *units, uint32_t n_units, const u
     }
 }
 
-static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, SiteTable *tab) {
+static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, DevPool *pool, SiteTable *tab) {
     tab->op = op;
     tab->n_src = op.in.size;
     tab->n_dst = op.out.size;
@@ -763,14 +780,14 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
     const int K = op.max_terms;
     const uint64_t n_slots = op.in.size * (uint64_t)K, n_dst = op.out.size, runs = unit_runs(n_dst);
     const cudaStream_t st = sc->st;
-    int rc = sc->reset(2 * Scratch::span(n_slots * 4) + Scratch::span((3 * n_dst + 3) * 4) + scan_bytes(n_dst) +
+    int rc = sc->reset(2 * Scratch::span(n_slots * 4) + Scratch::span((3 * n_dst + 4) * 4) + scan_bytes(n_dst) +
                        2 * Scratch::span((runs + 1) * 4) + scan_bytes(runs));
     if (rc) return rc;
     uint32_t *slot_dst = sc->take<uint32_t>(n_slots), *slot_edge = sc->take<uint32_t>(n_slots);
-    uint32_t *cnt = sc->take<uint32_t>(3 * n_dst + 3), *cursor = cnt + n_dst, *csum = cursor + n_dst;
-    int *err = reinterpret_cast<int *>(csum + n_dst);
-    if ((rc = dev_alloc((void **)&tab->row_ptr, (n_dst + 1) * 4))) return rc;
-    CP_CUDA_TRY(cudaMemsetAsync(cnt, 0, (3 * n_dst + 3) * 4, st));
+    uint32_t *cnt = sc->take<uint32_t>(3 * n_dst + 4), *cursor = cnt + n_dst, *csum = cursor + n_dst;
+    int *err = reinterpret_cast<int *>(csum + n_dst);  // error bits, largest sum, largest coefficient, edges
+    if ((rc = pool->alloc((void **)&tab->row_ptr, (n_dst + 1) * 4))) return rc;
+    CP_CUDA_TRY(cudaMemsetAsync(cnt, 0, (3 * n_dst + 4) * 4, st));
     const int bt = 128;
     if (op.fused) {
         auto go = [&](auto kernel, int lanes) {
@@ -784,11 +801,10 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
         build_terms_kernel<<<(unsigned)((op.in.size + bt - 1) / bt), bt, 0, st>>>(op, T_dev, slot_dst, slot_edge, K, err);
     count_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, op.src_bits, cnt, csum, err + 2);
     CP_CUDA_TRY(cudaGetLastError());
-    if ((rc = scan_exclusive(cnt, n_dst, tab->row_ptr, sc, csum, err + 1))) return rc;
-    int herr[3] = {0, 0, 0};
-    uint32_t nnz = 0;
-    CP_CUDA_TRY(cudaMemcpyAsync(herr, err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
-    CP_CUDA_TRY(cudaMemcpyAsync(&nnz, tab->row_ptr + n_dst, 4, cudaMemcpyDeviceToHost, st));
+    if ((rc = scan_exclusive(cnt, n_dst, tab->row_ptr, sc, csum, err + 1, reinterpret_cast<uint32_t *>(err + 3))))
+        return rc;
+    int herr[4] = {0, 0, 0, 0};
+    CP_CUDA_TRY(cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, st));
     const cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(CP_ECUDA, std::string("table build: ") + cudaGetErrorString(e));
     // The gathers reduce p 2^21 + sum_e coef_e x_e (x_e < p) exactly while
@@ -802,45 +818,37 @@ static int build_table(const OpDesc &op, const RankTables *T_dev, Scratch *sc, S
         return fail(CP_ESTATE, "transition table check failed (flags " + std::to_string(herr[0]) + ") for op kind " +
                                    std::to_string(op.kind) + " m=" + std::to_string(op.m) + " i=" +
                                    std::to_string(op.i));
+    const uint32_t nnz = (uint32_t)herr[3];
     tab->nnz = nnz;
     tab->max_coef_sum = (uint32_t)herr[1];
     tab->max_abs_coef = (uint32_t)herr[2];
-    if ((rc = dev_alloc((void **)&tab->edges, (size_t)(nnz ? nnz : 1) * 4))) return rc;
+    rc = nnz >= kBigTable ? dev_alloc((void **)&tab->edges, (size_t)nnz * 4)
+                          : sc->edges.alloc((void **)&tab->edges, (size_t)nnz * 4);
+    if (rc) return rc;
     fill_kernel<<<1216, 256, 0, st>>>(slot_dst, slot_edge, n_slots, tab->row_ptr, cursor, tab->edges);
     sort_segments_kernel<<<(unsigned)((n_dst + 7) / 8), 256, 0, st>>>(tab->row_ptr, n_dst, tab->edges);
     CP_CUDA_TRY(cudaGetLastError());
-    return build_units(tab, sc);
+    return build_units(tab, sc, pool);
 }
 
 TableSet::~TableSet() {
-    for (auto p : x_prefix) dev_free(p);
-    for (auto p : wins) dev_free(p);
-    for (auto &t : row) {
-        dev_free(t.row_ptr);
-        dev_free(t.edges);
-        dev_free(t.wedges);
-        dev_free(t.units);
-    }
-    for (auto &t : last) {
-        dev_free(t.row_ptr);
-        dev_free(t.edges);
-        dev_free(t.wedges);
-        dev_free(t.units);
-    }
+    for (auto *chain : {&row, &last})  // (only of a build that failed)
+        for (auto &t : *chain)
+            if (t.nnz >= kBigTable) dev_free(t.edges);
 }
 
 // Window words of every space of the two chains (cp_internal.h): the blocks by
 // unranking, lo by relaxing the row's tables from e_0 until a whole row changes
 // nothing (values only fall, a row per pass; a state needs about as many rows as
-// its blocks are nested, so L / 2 + 1 passes mostly do, each a no-op once
-// nothing changes), then the read-out's tables once.
+// its blocks are nested: up to width 17 the last change came in pass (L + 1) / 2, of
+// Potts strips L / 2 + 1, so one more does in a round, each a no-op once nothing
+// changes), then the read-out's tables once.
 static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
     const cudaStream_t st = sc->st;
     auto grid = [](uint64_t n) { return (unsigned)((n + 127) / 128); };
     int rc;
     auto new_win = [&](uint64_t n, uint16_t **w) -> int {
-        if ((rc = dev_alloc((void **)w, n * 2))) return rc;
-        ts->wins.push_back(*w);
+        if ((rc = ts->pool.alloc((void **)w, n * 2))) return rc;
         ts->bytes += n * 2;
         return CP_OK;
     };
@@ -863,59 +871,57 @@ static int build_windows(TableSet *ts, const RankTables *T_dev, Scratch *sc) {
         t.win_out = o;
         w = o;
     }
-    constexpr int kMaxPasses = 64;
-    const int per_round = ts->L / 2 + 1;
-    if ((rc = sc->reset((kMaxPasses + 1) * sizeof(int)))) return rc;
-    int *flags = sc->take<int>(kMaxPasses + 1);  // changed, one per pass; then the checks' flag
-    cudaError_t e = cudaMemsetAsync(flags, 0, (kMaxPasses + 1) * sizeof(int), st);
+    const int per_round = ts->potts ? ts->L / 2 + 2 : (ts->L + 1) / 2 + 1;
+    int *flags = reinterpret_cast<int *>(sc->counts + kMaxTables);
+    cudaError_t e = cudaMemsetAsync(flags, 0, kWinFlags * sizeof(int), st);
     auto relax = [&](const SiteTable &t, const int *prev, int *changed) {
         const bool many = t.n_dst <= kWinManyLanes;
         (many ? relax_win_kernel<8> : relax_win_kernel<1>)<<<grid(t.n_dst * (many ? 8 : 1)), 128, 0, st>>>(
             t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.win_in, const_cast<uint16_t *>(t.win_out), prev, changed);
     };
-    int host[kMaxPasses + 1] = {}, pass = 0;
+    int back[kMaxTables + kWinFlags] = {}, pass = 0;  // counts and flags
+    const int *host = back + kMaxTables;
     bool done = false;
     while (e == cudaSuccess && !done && pass < kMaxPasses) {
         const int to = std::min(kMaxPasses, pass + per_round);
         for (; pass < to; ++pass)
             for (auto &t : ts->row) relax(t, pass ? flags + pass - 1 : nullptr, flags + pass);
         // (the row's part is complete when the last pass changed nothing; the rest is redone otherwise)
-        for (auto &t : ts->last) relax(t, nullptr, flags + kMaxPasses);
-        e = cudaMemsetAsync(flags + kMaxPasses, 0, sizeof(int), st);
+        for (auto &t : ts->last) relax(t, nullptr, flags + kMaxPasses + 1);
+        if (pass > per_round) e = cudaMemsetAsync(flags + kMaxPasses, 0, sizeof(int), st);
         for (auto *chain : {&ts->row, &ts->last})
             for (auto &t : *chain) {
                 const bool many = t.n_dst <= kWinManyLanes;
                 (many ? check_win_kernel<8> : check_win_kernel<1>)<<<grid(t.n_dst * (many ? 8 : 1)), 128, 0, st>>>(
-                    t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.sites, t.win_in, t.win_out, flags + kMaxPasses);
+                    t.row_ptr, t.edges, t.n_dst, t.op.src_bits, t.sites, t.win_in, t.win_out, t.win_out == win[0] ? 1 : 0,
+                    flags + kMaxPasses);
             }
-        check_e0_kernel<<<grid(ts->row[0].n_src), 128, 0, st>>>(win[0], ts->row[0].n_src, flags + kMaxPasses);
         if (e == cudaSuccess) e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host, flags, sizeof(host), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(back, sc->counts, sizeof(back), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         done = host[pass - 1] == 0;
     }
     if (e != cudaSuccess) return fail(CP_ECUDA, std::string("degree windows: ") + cudaGetErrorString(e));
     if (!done || host[kMaxPasses]) return fail(CP_ESTATE, "degree windows of the state spaces are inconsistent");
+    int k = 0;
+    for (auto *chain : {&ts->row, &ts->last})
+        for (auto &t : *chain) t.n_units = (uint32_t)back[k++];
     // the edges as the gathers read them replace the plain ones
     for (auto *chain : {&ts->row, &ts->last})
         for (auto &t : *chain) {
-            if ((rc = dev_alloc((void **)&t.wedges, std::max<size_t>(1, t.nnz) * sizeof(uint2)))) return rc;
+            if ((rc = ts->pool.alloc((void **)&t.wedges, t.nnz * sizeof(uint2)))) return rc;
             if (t.n_units)
                 fill_wedges_kernel<<<(t.n_units + 7) / 8, 256, 0, st>>>(t.units, t.n_units, t.row_ptr, t.edges,
                                                                        t.op.src_bits, t.win_in, t.wedges);
             CP_CUDA_TRY(cudaGetLastError());
-            if (t.nnz >= (1u << 24)) {  // a wide strip's tables take gigabytes: no second copy of more than one of them
+            if (t.nnz >= kBigTable) {
                 CP_CUDA_TRY(cudaStreamSynchronize(st));
                 dev_free(t.edges);
-                t.edges = nullptr;
             }
+            t.edges = nullptr;  // (the others go with the build's working memory)
         }
     CP_CUDA_TRY(cudaStreamSynchronize(st));
-    for (auto *chain : {&ts->row, &ts->last})
-        for (auto &t : *chain) {
-            dev_free(t.edges);
-            t.edges = nullptr;
-        }
+    sc->idle = true;
     return CP_OK;
 }
 
@@ -936,7 +942,7 @@ int add_window_degrees(const uint16_t *win, uint64_t n, int v, int cap, unsigned
 }
 
 // Identity factor on a 1-state space (T_1^last = D_1 on the width-1 strip).
-static int identity_table(int m, Scratch *sc, SiteTable *tab) {
+static int identity_table(int m, Scratch *sc, DevPool *pool, SiteTable *tab) {
     OpDesc op{};
     op.kind = OP_IDENTITY;
     op.m = m;
@@ -946,14 +952,13 @@ static int identity_table(int m, Scratch *sc, SiteTable *tab) {
     tab->op = op;
     tab->n_src = tab->n_dst = tab->nnz = tab->n_site_out = 1;
     tab->max_coef_sum = tab->max_abs_coef = 1;
-    int rc = dev_alloc((void **)&tab->row_ptr, 8);
+    int rc = pool->alloc((void **)&tab->row_ptr, 12);  // row_ptr and its edge
     if (rc) return rc;
-    if ((rc = dev_alloc((void **)&tab->edges, 4))) return rc;
-    uint32_t rp[2] = {0, 1}, ed = 0u | (1u << (kSrcBits + 2));
-    CP_CUDA_TRY(cudaMemcpy(tab->row_ptr, rp, 8, cudaMemcpyHostToDevice));
-    CP_CUDA_TRY(cudaMemcpy(tab->edges, &ed, 4, cudaMemcpyHostToDevice));
+    tab->edges = tab->row_ptr + 2;
+    const uint32_t words[3] = {0, 1, 0u | (1u << (kSrcBits + 2))};
+    CP_CUDA_TRY(cudaMemcpyAsync(tab->row_ptr, words, sizeof(words), cudaMemcpyHostToDevice, sc->st));
     if ((rc = sc->reset(4096))) return rc;
-    return build_units(tab, sc);
+    return build_units(tab, sc, pool);
 }
 
 // Tables of a chain of per-site factors: one per factor, or (paired) one
@@ -975,12 +980,12 @@ static int build_chain(const std::vector<OpDesc> &ops, int paired, int lattice, 
             f.out = ops[i + 1].out;
             f.max_terms = ops[i].kind == OP_LAST ? 4 : (lattice == CP_SQUARE ? 16 : 24);
             f.src_bits = lattice == CP_SQUARE ? 26 : 25;
-            rc = build_table(f, T_dev, sc, &tab);
+            rc = build_table(f, T_dev, sc, &ts->pool, &tab);
             tab.n_site_out = ops[i].out.size + ops[i + 1].out.size;
             tab.sites = 2;
             i += 2;
         } else {
-            rc = build_table(ops[i], T_dev, sc, &tab);
+            rc = build_table(ops[i], T_dev, sc, &ts->pool, &tab);
             i += 1;
         }
         if (rc) {
@@ -1011,7 +1016,7 @@ static int build_tableset(int lattice, int L, int paired, cudaStream_t st, std::
     if (lattice == CP_SQUARE) {
         for (int e = 0; e + 1 < L; ++e) {
             uint32_t *pre = nullptr;
-            if ((rc = build_x_prefix(L, e, &sc, &pre))) return rc;
+            if ((rc = build_x_prefix(L, e, &sc, &ts->pool, &pre))) return rc;
             ts->x_prefix.push_back(pre);
             ts->bytes += (Sb + 1) * 4;
         }
@@ -1049,7 +1054,7 @@ static int build_tableset(int lattice, int L, int paired, cudaStream_t st, std::
     if ((rc = build_chain(row_ops, paired, lattice, T_dev, &sc, ts.get(), &ts->row))) return rc;
     if (L == 1) {
         SiteTable tab;
-        if ((rc = identity_table(1, &sc, &tab))) return rc;
+        if ((rc = identity_table(1, &sc, &ts->pool, &tab))) return rc;
         ts->last.push_back(tab);
     } else if ((rc = build_chain(last_ops, paired, lattice, T_dev, &sc, ts.get(), &ts->last))) {
         return rc;
@@ -1086,14 +1091,14 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
         op.in = Space{SPACE_C, L, 0, 0, S, nullptr};
         op.out = op.in;
         SiteTable tab;
-        rc = build_table(op, T_dev, &sc, &tab);
+        rc = build_table(op, T_dev, &sc, &ts->pool, &tab);
         ts->bytes += (tab.n_dst + 1 + 2 * tab.nnz) * 4;
         ts->row.push_back(tab);
         if (rc) return rc;
     }
     if (L == 1) {
         SiteTable tab;
-        if ((rc = identity_table(1, &sc, &tab))) return rc;
+        if ((rc = identity_table(1, &sc, &ts->pool, &tab))) return rc;
         ts->last.push_back(tab);
     } else {
         for (int i = 0; i + 1 < L; ++i) {  // D_L is the identity on e_0
@@ -1107,7 +1112,7 @@ static int build_potts_tableset(int lattice, int L, int v, cudaStream_t st, std:
             op.in = Space{SPACE_C, L, 0, 0, T.cntc[L - i], nullptr};
             op.out = Space{SPACE_C, L, 0, 0, T.cntc[L - i - 1], nullptr};
             SiteTable tab;
-            rc = build_table(op, T_dev, &sc, &tab);
+            rc = build_table(op, T_dev, &sc, &ts->pool, &tab);
             ts->bytes += (tab.n_dst + 1 + 2 * tab.nnz) * 4;
             ts->last.push_back(tab);
             if (rc) return rc;
@@ -1279,21 +1284,17 @@ int check_space(int kind, int m, int e, uint64_t *n_bad, uint64_t *size) {
     Space sp{kind, m, e, 0, kind == SPACE_X ? T.cnt[m] + T.cnt[m - 1] : (kind == SPACE_C ? T.cntc[m] : T.cnt[m]),
              nullptr};
     uint32_t *pre = nullptr;
+    DevPool pool;
     Scratch sc(nullptr);
-    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pre))) return rc;
+    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pool, &pre))) return rc;
     sp.prefix = pre;
     unsigned long long *bad = nullptr;
-    if ((rc = dev_alloc((void **)&bad, 8))) {
-        dev_free(pre);
-        return rc;
-    }
+    if ((rc = pool.alloc((void **)&bad, 8))) return rc;
     CP_CUDA_TRY(cudaMemset(bad, 0, 8));
     check_space_kernel<<<(unsigned)((sp.size + 127) / 128), 128>>>(sp, T_dev, bad);
     CP_CUDA_TRY(cudaGetLastError());
     unsigned long long h = 0;
     CP_CUDA_TRY(cudaMemcpy(&h, bad, 8, cudaMemcpyDeviceToHost));
-    dev_free(bad);
-    dev_free(pre);
     *n_bad = h;
     *size = sp.size;
     return CP_OK;
@@ -1320,19 +1321,15 @@ int enumerate_space(int kind, int m, int e, uint8_t *out_host, uint64_t max_stat
     *size = sp.size;
     if (sp.size > max_states) return fail(CP_EINVAL, "output buffer too small");
     uint32_t *pre = nullptr;
+    DevPool pool;
     Scratch sc(nullptr);
-    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pre))) return rc;
+    if (kind == SPACE_X && (rc = build_x_prefix(m, e, &sc, &pool, &pre))) return rc;
     sp.prefix = pre;
     uint8_t *d = nullptr;
-    if ((rc = dev_alloc((void **)&d, sp.size * m))) {
-        dev_free(pre);
-        return rc;
-    }
+    if ((rc = pool.alloc((void **)&d, sp.size * m))) return rc;
     enumerate_kernel<<<(unsigned)((sp.size + 127) / 128), 128>>>(sp, T_dev, d);
     CP_CUDA_TRY(cudaGetLastError());
     CP_CUDA_TRY(cudaMemcpy(out_host, d, sp.size * m, cudaMemcpyDeviceToHost));
-    dev_free(d);
-    dev_free(pre);
     return CP_OK;
 }
 

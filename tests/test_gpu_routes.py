@@ -283,3 +283,20 @@ def test_long_rows_dealt_out_by_degrees(lattice, L, N, P):
 def test_tall_strips_keep_their_speed(L, N, P, ms):
     # ms: what the rows and the read-out took with a block for the columns of a row (before the chunk kernel)
     assert solve_ms("square", L, N, gpu_util.seed_primes(P, seed=54)) < ms
+
+
+@pytest.mark.parametrize("lattice,L,v,ms", [("square", 7, 2, 1.65), ("triangular", 7, 2, 1.85), ("square", 9, None, 2.70),
+                                            ("triangular", 9, None, 2.32), ("square", 14, None, 7.9)])
+def test_small_tables_keep_their_build_time(lattice, L, v, ms):
+    # ms: the cold tables and vectors before degree windows; one table per factor (any-v, or rows of 336 bytes)
+    import time
+
+    import torch
+    primes, stream, got = gpu_util.seed_primes(4, seed=55), torch.cuda.Stream(), []
+    for _ in range(16):
+        cp.load().cp_clear_table_cache()
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        cp.Strip(lattice, L, primes, max_degree=20, max_rows=3, v=v, stream=stream).close()
+        got.append((time.perf_counter() - t) * 1e3)
+    assert sorted(got)[3] < ms
